@@ -18,6 +18,7 @@
 // Rows and columns beyond the real group count n (<= NP) are padded with the identity.
 // The pivot search, pivot-row broadcast and the natural-order inverse go through
 // shared memory; the inverse of each zone is streamed to the caller's factor buffer.
+#include "async.cuh"
 #include "mgfld_internal.cuh"
 
 namespace mgfld {
@@ -519,28 +520,6 @@ k_solve_rows(int n, int n_r, int n_sys, int spr, const T *__restrict__ dinv, con
 // cheaper than FP64 on this GPU, so these kernels are bound by the dependency chain along the
 // zones and by the instruction and shared-memory traffic of each zone step.
 constexpr int kWarpsPerCta = 4;
-
-// Per-thread 16-byte asynchronous global-to-shared copies (completion waited by the issuing thread).
-__device__ inline void cp_async16(void *dst, const void *src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ inline void cp_async4(void *dst, const void *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ inline void cp_async8(void *dst, const void *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-// one element of 4 or 8 bytes
-template <typename TE> __device__ inline void cp_async_elem(TE *dst, const TE *src) {
-  if constexpr (sizeof(TE) == 4) cp_async4(dst, src);
-  else cp_async8(dst, src);
-}
-__device__ inline void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ inline void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-template <int N> __device__ inline void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // FP32 reciprocal: the hardware approximation (rcp.approx.ftz) refined by one Newton step, a
 // few multiply-adds instead of the correctly rounded library reciprocal; ample for the FP32
@@ -1125,329 +1104,6 @@ k_solve_w32(int n, int n_r, int n_sys, const float *__restrict__ dinv, const dou
   }
 }
 
-#define MGFLD_DISPATCH_NP(n, ...)                          \
-  if (n <= 4) { constexpr int NP = 4; __VA_ARGS__; }         \
-  else if (n <= 8) { constexpr int NP = 8; __VA_ARGS__; }    \
-  else if (n <= 12) { constexpr int NP = 12; __VA_ARGS__; }  \
-  else if (n <= 16) { constexpr int NP = 16; __VA_ARGS__; }  \
-  else if (n <= 20) { constexpr int NP = 20; __VA_ARGS__; }  \
-  else if (n <= 24) { constexpr int NP = 24; __VA_ARGS__; }  \
-  else { constexpr int NP = 32; __VA_ARGS__; }
-
-// ---------------------------------------------------------------------------------------
-// TMA-fed warp solve (MIXED, even n): each warp streams its system's per-zone inverse block and
-// the zone's right-hand side / coupling vectors into a ring of shared-memory slots with bulk
-// asynchronous copies (cp.async.bulk, completion counted on an mbarrier per slot), issued
-// STAGES-1 zones ahead by lane 0, so the recurrence never waits on a global-memory round trip.
-// Every wait is bounded: on timeout the warp flags `err`, waits (bounded) for its copies in
-// flight and returns.
-template <int NP>
-struct SolveRing {
-  // Ring depth: a power of two (slot and phase by masks), 8 for N <= 20 and 4 above, so that
-  // the rings of both warps (<= 26 KB) let every CTA of a 1024-system launch be resident.
-  static constexpr int STAGES = NP <= 20 ? 8 : 4;
-  static constexpr int WPC = 2;                              // warps per CTA (the two halves of one system)
-  static constexpr int SLOT = NP * NP * 4;                   // bytes: one inverse block
-};
-
-__device__ inline unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-__device__ inline void mbar_init(unsigned long long *bar, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-}
-__device__ inline void mbar_fence_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-__device__ inline void mbar_expect_tx(unsigned long long *bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
-               : "memory");
-}
-__device__ inline void bulk_g2s(void *dst, const void *src, unsigned bytes, unsigned long long *bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
-                   "r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(bar))
-               : "memory");
-}
-__device__ inline bool mbar_try_wait(unsigned long long *bar, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_addr(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-constexpr int kWaitLimit = 1 << 22;
-__device__ inline bool mbar_wait_bounded(unsigned long long *bar, unsigned parity) {
-  for (int it = 0; it < kWaitLimit; ++it)
-    if (mbar_try_wait(bar, parity)) return true;
-  return false;
-}
-
-// The power-of-two scaling of one system's right-hand side for the FP32 substitution: k such that
-// max |rhs| 2^k lies in [1/2, 1) (from the largest exponent, so the maximum is taken over the
-// upper words of the bit patterns: integer pipe only), and the FP32 copy rhs 2^k.  All threads of
-// the block call it.
-__device__ inline void sysmax_scale(const double *__restrict__ rhs, int cnt, int *__restrict__ sys_exp,
-                                    float *__restrict__ rhs32) {
-  __shared__ unsigned red[256];
-  __shared__ int kexp_s;
-  unsigned m = 0u;
-  for (int e = threadIdx.x; e < cnt; e += blockDim.x)
-    m = max(m, (unsigned)(__double_as_longlong(rhs[e]) >> 32) & 0x7fffffffu);
-  red[threadIdx.x] = m;
-  __syncthreads();
-  for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) red[threadIdx.x] = max(red[threadIdx.x], red[threadIdx.x + h]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    const int e = (int)(red[0] >> 20);
-    const int k = (e > 0 && e < 0x7ff) ? 1022 - e : 0;
-    *sys_exp = k;
-    kexp_s = k;
-  }
-  __syncthreads();
-  const int k = kexp_s;
-  for (int e = threadIdx.x; e < cnt; e += blockDim.x) rhs32[e] = d2f_exp2(rhs[e], k);
-}
-
-// Per-system power-of-two scaling of the FP32 solve: k with max |rhs| 2^k in [0.5, 1) (the
-// exponent field of the maximum), then the scaled right-hand side rounded to FP32 once, so that
-// the substitution reads FP32 values.  One CTA per listed system; its n_r x n right-hand side is
-// contiguous (coalesced loads; the second pass reads it from L2).
-__global__ void k_sysmax(int n, int n_r, const double *__restrict__ rhs, const int *__restrict__ ray_list,
-                         int *__restrict__ sys_exp, float *__restrict__ rhs32, const int *__restrict__ n_dev) {
-  if ((int)blockIdx.x >= listed_sys(gridDim.x, n_dev, NS)) return;    // the whole block
-  const size_t base = (size_t)system_of(blockIdx.x, ray_list) * n_r * n;
-  sysmax_scale(rhs + base, n_r * n, sys_exp + blockIdx.x, rhs32 + base);
-}
-
-// k_sysmax for systems listed with `spr` systems per ray.
-__global__ void k_sysmax_spr(int n, int n_r, const double *__restrict__ rhs, const int *__restrict__ ray_list, int spr,
-                             int *__restrict__ sys_exp, float *__restrict__ rhs32, const int *__restrict__ n_dev) {
-  if ((int)blockIdx.x >= listed_sys(gridDim.x, n_dev, spr)) return;   // the whole block
-  const size_t base = (size_t)system_of_spr(blockIdx.x, ray_list, spr) * n_r * n;
-  sysmax_scale(rhs + base, n_r * n, sys_exp + blockIdx.x, rhs32 + base);
-}
-
-// Row r of a zone's inverse times the zone vector held in shared memory (vb).  VEC: n == NP,
-// rows 16-byte aligned, float4 loads; otherwise scalar loads masked to the n real columns.
-template <int NP, bool VEC>
-__device__ inline float row_dot(const float *__restrict__ row, const float *__restrict__ vb, int n) {
-  float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-  if (VEC) {
-#pragma unroll
-    for (int c = 0; c < NP; c += 4) {
-      const float4 m = *reinterpret_cast<const float4 *>(row + c);
-      const float4 v = *reinterpret_cast<const float4 *>(vb + c);
-      a0 = fmaf(m.x, v.x, a0);
-      a1 = fmaf(m.y, v.y, a1);
-      a2 = fmaf(m.z, v.z, a2);
-      a3 = fmaf(m.w, v.w, a3);
-    }
-  } else {
-#pragma unroll
-    for (int c = 0; c < NP; ++c)
-      if (c < n) {
-        if (c % 2 == 0) a0 = fmaf(row[c], vb[c], a0);
-        else a1 = fmaf(row[c], vb[c], a1);
-      }
-  }
-  return (a0 + a1) + (a2 + a3);
-}
-
-// MIXED-precision substitution with the twisted FP32 factors: one CTA per system, warp 0 the
-// top-down half (zones 0..m-1, then the middle zone m, then back up from m-1 to 0), warp 1 the
-// bottom-up half (zones n_r-1..m+1, then back down from m+1).  Each warp streams its zones'
-// inverse blocks through its own ring of bulk copies (one copy per use, mbarrier completion,
-// bounded waits); the halves meet at the middle through shared memory and CTA barriers.  Lane
-// r owns block row r; the zone vector is broadcast through shared memory.  The right-hand side
-// arrives scaled and rounded to FP32 (k_sysmax); the result is scaled back by an exact FP64
-// multiplication by 2^-k.  Offsets inside a system are 32-bit.  Every block is read twice (the
-// inward and the outward sweep), so the kernel is bound by the HBM bandwidth of those reads.
-template <int NP, bool VEC>
-__global__ void __launch_bounds__(SolveRing<NP>::WPC * 32)
-k_solve_tma(int n, int n_r, int n_sys, const float *__restrict__ dinv, const float *__restrict__ lower,
-            const float *__restrict__ upper, const float *__restrict__ rhs32, double *__restrict__ x,
-            float *__restrict__ g32, const int *__restrict__ ray_list, const int *__restrict__ sys_exp, int *err,
-            const int *__restrict__ n_dev) {
-  using R = SolveRing<NP>;
-  static_assert(R::WPC == 2, "one system per CTA: two warps, one per half");
-  constexpr int S = R::STAGES;
-  static_assert((S & (S - 1)) == 0 && S % 4 == 0, "power-of-two ring, refilled four slots at a time");
-  constexpr int D = 8;                                      // depth of the per-lane vector queue
-  __shared__ __align__(128) unsigned char ring[2][S][NP * NP * 4];
-  __shared__ __align__(16) float vbuf[2][NP];               // the zone vector, broadcast through smem
-  __shared__ __align__(16) float qbuf[2][D][2][32];         // per-lane queue: (rhs or g, coupling)
-  __shared__ __align__(8) unsigned long long bar[2][S];
-  __shared__ float hbuf[32], xbuf[32];                      // h_{m+1} and x_m, exchanged at the middle
-  const unsigned full = 0xffffffffu;
-  const int half = threadIdx.x >> 5, r = threadIdx.x & 31;
-  const long jsys = blockIdx.x;
-  if (jsys >= listed_sys(n_sys, n_dev, NS)) return;         // whole CTA
-  const long sys = system_of(jsys, ray_list);
-  const bool real = r < n;
-  const int rr = real ? r : 0;                              // lanes without a row use row 0 (unused)
-  const unsigned blk = (unsigned)(n * n * 4);
-  const double unscale = ldexp(1.0, -sys_exp[jsys]);       // rhs was scaled by 2^k before rounding
-  const int m = n_r / 2, B = n_r - 1 - m;
-  const int F = half == 0 ? m : B;                          // forward steps of this half
-  const int U = half == 0 ? 2 * m + 1 : 2 * B;              // ring uses of this half
-  // Zone sequences: forward zf0 + j dz, backward zb0 - j dz; element offsets z n (32-bit).
-  const int dz = half == 0 ? 1 : -1;
-  const int dzn = dz * n;
-  const int zf0 = half == 0 ? 0 : n_r - 1, zb0 = half == 0 ? m - 1 : m + 1;
-  // Per-lane element pointers of this system (row r of zone z is [z * n]).
-  const size_t sb = (size_t)sys * n_r * n;
-  const float *rhs_l = rhs32 + sb + rr;
-  const float *cin_l = (half == 0 ? lower : upper) + sb + rr;   // coupling used going inward
-  const float *cout_l = (half == 0 ? upper : lower) + sb + rr;  // coupling used going outward
-  float *g_l = g32 + sb + rr;
-  double *x_l = x + sb + rr;
-  const float *dsys = dinv + sb * n;
-  const unsigned rowoff = (unsigned)rr * (unsigned)n * 4u; // byte offset of row r in a slot
-  if (r == 0) {
-    for (int k = 0; k < S; ++k) mbar_init(&bar[half][k], 1);
-    mbar_fence_init();
-  }
-  __syncwarp();
-  // Lane 0 issues the bulk copies in use order, tracking the source block of the next use:
-  // top-down half +1 zone up to the middle, then -1; bottom-up half -1 to zone m + 1, which is
-  // used twice (last forward, first backward), then +1.  All S slots are filled up front, then
-  // four at a time once the four uses that held them are consumed.
-  int iu = 0;
-  const float *src = dsys + (size_t)zf0 * n * n;
-  const int bstep = n * n;
-  auto issue_next = [&]() {
-    unsigned long long *b = &bar[half][iu & (S - 1)];
-    mbar_expect_tx(b, blk);
-    bulk_g2s(ring[half][iu & (S - 1)], src, blk, b);
-    ++iu;
-    if (half == 0) src += iu <= m ? bstep : -bstep;
-    else src += iu < B ? -bstep : (iu == B ? 0 : bstep);
-  };
-  bool ok = true;                                           // warp-uniform
-  auto wait = [&](int u) -> bool {
-    if (!ok) return false;
-    if (mbar_try_wait(&bar[half][u & (S - 1)], (unsigned)((u / S) & 1))) return true;
-    bool w = mbar_wait_bounded(&bar[half][u & (S - 1)], (unsigned)((u / S) & 1));
-    ok = __all_sync(full, w);
-    if (!ok) {                                    // give up: flag and drain own copies
-      if (r == 0) {
-        atomicExch(err, 1);
-        for (int v = u + 1; v < iu; ++v) mbar_wait_bounded(&bar[half][v & (S - 1)], (unsigned)((v / S) & 1));
-      }
-      __syncwarp();
-    }
-    return ok;
-  };
-  auto advance = [&](int u) {                     // use u consumed: refill four slots after every fourth
-    if ((u & 3) == 3) {
-      __syncwarp();
-      if (r == 0 && ok)
-        for (int k = 0; k < 4 && iu < U; ++k) issue_next();
-    }
-  };
-  auto slot_row = [&](int u) {
-    return reinterpret_cast<const float *>(ring[half][u & (S - 1)] + rowoff);
-  };
-  // Per-lane queue of (rhs or forward result, coupling) for the uses D ahead, in shared memory
-  // through 4-byte asynchronous copies: one copy group per use, waited for with
-  // cp.async.wait_group D-1, so that no register load is outstanding across the recurrence.
-  float (*q)[2][32] = qbuf[half];
-  auto fill = [&](int d, const float *a, const float *c, int zo) {
-    cp_async4(&q[d][0][r], a + zo);
-    cp_async4(&q[d][1][r], c + zo);
-    cp_async_commit();
-  };
-  // the middle zone's right-hand side and couplings (top-down half), fetched up front
-  const int zm = m * n;
-  const float bm_raw = rhs_l[zm], lm_raw = cin_l[zm], um_raw = cout_l[zm];
-  float *vb = vbuf[half];
-
-  if (r == 0)
-    for (int k = 0; k < S && k < U; ++k) issue_next();
-  iu = __shfl_sync(full, iu, 0);
-#pragma unroll
-  for (int d = 0; d < D; ++d) fill(d, rhs_l, cin_l, (d < F ? zf0 + d * dz : zf0) * n);
-  float prev = 0.f;
-  int zfo = zf0 * n;                              // element offset of the current forward zone
-  for (int j = 0; j < F; ++j) {
-    const int d = j & (D - 1);
-    cp_async_wait_group<D - 1>();
-    const float b = q[d][0][r], l = j > 0 ? q[d][1][r] : 0.f;
-    if (wait(j)) {
-      if (r < NP) vb[r] = real ? b - l * prev : 0.f;
-      __syncwarp();
-      const float g = row_dot<NP, VEC>(slot_row(j), vb, n);
-      if (real) g_l[zfo] = g;
-      prev = g;
-    }
-    fill(d, rhs_l, cin_l, j + D < F ? zfo + D * dzn : zfo);   // the slot just read: the zone D ahead
-    advance(j);
-    zfo += dzn;
-  }
-  cp_async_wait_all();
-  if (half == 1) hbuf[r] = B > 0 ? prev : 0.f;
-  __syncthreads();
-  if (half == 0) {
-    // Middle zone: x_m = Dinv_m (r_m - l_m g_{m-1} - u_m h_{m+1}).
-    const float bm = real ? bm_raw : 0.f;
-    const float lm = (real && m > 0) ? lm_raw : 0.f;
-    const float um = (real && m < n_r - 1) ? um_raw : 0.f;
-    float xm = 0.f;
-    if (wait(m)) {
-      if (r < NP) vb[r] = real ? bm - lm * prev - um * hbuf[r] : 0.f;
-      __syncwarp();
-      xm = row_dot<NP, VEC>(slot_row(m), vb, n);
-      if (real) x_l[zm] = (double)xm * unscale;
-    }
-    advance(m);
-    xbuf[r] = xm;
-    prev = xm;
-  }
-  __syncthreads();
-  if (half == 1) prev = xbuf[r];
-  // Backward: top x_i = g_i - Dinv_i (u_i x_{i+1}); bottom x_i = h_i - Dinv_i (l_i x_{i-1}).
-#pragma unroll
-  for (int d = 0; d < D; ++d) fill(d, g_l, cout_l, (d < F ? zb0 - d * dz : m) * n);   // m: valid whatever F is
-  int zbo = zb0 * n;
-  const int ub = U - F;                           // first backward use
-  for (int j = 0; j < F; ++j) {
-    const int d = j & (D - 1);
-    const int u = ub + j;
-    cp_async_wait_group<D - 1>();
-    const float gz = q[d][0][r], c = q[d][1][r];
-    if (wait(u)) {
-      if (r < NP) vb[r] = real ? c * prev : 0.f;
-      __syncwarp();
-      const float xi = gz - row_dot<NP, VEC>(slot_row(u), vb, n);
-      if (real) x_l[zbo] = (double)xi * unscale;
-      prev = xi;
-    }
-    fill(d, g_l, cout_l, j + D < F ? zbo - D * dzn : zbo);
-    advance(u);
-    zbo -= dzn;
-  }
-  cp_async_wait_all();
-}
-
-cudaError_t launch_solve_tma(int n, int n_r, int n_sys, const void *dinv, const float *lower32,
-                             const float *upper32, const double *rhs, float *rhs32, double *x, float *g32,
-                             const int *ray_list, int *sys_exp, int *err, cudaStream_t s, const int *n_dev) {
-  if (n_sys == 0) return cudaSuccess;
-  k_sysmax<<<n_sys, 256, 0, s>>>(n, n_r, rhs, ray_list, sys_exp, rhs32, n_dev);
-  MGFLD_DISPATCH_NP(n, {
-    using R = SolveRing<NP>;
-    const unsigned grid = (unsigned)n_sys;                 // one system (two warps) per CTA
-    if (n == NP)
-      k_solve_tma<NP, true><<<grid, R::WPC * 32, 0, s>>>(n, n_r, n_sys, (const float *)dinv, lower32, upper32, rhs32,
-                                                         x, g32, ray_list, sys_exp, err, n_dev);
-    else
-      k_solve_tma<NP, false><<<grid, R::WPC * 32, 0, s>>>(n, n_r, n_sys, (const float *)dinv, lower32, upper32,
-                                                          rhs32, x, g32, ray_list, sys_exp, err, n_dev);
-    return cudaGetLastError();
-  })
-}
-
 template <int NP>
 static cudaError_t run_factor(int n, int n_r, int n_sys, const void *diag, int diag_fp32, const double *lower,
                               const double *upper, void *dinv, const int *ray_list, cudaStream_t s,
@@ -1545,7 +1201,8 @@ cudaError_t launch_solve_rows(int nb, int n_r, int n_sys, int spr, const void *d
   if (nb > 48) return cudaErrorInvalidValue;
   if (fp32) {
     // per-system power-of-two scaling of the right-hand side for the FP32 sweeps
-    k_sysmax_spr<<<n_sys, 256, 0, s>>>(nb, n_r, rhs, ray_list, spr, sys_exp, rhs32, n_dev);
+    const cudaError_t e = launch_sysmax(nb, n_r, n_sys, rhs, ray_list, spr, sys_exp, rhs32, s, n_dev);
+    if (e != cudaSuccess) return e;
     MGFLD_DISPATCH_NPW(nb, using C = RowCta<NP, float>;
                        k_solve_rows<NP, float><<<(unsigned)((n_sys + C::SPC / 2 - 1) / (C::SPC / 2)), C::THREADS, 0, s>>>(
                            nb, n_r, n_sys, spr, (const float *)dinv, (const float *)lower, (const float *)upper, rhs,

@@ -255,12 +255,24 @@ cudaError_t launch_assemble(const Prob &p, const Ws &w, const double *psi, void 
 cudaError_t launch_factor(int n, int n_r, int n_sys, const void *diag, int diag_fp32, const double *lower,
                           const double *upper, void *dinv, int precision, const int *ray_list,
                           cudaStream_t s, const int *n_dev = nullptr);
-// MIXED-precision solve fed by bulk asynchronous copies; requires even n, 16-byte aligned
-// arrays and rhs != x.  Sets *err on a bounded-wait timeout.
-cudaError_t launch_solve_tma(int n, int n_r, int n_sys, const void *dinv, const float *lower32,
-                             const float *upper32, const double *rhs, float *rhs32, double *x, float *g32,
-                             const int *ray_list, int *sys_exp, int *err, cudaStream_t s,
-                             const int *n_dev = nullptr);
+// The FP32 substitution of the outer iteration (blocks, couplings and vectors in the workspace,
+// rhs != x): the right-hand sides are scaled into rhs32 first.  Sets *err on a bounded-wait timeout.
+cudaError_t launch_solve_ring(int n, int n_r, int n_sys, const void *dinv, const float *lower32, const float *upper32,
+                              const double *rhs, float *rhs32, double *x, float *g32, const int *ray_list,
+                              int *sys_exp, int *err, cudaStream_t s, const int *n_dev = nullptr);
+// Per system (spr per ray): the power of two k that brings max |rhs| into [1/2, 1), and rhs 2^k in FP32.
+cudaError_t launch_sysmax(int n, int n_r, int n_sys, const double *rhs, const int *ray_list, int spr, int *sys_exp,
+                          float *rhs32, cudaStream_t s, const int *n_dev = nullptr);
+
+// The compile-time block size NP >= n of a kernel.
+#define MGFLD_DISPATCH_NP(n, ...)                          \
+  if (n <= 4) { constexpr int NP = 4; __VA_ARGS__; }         \
+  else if (n <= 8) { constexpr int NP = 8; __VA_ARGS__; }    \
+  else if (n <= 12) { constexpr int NP = 12; __VA_ARGS__; }  \
+  else if (n <= 16) { constexpr int NP = 16; __VA_ARGS__; }  \
+  else if (n <= 20) { constexpr int NP = 20; __VA_ARGS__; }  \
+  else if (n <= 24) { constexpr int NP = 24; __VA_ARGS__; }  \
+  else { constexpr int NP = 32; __VA_ARGS__; }
 
 // An opacity entry of (species q, group k) times the optional per-(q, k) scale (no multiplication
 // without a scale: an FP64 operation saved per use, the same value).

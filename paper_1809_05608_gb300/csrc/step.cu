@@ -846,9 +846,9 @@ static cudaError_t enqueue_iteration(const StepCall &c, int it, int n_act, int n
     MGFLD_ENQ(launch_solve_rows(2 * n, NR, n_act * 2, 2, w.dinv, tl.mixed ? (const void *)w.lower32 : w.lower,
                                 tl.mixed ? (const void *)w.upper32 : w.upper, w.rhs, w.rhs32, w.sscale, w.x, tl.mixed,
                                 w.list_act, s, cnt_act));
-  else if (tl.mixed && n % 2 == 0)
-    MGFLD_ENQ(launch_solve_tma(n, NR, n_act * NS, w.dinv, w.lower32, w.upper32, w.rhs, w.rhs32, w.x, w.g32,
-                               w.list_act, w.sscale, w.counters + 3, s, cnt_act));
+  else if (tl.mixed)
+    MGFLD_ENQ(launch_solve_ring(n, NR, n_act * NS, w.dinv, w.lower32, w.upper32, w.rhs, w.rhs32, w.x, w.g32,
+                                w.list_act, w.sscale, w.counters + 3, s, cnt_act));
   else
     MGFLD_ENQ(launch_solve(n, NR, n_act * NS, w.dinv, w.lower, w.upper, w.rhs, w.x, c.precision, w.list_act, s,
                            cnt_act));
