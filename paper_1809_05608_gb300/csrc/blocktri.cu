@@ -273,7 +273,7 @@ k_solve(int n, int n_r, int n_sys, const double *__restrict__ dinv, const double
 
 // ---------------------------------------------------------------------------------------
 // Thread-per-row elimination and substitution for systems of any block width up to 64 rows
-// (the coupled nu / antinu blocks of the pair process: 2 n_e rows), in FP64 or FP32, with
+// (the coupled nu / antinu blocks of the pair process: 2 n_e rows; the substitution in FP64 only), with
 // `spr` systems per ray (the launch's j-th system is system j % spr of ray ray_list[j / spr]).
 // Same algorithm and thread mapping as k_factor / k_solve above: partial pivoting through integer
 // keys (6 row bits for blocks wider than 32), the next zone's rows fetched one zone ahead, the
@@ -318,7 +318,7 @@ template <int NP, typename TIn, typename T>
 __global__ void __launch_bounds__(RowCta<NP, T>::THREADS)
 k_factor_rows(int n, int n_r, int n_sys, int spr, const TIn *__restrict__ diag, const T *__restrict__ lower,
               const T *__restrict__ upper, T *__restrict__ dinv, const int *__restrict__ ray_list,
-              const int *__restrict__ n_dev) {
+              const int *__restrict__ bad, const int *__restrict__ n_dev) {
   using C = RowCta<NP, T>;
   constexpr int SPC = C::SPC, KB = C::KB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -334,6 +334,14 @@ k_factor_rows(int n, int n_r, int n_sys, int spr, const TIn *__restrict__ diag, 
   const int half = s & 1;                            // 0: zones 0..m top-down, 1: zones n_r-1..m+1 bottom-up
   const int n_sys_e = listed_sys(n_sys, n_dev, spr);
   if ((long)blockIdx.x * (SPC / 2) >= n_sys_e) return;   // the whole CTA
+  if (bad) {                                         // only where the unpivoted elimination failed
+    bool any = false;
+    for (int c = 0; c < SPC / 2; ++c) {
+      const long js = (long)blockIdx.x * (SPC / 2) + c;
+      any = any || (js < n_sys_e && bad[js]);
+    }
+    if (!any) return;                                // the whole CTA
+  }
   const long jsys = (long)blockIdx.x * (SPC / 2) + (s >> 1);
   const bool valid = jsys < n_sys_e;
   const long sys = valid ? system_of_spr(jsys, ray_list, spr) : 0;
@@ -421,17 +429,15 @@ k_factor_rows(int n, int n_r, int n_sys, int spr, const TIn *__restrict__ diag, 
   }
 }
 
-// Substitution with those factors (twisted, as k_solve).  FP64: rhs and x as given.  FP32: the
-// right-hand side arrives scaled by 2^k per system and rounded to FP32 (rhs32, k in sys_exp, from
-// k_sysmax), the sweeps run in FP32 and x is scaled back by an exact multiplication by 2^-k; the
-// forward results are kept in x (in the scaled units) until the backward sweep replaces them.
-template <int NP, typename T>
-__global__ void __launch_bounds__(RowCta<NP, T>::THREADS)
-k_solve_rows(int n, int n_r, int n_sys, int spr, const T *__restrict__ dinv, const T *__restrict__ lower,
-             const T *__restrict__ upper, const double *rhs, const float *__restrict__ rhs32,
-             const int *__restrict__ sys_exp, double *x, const int *__restrict__ ray_list,
+// FP64 substitution with those factors (twisted, as k_solve); the forward results are kept in x until
+// the backward sweep replaces them.
+template <int NP>
+__global__ void __launch_bounds__(RowCta<NP, double>::THREADS)
+k_solve_rows(int n, int n_r, int n_sys, int spr, const double *__restrict__ dinv, const double *__restrict__ lower,
+             const double *__restrict__ upper, const double *rhs, double *x, const int *__restrict__ ray_list,
              const int *__restrict__ n_dev) {
-  constexpr int SPC = RowCta<NP, T>::SPC;
+  using T = double;
+  constexpr int SPC = RowCta<NP, double>::SPC;
   __shared__ T v[SPC][NP];
   __shared__ T mid[SPC / 2][NP];
   const int s = threadIdx.x / NP, r = threadIdx.x % NP;
@@ -445,10 +451,7 @@ k_solve_rows(int n, int n_r, int n_sys, int spr, const T *__restrict__ dinv, con
   const size_t base = (size_t)sys * n_r * n;
   const int m = n_r / 2, B = n_r - 1 - m;
   const int F = half == 0 ? m : B;
-  const bool f32 = sizeof(T) == 4;
-  const double unscale = (f32 && valid) ? ldexp(1.0, -sys_exp[jsys]) : 1.0;
   const T zero = T(0);
-  auto b_at = [&](size_t zr) -> T { return f32 ? (T)rhs32[zr] : (T)rhs[zr]; };
   auto rowdot = [&](int z, bool real) {
     const T *src = dinv + (base + (size_t)z * n + r) * n;
     T acc0 = zero, acc1 = zero;
@@ -468,12 +471,12 @@ k_solve_rows(int n, int n_r, int n_sys, int spr, const T *__restrict__ dinv, con
     const int z = half == 0 ? j : n_r - 1 - j;
     const size_t zr = base + (size_t)(real ? z : 0) * n + r;
     const T c = (real && j > 0) ? (half == 0 ? lower[zr] : upper[zr]) : zero;
-    const T b = real ? b_at(zr) : zero;
+    const T b = real ? rhs[zr] : zero;
     v[s][r] = real ? b - c * prev : zero;
     __syncthreads();
     const T g = rowdot(z, real);
     if (real) {
-      x[zr] = (double)g;
+      x[zr] = g;
       prev = g;
     }
     __syncthreads();
@@ -484,12 +487,12 @@ k_solve_rows(int n, int n_r, int n_sys, int spr, const T *__restrict__ dinv, con
     const size_t zr = base + (size_t)m * n + r;
     const T l = (realr && m > 0) ? lower[zr] : zero;
     const T u = (realr && m < n_r - 1) ? upper[zr] : zero;
-    v[s][r] = realr ? b_at(zr) - l * prev - u * mid[sl][r] : zero;
+    v[s][r] = realr ? rhs[zr] - l * prev - u * mid[sl][r] : zero;
   }
   __syncthreads();
   if (half == 0) {
     const T xm = rowdot(m, realr);
-    if (realr) x[base + (size_t)m * n + r] = (double)xm * unscale;
+    if (realr) x[base + (size_t)m * n + r] = xm;
     prev = xm;
   }
   __syncthreads();
@@ -506,8 +509,8 @@ k_solve_rows(int n, int n_r, int n_sys, int spr, const T *__restrict__ dinv, con
     __syncthreads();
     const T acc = rowdot(z, real);
     if (real) {
-      const T xi = (T)x[zr] - acc;
-      x[zr] = (double)xi * unscale;
+      const T xi = x[zr] - acc;
+      x[zr] = xi;
       prev = xi;
     }
     __syncthreads();
@@ -593,74 +596,6 @@ __device__ inline void gj_invert(float *a, float (*prow)[NP + 4], int r, bool ro
   }
 }
 
-// In-place Gauss-Jordan inverse without row exchanges, lane r holding row r, with 2 x 2 pivot
-// blocks: at step b the owners of rows p = 2b and p + 1 publish both rows (double-buffered
-// shared memory), every lane forms the inverse of the pivot block
-// P = [[d00, d01], [d10, d11]] in closed form (one reciprocal of its determinant) and eliminates
-// with the two multipliers (a_p, a_{p+1}) P^{-1}; the owners take the rows of P^{-1} times the
-// pivot rows by the same formula.  Half as many broadcast steps on the chain of each block, the
-// same number of FMAs.  Leading 2 x 2 blocks of the Schur complements of an M-matrix (or of a
-// column diagonally dominant matrix) are nonsingular, so no exchanges are needed; returns false
-// (the same in every lane) when a determinant was zero or not finite.  NP must be even.
-template <int NP>
-__device__ inline bool gj_invert_np2(float *a, float (*prow)[2][NP + 4], int r) {
-  static_assert(NP % 4 == 0, "pivot pairs inside 16-byte pieces");
-  bool ok = true;
-#pragma unroll
-  for (int b = 0; b < NP / 2; ++b) {
-    const int p = 2 * b;
-    float (*pb)[NP + 4] = prow[b & 1];
-    if (r == p || r == p + 1) {
-      float *dst = pb[r - p];
-#pragma unroll
-      for (int c = 0; c < NP; c += 2) *reinterpret_cast<float2 *>(dst + c) = make_float2(a[c], a[c + 1]);
-    }
-    __syncwarp();
-    // the pivot block (columns p, p + 1 of both pivot rows) first
-    const float2 q0 = *reinterpret_cast<const float2 *>(&pb[0][p]);
-    const float2 q1 = *reinterpret_cast<const float2 *>(&pb[1][p]);
-    const float det = fmaf(q0.x, q1.y, -(q0.y * q1.x));
-    const float idet = rcp_nr(det);
-    ok = ok && isfinite(idet) && det != 0.f;
-    const float i00 = q1.y * idet, i01 = -q0.y * idet, i10 = -q1.x * idet, i11 = q0.x * idet;
-    float f0, f1;
-    if (r == p) {
-      f0 = 1.f - i00;
-      f1 = -i01;
-    } else if (r == p + 1) {
-      f0 = -i10;
-      f1 = 1.f - i11;
-    } else {
-      f0 = fmaf(a[p], i00, a[p + 1] * i10);
-      f1 = fmaf(a[p], i01, a[p + 1] * i11);
-    }
-#pragma unroll
-    for (int c = 0; c < NP; c += 4) {
-      const float4 v0 = *reinterpret_cast<const float4 *>(&pb[0][c]);
-      const float4 v1 = *reinterpret_cast<const float4 *>(&pb[1][c]);
-      float2 lo = __ffma2_rn(make_float2(-f0, -f0), make_float2(v0.x, v0.y), make_float2(a[c], a[c + 1]));
-      float2 hi = __ffma2_rn(make_float2(-f0, -f0), make_float2(v0.z, v0.w), make_float2(a[c + 2], a[c + 3]));
-      lo = __ffma2_rn(make_float2(-f1, -f1), make_float2(v1.x, v1.y), lo);
-      hi = __ffma2_rn(make_float2(-f1, -f1), make_float2(v1.z, v1.w), hi);
-      a[c] = lo.x;
-      a[c + 1] = lo.y;
-      a[c + 2] = hi.x;
-      a[c + 3] = hi.y;
-    }
-    if (r == p) {
-      a[p] = i00;
-      a[p + 1] = i01;
-    } else if (r == p + 1) {
-      a[p] = i10;
-      a[p + 1] = i11;
-    } else {
-      a[p] = -f0;
-      a[p + 1] = -f1;
-    }
-  }
-  return __all_sync(0xffffffffu, ok);
-}
-
 // CTAs per SM the FP32 factor is compiled for (its register budget): the kernel is bound by the
 // latency of its pivot chain, so resident warps matter more than a few spilled registers.
 #ifndef MGFLD_FW32_MINB
@@ -673,11 +608,8 @@ template <int NP> __host__ __device__ constexpr int fw_wpc() { return NP > 24 ? 
 
 // At most 128 registers (NP <= 24), so that four CTAs (eight systems) fit on an SM and the
 // 256-ray workload's 512 CTAs run in a single wave on 152 SMs.
-// PIVOT: partial pivoting in every zone (the C ABI's factor of arbitrary systems); otherwise
-// elimination without row exchanges (the outer iteration's M-matrix blocks, see gj_invert_np2)
-// with partial pivoting only for a zone whose unpivoted elimination met a zero or non-finite
-// pivot.
-template <int NP, typename TIn, typename TC, bool PIVOT>
+// The C ABI's factor of arbitrary systems: partial pivoting in every zone.
+template <int NP, typename TIn, typename TC>
 __global__ void __launch_bounds__(fw_wpc<NP>() * 32, MGFLD_FW32_MINB)
 k_factor_w32(int n, int n_r, int n_sys, const TIn *__restrict__ diag, const TC *__restrict__ lower,
              const TC *__restrict__ upper, float *__restrict__ dinv, const int *__restrict__ ray_list,
@@ -689,7 +621,6 @@ k_factor_w32(int n, int n_r, int n_sys, const TIn *__restrict__ diag, const TC *
   __shared__ __align__(16) float tile[W][NP][NP];
   __shared__ __align__(16) float ushr[W][NP];
   __shared__ __align__(16) float prow[W][2][NP + 4];
-  __shared__ __align__(16) float prow2[W][2][2][NP + 4];
   __shared__ __align__(16) float rowbuf[W][2][NP][NP];
   __shared__ __align__(16) TC cplb[W][2][2][32];      // per lane: the next zone's couplings (rows path)
   const int wid = threadIdx.x >> 5, r = threadIdx.x & 31;
@@ -749,9 +680,8 @@ k_factor_w32(int n, int n_r, int n_sys, const TIn *__restrict__ diag, const TC *
     const bool mid = half == 0 && j == m;
     if (mid) asm volatile("bar.sync %0, 64;" ::"r"(1 + (wid >> 1)) : "memory");
     float a[NP];
-    // The zone's Schur complement from its raw rows (still in the row buffer) and the previous
-    // zone's inverse (still in this warp's tile), so that it can be rebuilt for the fallback.
-    auto build_a = [&]() {
+    // The zone's Schur complement from its raw rows and the previous zone's inverse (this warp's tile).
+    {
       if (row) {
 #pragma unroll
         for (int c = 0; c < NP; c += 4) {
@@ -786,26 +716,14 @@ k_factor_w32(int n, int n_r, int n_sys, const TIn *__restrict__ diag, const TC *
 #pragma unroll
         for (int c = 0; c < NP; ++c) a[c] = a[c] - (ur * tile[wid ^ 1][r][c]) * ushr[wid ^ 1][c];
       }
-    };
-    build_a();
-    const bool ok = PIVOT ? false : gj_invert_np2<NP>(a, prow2[wid], r);
+    }
+    int my_step;
+    unsigned piv[NP / 4];
+    gj_invert<NP>(a, prow[wid], r, row, my_step, piv);
     __syncwarp();                  // every lane has read the previous zone's tile row
-    if (ok) {
-      if (row) {
+    if (row) {
 #pragma unroll
-        for (int c = 0; c < NP; c += 2) *reinterpret_cast<float2 *>(&tile[wid][r][c]) = make_float2(a[c], a[c + 1]);
-      }
-    } else {
-      // pivoting requested, or a zero or non-finite pivot: the block with partial pivoting
-      if (!PIVOT) build_a();
-      int my_step;
-      unsigned piv[NP / 4];
-      gj_invert<NP>(a, prow[wid], r, row, my_step, piv);
-      __syncwarp();
-      if (row) {
-#pragma unroll
-        for (int c = 0; c < NP; ++c) tile[wid][my_step][(piv[c / 4] >> (8 * (c % 4))) & 0xffu] = a[c];
-      }
+      for (int c = 0; c < NP; ++c) tile[wid][my_step][(piv[c / 4] >> (8 * (c % 4))) & 0xffu] = a[c];
     }
     __syncwarp();
     if (row) ushr[wid][r] = ur;   // column scaling of this zone's Schur term in the next zone
@@ -829,16 +747,23 @@ k_factor_w32(int n, int n_r, int n_sys, const TIn *__restrict__ diag, const TC *
 // ---------------------------------------------------------------------------------------
 // FP32 factor of the outer iteration with two block rows per lane (the mixed path's zone blocks,
 // M-matrices: no row exchanges).  L = NP/2 lanes hold a half-system, lane m rows m and m + L, and a
-// warp holds S = 32 / L half-systems (three at NP = 20); warp 0 of a CTA takes the top-down halves
-// and warp 1 the bottom-up halves of the same S systems.  Every pivot row is read from shared memory
-// once per lane for its two rows, so a broadcast serves twice the rows and S systems at once: the
-// shared-memory traffic per system, which bounds the one-row-per-lane kernel, drops about threefold.
-// Gauss-Jordan with 2 x 2 pivot blocks as gj_invert_np2; the Schur term of the next zone is formed
-// from the lane's own rows of the inverse, still in registers (row r of the inverse stays with the
-// lane of row r); the next zone's rows and couplings arrive by asynchronous copies issued one zone
-// ahead.  A zone whose 2 x 2 pivot block is singular or not finite leaves its inverse non-finite
-// (the outer iteration then reports ENAN for the ray); the ABI's factor of arbitrary systems uses
-// the pivoting kernel above.
+// warp holds S = 32 / L half-systems (three at NP = 20, one at the pair systems' NP = 40); warp 0 of a
+// CTA takes the top-down halves and warp 1 the bottom-up halves of the same S systems.  Every pivot row
+// is read from shared memory once per lane for its two rows, so a broadcast serves twice the rows and S
+// systems at once: the shared-memory traffic per system, which bounds a one-row-per-lane kernel, drops
+// about threefold.  Gauss-Jordan with 2 x 2 pivot blocks: the owners of rows p and p + 1 publish both,
+// every lane inverts the pivot block in closed form (one reciprocal of its determinant) and
+// eliminates with the two multipliers (a_p, a_{p+1}) P^{-1}; leading 2 x 2 blocks of the Schur
+// complements of an M-matrix are nonsingular, so no exchanges are needed.  The Schur term of the next
+// zone is formed from the lane's own rows of the inverse, still in registers (row r of the inverse stays
+// with the lane of row r); the next zone's rows and couplings arrive by asynchronous copies issued one
+// zone ahead.  A zone whose 2 x 2 pivot block is singular or not finite leaves its inverse non-finite;
+// where the launch keeps flags, its system is done again with partial pivoting (without them the outer
+// iteration reports ENAN for the ray).
+// Bound by the latency of the pivot chain.  Measured at 256 rays of 512 x 20 with the pair process (512
+// systems of 40-row blocks) 2.8 ms, against 8.0 ms for one row per thread with CTA barriers and partial
+// pivoting (k_factor_rows); at 173 rays of 301 x 13 (padded to 16) 0.44 ms, against 0.57 ms for one
+// row per lane.
 template <int NP>
 struct Row2 {
   static constexpr int L = NP / 2;                 // lanes per half-system
@@ -853,12 +778,19 @@ struct Row2 {
 #endif
 
 template <int NP>
-__global__ void __launch_bounds__(64, MGFLD_ROW2_MINB)
-k_factor_row2(int n_r, int n_sys, const float *__restrict__ diag, const float *__restrict__ lower,
+__host__ __device__ constexpr int row2_minb() { return NP <= 20 ? MGFLD_ROW2_MINB : (NP <= 32 ? 6 : 4); }
+
+// FULL: n = NP, rows in 16-byte pieces; otherwise rows and columns beyond n are padded with the
+// identity.  spr: systems per ray.  FLAG: bad[listed system] is set to whether a pivot block was
+// singular or not finite.
+template <int NP, bool FULL, bool FLAG>
+__global__ void __launch_bounds__(64, row2_minb<NP>())
+k_factor_row2(int n_, int n_r, int n_sys, int spr, const float *__restrict__ diag, const float *__restrict__ lower,
               const float *__restrict__ upper, float *__restrict__ dinv, const int *__restrict__ ray_list,
-              const int *__restrict__ n_dev) {
+              int *__restrict__ bad, const int *__restrict__ n_dev) {
   using C = Row2<NP>;
   constexpr int L = C::L, S = C::S, PD = C::PAD;
+  const int n = FULL ? NP : n_;
   static_assert(NP % 4 == 0 && L % 2 == 0, "pivot pairs in one lane pair, rows in 16-byte pieces");
   // The next zone's rows and couplings arrive by cp.async, per warp (each lane copies and later
   // reads only its own two rows: 80-byte rows are conflict-free for its 16-byte reads); after its
@@ -868,38 +800,66 @@ k_factor_row2(int n_r, int n_sys, const float *__restrict__ diag, const float *_
   __shared__ __align__(16) float cpl[2][S][2][NP];         // its couplings (to the previous / next zone)
   __shared__ __align__(16) float prow[2][2][S][2][PD];     // per warp, double-buffered pivot row pairs
   __shared__ __align__(16) float ucol[2][S][NP];           // column scaling of the next zone's Schur term
+  __shared__ int okb[S];                                   // the bottom-up half's pivots were fine
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int half = wid;                                    // 0: zones 0..m top-down, 1: n_r-1..m+1 bottom-up
   const int g = lane / L, mm = lane % L;                   // half-system of the warp, lane in it
-  const int n_sys_e = listed_sys(n_sys, n_dev, NS);
+  const int n_sys_e = listed_sys(n_sys, n_dev, spr);
   const long j0 = (long)blockIdx.x * S;
   if (j0 >= n_sys_e) return;                               // the whole CTA
   const long jsys = j0 + g;
   const bool valid = g < S && jsys < n_sys_e;
-  const long sys = valid ? system_of(jsys, ray_list) : 0;
+  const long sys = valid ? system_of_spr(jsys, ray_list, spr) : 0;
   const int gs = g < S ? g : 0;                            // shared-memory slot (idle lanes use 0)
   const int m = n_r / 2;
   const int len = half == 0 ? m + 1 : n_r - 1 - m;
   auto zone = [&](int j) { return half == 0 ? j : n_r - 1 - j; };
   const int r0 = mm, r1 = mm + L;                          // this lane's two rows
+  // a padded row: the identity (its lane's own rows only; no copy touches columns beyond n)
+  if (!FULL && g < S) {
+#pragma unroll
+    for (int c = 0; c < NP; ++c) {
+      rows[wid][gs][r0][c] = c == r0 ? 1.f : 0.f;
+      rows[wid][gs][r1][c] = c == r1 ? 1.f : 0.f;
+    }
+    cpl[wid][gs][0][r0] = cpl[wid][gs][0][r1] = cpl[wid][gs][1][r0] = cpl[wid][gs][1][r1] = 0.f;
+  }
   auto issue = [&](int j) {                                // rows and couplings of zone j
     if (valid && j < len) {
-      const size_t zb = ((size_t)sys * n_r + zone(j)) * NP;
-#pragma unroll
-      for (int c = 0; c < NP; c += 4) {
-        cp_async16(&rows[wid][gs][r0][c], diag + (zb + r0) * NP + c);
-        cp_async16(&rows[wid][gs][r1][c], diag + (zb + r1) * NP + c);
-      }
+      const size_t zb = ((size_t)sys * n_r + zone(j)) * n;
       const float *lin = half == 0 ? lower : upper, *lout = half == 0 ? upper : lower;
-      cp_async4(&cpl[wid][gs][0][r0], lin + zb + r0);
-      cp_async4(&cpl[wid][gs][0][r1], lin + zb + r1);
-      cp_async4(&cpl[wid][gs][1][r0], lout + zb + r0);
-      cp_async4(&cpl[wid][gs][1][r1], lout + zb + r1);
+      if (FULL) {
+#pragma unroll
+        for (int c = 0; c < NP; c += 4) {
+          cp_async16(&rows[wid][gs][r0][c], diag + (zb + r0) * NP + c);
+          cp_async16(&rows[wid][gs][r1][c], diag + (zb + r1) * NP + c);
+        }
+        cp_async4(&cpl[wid][gs][0][r0], lin + zb + r0);
+        cp_async4(&cpl[wid][gs][0][r1], lin + zb + r1);
+        cp_async4(&cpl[wid][gs][1][r0], lout + zb + r0);
+        cp_async4(&cpl[wid][gs][1][r1], lout + zb + r1);
+      } else {
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+          const int r = p == 0 ? r0 : r1;
+          if (r < n) {
+            const float *src = diag + (zb + r) * n;
+            float *dst = &rows[wid][gs][r][0];
+            if (n % 2 == 0)
+              for (int c = 0; c < n; c += 2) cp_async8(dst + c, src + c);
+            else
+              for (int c = 0; c < n; ++c) cp_async4(dst + c, src + c);
+            cp_async4(&cpl[wid][gs][0][r], lin + zb + r);
+            cp_async4(&cpl[wid][gs][1][r], lout + zb + r);
+          }
+        }
+      }
     }
     cp_async_commit();
   };
   float (*midt)[NP][NP] = rows[1];                         // the bottom-up warp's last inverse
   float a0[NP], a1[NP];
+  bool ok = true;
   issue(0);
   for (int j = 0; j < len; ++j) {
     cp_async_wait_all();
@@ -962,6 +922,7 @@ k_factor_row2(int n_r, int n_sys, const float *__restrict__ diag, const float *_
       const float2 q1 = *reinterpret_cast<const float2 *>(&pb[gs][1][p]);
       const float det = fmaf(q0.x, q1.y, -(q0.y * q1.x));
       const float idet = rcp_nr(det);
+      if (FLAG) ok = ok && fabsf(idet) < INFINITY;
       const float i00 = q1.y * idet, i01 = -q0.y * idet, i10 = -q1.x * idet, i11 = q0.x * idet;
       // multipliers of the two rows: owners take the rows of P^{-1} times the pivot rows
       float f00, f01, f10, f11;
@@ -996,12 +957,20 @@ k_factor_row2(int n_r, int n_sys, const float *__restrict__ diag, const float *_
     // the inverse rows to the factor buffer, and this zone's coupling to the next zone of the
     // sequence (column scaling of the next Schur term) to the warp's shared row
     if (valid) {
-      float *o0 = dinv + (((size_t)sys * n_r + zone(j)) * NP + r0) * NP;
-      float *o1 = dinv + (((size_t)sys * n_r + zone(j)) * NP + r1) * NP;
+      float *o0 = dinv + (((size_t)sys * n_r + zone(j)) * n + r0) * n;
+      float *o1 = dinv + (((size_t)sys * n_r + zone(j)) * n + r1) * n;
+      if (FULL) {
 #pragma unroll
-      for (int c = 0; c < NP; c += 4) {
-        *reinterpret_cast<float4 *>(o0 + c) = make_float4(a0[c], a0[c + 1], a0[c + 2], a0[c + 3]);
-        *reinterpret_cast<float4 *>(o1 + c) = make_float4(a1[c], a1[c + 1], a1[c + 2], a1[c + 3]);
+        for (int c = 0; c < NP; c += 4) {
+          *reinterpret_cast<float4 *>(o0 + c) = make_float4(a0[c], a0[c + 1], a0[c + 2], a0[c + 3]);
+          *reinterpret_cast<float4 *>(o1 + c) = make_float4(a1[c], a1[c + 1], a1[c + 2], a1[c + 3]);
+        }
+      } else {
+#pragma unroll
+        for (int c = 0; c < NP; ++c) {
+          if (r0 < n && c < n) o0[c] = a0[c];
+          if (r1 < n && c < n) o1[c] = a1[c];
+        }
       }
     }
     if (g < S) {
@@ -1019,7 +988,12 @@ k_factor_row2(int n_r, int n_sys, const float *__restrict__ diag, const float *_
     __syncwarp();
   }
   cp_async_wait_all();
-  if (half == 1) asm volatile("bar.sync 1, 64;" ::: "memory");
+  if (half == 1) {
+    if (FLAG && g < S && mm == 0) okb[gs] = ok;            // (read after the barrier, the top half's last zone)
+    asm volatile("bar.sync 1, 64;" ::: "memory");
+  } else if (FLAG && valid && mm == 0) {
+    bad[jsys] = !(ok && okb[gs]);
+  }
 }
 
 // Forward/back substitution with the twisted FP32 factors, two warps per system (the top-down
@@ -1138,13 +1112,13 @@ cudaError_t launch_factor(int n, int n_r, int n_sys, const void *diag, int diag_
     if (diag_fp32) {
       MGFLD_DISPATCH_NP(n, constexpr int W = fw_wpc<NP>();
                         const unsigned grid = (unsigned)((n_sys + W / 2 - 1) / (W / 2));
-                        k_factor_w32<NP, float, double, true><<<grid, W * 32, 0, s>>>(
+                        k_factor_w32<NP, float, double><<<grid, W * 32, 0, s>>>(
                             n, n_r, n_sys, (const float *)diag, lower, upper, (float *)dinv, ray_list, n_dev);
                         return cudaGetLastError())
     } else {
       MGFLD_DISPATCH_NP(n, constexpr int W = fw_wpc<NP>();
                         const unsigned grid = (unsigned)((n_sys + W / 2 - 1) / (W / 2));
-                        k_factor_w32<NP, double, double, true><<<grid, W * 32, 0, s>>>(
+                        k_factor_w32<NP, double, double><<<grid, W * 32, 0, s>>>(
                             n, n_r, n_sys, (const double *)diag, lower, upper, (float *)dinv, ray_list, n_dev);
                         return cudaGetLastError())
     }
@@ -1154,18 +1128,10 @@ cudaError_t launch_factor(int n, int n_r, int n_sys, const void *diag, int diag_
   }
 }
 
-#define MGFLD_DISPATCH_NPW(n, ...)                          \
-  if (n <= 8) { constexpr int NP = 8; __VA_ARGS__; }          \
-  else if (n <= 16) { constexpr int NP = 16; __VA_ARGS__; }   \
-  else if (n <= 24) { constexpr int NP = 24; __VA_ARGS__; }   \
-  else if (n <= 32) { constexpr int NP = 32; __VA_ARGS__; }   \
-  else if (n <= 40) { constexpr int NP = 40; __VA_ARGS__; }   \
-  else { constexpr int NP = 48; __VA_ARGS__; }
-
 template <int NP, typename TIn, typename T>
 static cudaError_t run_factor_rows(int nb, int n_r, int n_sys, int spr, const TIn *diag, const T *lower,
-                                   const T *upper, T *dinv, const int *ray_list, cudaStream_t s,
-                                   const int *n_dev) {
+                                   const T *upper, T *dinv, const int *ray_list, const int *bad,
+                                   cudaStream_t s, const int *n_dev) {
   using C = RowCta<NP, T>;
   const unsigned grid = (unsigned)((n_sys + C::SPC / 2 - 1) / (C::SPC / 2));
   if (C::BYTES > 48 * 1024) {
@@ -1174,66 +1140,73 @@ static cudaError_t run_factor_rows(int nb, int n_r, int n_sys, int spr, const TI
     if (e != cudaSuccess) return e;
   }
   k_factor_rows<NP, TIn, T><<<grid, C::THREADS, C::BYTES, s>>>(nb, n_r, n_sys, spr, diag, lower, upper, dinv, ray_list,
-                                                               n_dev);
+                                                               bad, n_dev);
   return cudaGetLastError();
 }
 
+template <int NP>
+static cudaError_t run_factor_row2(int n, int n_r, int n_sys, int spr, const float *diag, const float *lower,
+                                   const float *upper, float *dinv, const int *ray_list, int *bad, cudaStream_t s,
+                                   const int *n_dev) {
+  constexpr int S = Row2<NP>::S;
+  const unsigned grid = (unsigned)((n_sys + S - 1) / S);
+  const auto kern = n == NP ? (bad ? k_factor_row2<NP, true, true> : k_factor_row2<NP, true, false>)
+                            : k_factor_row2<NP, false, true>;
+  kern<<<grid, 64, 0, s>>>(n, n_r, n_sys, spr, diag, lower, upper, dinv, ray_list, bad, n_dev);
+  return cudaGetLastError();
+}
+
+// FP32 (bad: n_sys flags of scratch): the blocks of the outer iteration are, up to the sign of the
+// antineutrinos' rows and columns, M-matrices (the pair process couples the partners with
+// non-negative entries, and its weighted column sums cancel against the diagonal as those of the
+// scattering do), so they are eliminated without row exchanges, two rows per lane; a system in which
+// a pivot block is singular or not finite all the same is done again with partial pivoting.
 cudaError_t launch_factor_rows(int nb, int n_r, int n_sys, int spr, const void *diag, const void *lower,
-                               const void *upper, void *dinv, int fp32, const int *ray_list, cudaStream_t s,
+                               const void *upper, void *dinv, int fp32, int *bad, const int *ray_list, cudaStream_t s,
                                const int *n_dev) {
   if (n_sys == 0) return cudaSuccess;
   if (nb > 48) return cudaErrorInvalidValue;
   if (fp32) {
-    MGFLD_DISPATCH_NPW(nb, return (run_factor_rows<NP, float, float>(nb, n_r, n_sys, spr, (const float *)diag,
-                                                                        (const float *)lower, (const float *)upper,
-                                                                        (float *)dinv, ray_list, s, n_dev)))
+    const float *d = (const float *)diag, *l = (const float *)lower, *u = (const float *)upper;
+    float *out = (float *)dinv;
+    MGFLD_DISPATCH_NPW(nb, {
+      const cudaError_t e = run_factor_row2<NP>(nb, n_r, n_sys, spr, d, l, u, out, ray_list, bad, s, n_dev);
+      if (e != cudaSuccess) return e;
+      return (run_factor_rows<NP, float, float>(nb, n_r, n_sys, spr, d, l, u, out, ray_list, bad, s, n_dev));
+    })
   } else {
     MGFLD_DISPATCH_NPW(nb, return (run_factor_rows<NP, double, double>(nb, n_r, n_sys, spr, (const double *)diag,
                                                                           (const double *)lower, (const double *)upper,
-                                                                          (double *)dinv, ray_list, s, n_dev)))
+                                                                          (double *)dinv, ray_list, nullptr, s, n_dev)))
   }
 }
 
-cudaError_t launch_solve_rows(int nb, int n_r, int n_sys, int spr, const void *dinv, const void *lower,
-                              const void *upper, const double *rhs, float *rhs32, int *sys_exp, double *x, int fp32,
-                              const int *ray_list, cudaStream_t s, const int *n_dev) {
+cudaError_t launch_solve_rows(int nb, int n_r, int n_sys, int spr, const double *dinv, const double *lower,
+                              const double *upper, const double *rhs, double *x, const int *ray_list, cudaStream_t s,
+                              const int *n_dev) {
   if (n_sys == 0) return cudaSuccess;
   if (nb > 48) return cudaErrorInvalidValue;
-  if (fp32) {
-    // per-system power-of-two scaling of the right-hand side for the FP32 sweeps
-    const cudaError_t e = launch_sysmax(nb, n_r, n_sys, rhs, ray_list, spr, sys_exp, rhs32, s, n_dev);
-    if (e != cudaSuccess) return e;
-    MGFLD_DISPATCH_NPW(nb, using C = RowCta<NP, float>;
-                       k_solve_rows<NP, float><<<(unsigned)((n_sys + C::SPC / 2 - 1) / (C::SPC / 2)), C::THREADS, 0, s>>>(
-                           nb, n_r, n_sys, spr, (const float *)dinv, (const float *)lower, (const float *)upper, rhs,
-                           rhs32, sys_exp, x, ray_list, n_dev);
-                       return cudaGetLastError())
-  } else {
-    MGFLD_DISPATCH_NPW(nb, using C = RowCta<NP, double>;
-                       k_solve_rows<NP, double><<<(unsigned)((n_sys + C::SPC / 2 - 1) / (C::SPC / 2)), C::THREADS, 0, s>>>(
-                           nb, n_r, n_sys, spr, (const double *)dinv, (const double *)lower, (const double *)upper, rhs,
-                           nullptr, nullptr, x, ray_list, n_dev);
-                       return cudaGetLastError())
-  }
+  MGFLD_DISPATCH_NPW(nb, using C = RowCta<NP, double>;
+                     k_solve_rows<NP><<<(unsigned)((n_sys + C::SPC / 2 - 1) / (C::SPC / 2)), C::THREADS, 0, s>>>(
+                         nb, n_r, n_sys, spr, dinv, lower, upper, rhs, x, ray_list, n_dev);
+                     return cudaGetLastError())
 }
 
 cudaError_t launch_factor_f32(int n, int n_r, int n_sys, const float *diag, const float *lower32,
-                              const float *upper32, float *dinv, const int *ray_list, cudaStream_t s,
+                              const float *upper32, float *dinv, int *bad, const int *ray_list, cudaStream_t s,
                               const int *n_dev) {
   if (n_sys == 0) return cudaSuccess;
   if (n % 4 == 0) {
-    // blocks of a multiple of 4 rows: two rows per lane
-    MGFLD_DISPATCH_NP(n, constexpr int S = Row2<NP>::S;
-                      k_factor_row2<NP><<<(unsigned)((n_sys + S - 1) / S), 64, 0, s>>>(n_r, n_sys, diag, lower32,
-                                                                                         upper32, dinv, ray_list,
-                                                                                         n_dev);
-                      return cudaGetLastError())
+    MGFLD_DISPATCH_NP(n, return (run_factor_row2<NP>(n, n_r, n_sys, NS, diag, lower32, upper32, dinv, ray_list, nullptr,
+                                                     s, n_dev)))
   }
-  MGFLD_DISPATCH_NP(n, constexpr int W = fw_wpc<NP>();
-                    const unsigned grid = (unsigned)((n_sys + W / 2 - 1) / (W / 2));
-                    k_factor_w32<NP, float, float, false><<<grid, W * 32, 0, s>>>(n, n_r, n_sys, diag, lower32, upper32,
-                                                                            dinv, ray_list, n_dev);
-                    return cudaGetLastError())
+  // padded blocks; a system whose pivots failed again with partial pivoting
+  MGFLD_DISPATCH_NP(n, {
+    const cudaError_t e = run_factor_row2<NP>(n, n_r, n_sys, NS, diag, lower32, upper32, dinv, ray_list, bad, s, n_dev);
+    if (e != cudaSuccess) return e;
+    constexpr int NW = (NP + 7) / 8 * 8;
+    return (run_factor_rows<NW, float, float>(n, n_r, n_sys, NS, diag, lower32, upper32, dinv, ray_list, bad, s, n_dev));
+  })
 }
 
 cudaError_t launch_solve(int n, int n_r, int n_sys, const void *dinv, const double *lower,

@@ -256,8 +256,9 @@ cudaError_t launch_factor(int n, int n_r, int n_sys, const void *diag, int diag_
                           const double *upper, void *dinv, int precision, const int *ray_list,
                           cudaStream_t s, const int *n_dev = nullptr);
 // The FP32 substitution of the outer iteration (blocks, couplings and vectors in the workspace,
-// rhs != x): the right-hand sides are scaled into rhs32 first.  Sets *err on a bounded-wait timeout.
-cudaError_t launch_solve_ring(int n, int n_r, int n_sys, const void *dinv, const float *lower32, const float *upper32,
+// rhs != x; spr systems per ray, n <= 48 for the pair systems' spr = 2): the right-hand sides are scaled into
+// rhs32 first.  Sets *err on a bounded-wait timeout.
+cudaError_t launch_solve_ring(int n, int n_r, int n_sys, int spr, const void *dinv, const float *lower32, const float *upper32,
                               const double *rhs, float *rhs32, double *x, float *g32, const int *ray_list,
                               int *sys_exp, int *err, cudaStream_t s, const int *n_dev = nullptr);
 // Per system (spr per ray): the power of two k that brings max |rhs| into [1/2, 1), and rhs 2^k in FP32.
@@ -273,6 +274,15 @@ cudaError_t launch_sysmax(int n, int n_r, int n_sys, const double *rhs, const in
   else if (n <= 20) { constexpr int NP = 20; __VA_ARGS__; }  \
   else if (n <= 24) { constexpr int NP = 24; __VA_ARGS__; }  \
   else { constexpr int NP = 32; __VA_ARGS__; }
+
+// The same for the wider blocks of the pair systems.
+#define MGFLD_DISPATCH_NPW(n, ...)                          \
+  if (n <= 8) { constexpr int NP = 8; __VA_ARGS__; }          \
+  else if (n <= 16) { constexpr int NP = 16; __VA_ARGS__; }   \
+  else if (n <= 24) { constexpr int NP = 24; __VA_ARGS__; }   \
+  else if (n <= 32) { constexpr int NP = 32; __VA_ARGS__; }   \
+  else if (n <= 40) { constexpr int NP = 40; __VA_ARGS__; }   \
+  else { constexpr int NP = 48; __VA_ARGS__; }
 
 // An opacity entry of (species q, group k) times the optional per-(q, k) scale (no multiplication
 // without a scale: an FP64 operation saved per use, the same value).
@@ -407,9 +417,10 @@ __device__ inline void mu_nue_zone_q(const Eos &e, double A, double B, double T,
   dmu = ((e.g1 - 1.0) * mu_e + T) * (yn * r) + ((e.g2 - 1.0) * mu_nn + T) * (ye * r);
 }
 
-// MIXED-precision factor with FP32 diagonal blocks and FP32 coupling coefficients.
+// MIXED-precision factor with FP32 diagonal blocks and FP32 coupling coefficients (bad: scratch of
+// n_sys ints).
 cudaError_t launch_factor_f32(int n, int n_r, int n_sys, const float *diag, const float *lower32,
-                              const float *upper32, float *dinv, const int *ray_list, cudaStream_t s,
+                              const float *upper32, float *dinv, int *bad, const int *ray_list, cudaStream_t s,
                               const int *n_dev = nullptr);
 // Pair process (pair.cu): the weighted kernels of every zone (after the neutrinosphere scan),
 // and the residual / Jacobian of the coupled pair systems (blocks of 2 n rows, vectors
@@ -420,16 +431,15 @@ cudaError_t launch_assemble_pair(const Prob &p, const Ws &w, const double *psi, 
                                  const int *jac_flag, cudaStream_t s, double *src_out, int first,
                                  const int *n_dev = nullptr);
 
-// Thread-per-row factor and substitution of systems of block width nb <= 48 with spr systems per
-// ray (the coupled nu / antinu pair systems: nb = 2 n, spr = 2), FP64 or FP32 (fp32: float blocks,
-// couplings and factors; the substitution scales each system's right-hand side by a power of two
-// into rhs32 / sys_exp first).
+// Factor and FP64 substitution of systems of block width nb <= 48 with spr systems per ray (the
+// coupled nu / antinu pair systems: nb = 2 n, spr = 2); the factor in FP64 or FP32 (fp32: float
+// blocks, couplings and factors; bad: scratch of n_sys ints).
 cudaError_t launch_factor_rows(int nb, int n_r, int n_sys, int spr, const void *diag, const void *lower,
-                               const void *upper, void *dinv, int fp32, const int *ray_list, cudaStream_t s,
+                               const void *upper, void *dinv, int fp32, int *bad, const int *ray_list, cudaStream_t s,
                                const int *n_dev = nullptr);
-cudaError_t launch_solve_rows(int nb, int n_r, int n_sys, int spr, const void *dinv, const void *lower,
-                              const void *upper, const double *rhs, float *rhs32, int *sys_exp, double *x, int fp32,
-                              const int *ray_list, cudaStream_t s, const int *n_dev = nullptr);
+cudaError_t launch_solve_rows(int nb, int n_r, int n_sys, int spr, const double *dinv, const double *lower,
+                              const double *upper, const double *rhs, double *x, const int *ray_list, cudaStream_t s,
+                              const int *n_dev = nullptr);
 cudaError_t launch_solve(int n, int n_r, int n_sys, const void *dinv, const double *lower,
                          const double *upper, const double *rhs, double *x, int precision,
                          const int *ray_list, cudaStream_t s, const int *n_dev = nullptr);

@@ -80,7 +80,9 @@ cudaError_t launch_sysmax(int n, int n_r, int n_sys, const double *rhs, const in
 // group, and the next step's row and vector entries fetched into registers right after the dot
 // product that frees them.  Measured
 // at 32 / 1024 rays of 512 x 20: 149 -> 89 us / 1146 -> 1080 us (one zone per slot and queue entry
-// before); at 173 rays of 301 x 13 (odd n, on the chain's own global loads before): 650 -> 100 us.
+// before); at 173 rays of 301 x 13 (odd n, on the chain's own global loads before): 650 -> 100 us; the
+// pair systems of 256 rays of 512 x 20 (40-row blocks, a thread per row with CTA barriers before): 2060 ->
+// 530 us.
 template <int NP, int RPL, typename T>
 struct Ring {
   // Zones per group: groups of up to 16 KB, two of them per half, so that the two rings of a CTA leave
@@ -450,14 +452,19 @@ static cudaError_t run_ring(int n, int n_r, int n_sys, int spr, const T *dinv, c
   return cudaGetLastError();
 }
 
-cudaError_t launch_solve_ring(int n, int n_r, int n_sys, const void *dinv, const float *lower32, const float *upper32,
-                              const double *rhs, float *rhs32, double *x, float *g32, const int *ray_list,
-                              int *sys_exp, int *err, cudaStream_t s, const int *n_dev) {
+cudaError_t launch_solve_ring(int n, int n_r, int n_sys, int spr, const void *dinv, const float *lower32,
+                              const float *upper32, const double *rhs, float *rhs32, double *x, float *g32,
+                              const int *ray_list, int *sys_exp, int *err, cudaStream_t s, const int *n_dev) {
   if (n_sys == 0) return cudaSuccess;
-  const cudaError_t e = launch_sysmax(n, n_r, n_sys, rhs, ray_list, NS, sys_exp, rhs32, s, n_dev);
+  const cudaError_t e = launch_sysmax(n, n_r, n_sys, rhs, ray_list, spr, sys_exp, rhs32, s, n_dev);
   if (e != cudaSuccess) return e;
   const float *f = (const float *)dinv;
-  MGFLD_DISPATCH_NP(n, return (run_ring<NP, 1, float>(n, n_r, n_sys, NS, f, lower32, upper32, rhs32, x, g32, ray_list,
+  if (spr != NS) {
+    if (n > 48) return cudaErrorInvalidValue;
+    MGFLD_DISPATCH_NPW(n, return (run_ring<NP, (NP > 32 ? 2 : 1), float>(n, n_r, n_sys, spr, f, lower32, upper32, rhs32,
+                                                                         x, g32, ray_list, sys_exp, err, s, n_dev)))
+  }
+  MGFLD_DISPATCH_NP(n, return (run_ring<NP, 1, float>(n, n_r, n_sys, spr, f, lower32, upper32, rhs32, x, g32, ray_list,
                                                       sys_exp, err, s, n_dev)))
 }
 

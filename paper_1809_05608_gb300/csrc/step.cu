@@ -833,22 +833,22 @@ static cudaError_t enqueue_iteration(const StepCall &c, int it, int n_act, int n
     if (prof) prof->begin(MGFLD_PROF_FACTOR);
     if (pair)
       MGFLD_ENQ(launch_factor_rows(2 * n, NR, nf * 2, 2, w.diag, tl.mixed ? (const void *)w.lower32 : w.lower,
-                                   tl.mixed ? (const void *)w.upper32 : w.upper, w.dinv, tl.mixed, flist, s, cnt_ref));
+                                   tl.mixed ? (const void *)w.upper32 : w.upper, w.dinv, tl.mixed, w.sscale, flist, s,
+                                   cnt_ref));
     else if (tl.mixed)
-      MGFLD_ENQ(launch_factor_f32(n, NR, nf * NS, (const float *)w.diag, w.lower32, w.upper32, (float *)w.dinv, flist,
-                                  s, cnt_ref));
+      MGFLD_ENQ(launch_factor_f32(n, NR, nf * NS, (const float *)w.diag, w.lower32, w.upper32, (float *)w.dinv,
+                                  w.sscale, flist, s, cnt_ref));
     else
       MGFLD_ENQ(launch_factor(n, NR, nf * NS, w.diag, 0, w.lower, w.upper, w.dinv, c.precision, flist, s, cnt_ref));
     if (prof) prof->end(MGFLD_PROF_FACTOR, 1);
   }
   if (prof) prof->begin(MGFLD_PROF_SOLVE);
-  if (pair)
-    MGFLD_ENQ(launch_solve_rows(2 * n, NR, n_act * 2, 2, w.dinv, tl.mixed ? (const void *)w.lower32 : w.lower,
-                                tl.mixed ? (const void *)w.upper32 : w.upper, w.rhs, w.rhs32, w.sscale, w.x, tl.mixed,
+  if (tl.mixed)
+    MGFLD_ENQ(launch_solve_ring(pair ? 2 * n : n, NR, n_act * (pair ? 2 : NS), pair ? 2 : NS, w.dinv, w.lower32, w.upper32,
+                                w.rhs, w.rhs32, w.x, w.g32, w.list_act, w.sscale, w.counters + 3, s, cnt_act));
+  else if (pair)
+    MGFLD_ENQ(launch_solve_rows(2 * n, NR, n_act * 2, 2, (const double *)w.dinv, w.lower, w.upper, w.rhs, w.x,
                                 w.list_act, s, cnt_act));
-  else if (tl.mixed)
-    MGFLD_ENQ(launch_solve_ring(n, NR, n_act * NS, w.dinv, w.lower32, w.upper32, w.rhs, w.rhs32, w.x, w.g32,
-                                w.list_act, w.sscale, w.counters + 3, s, cnt_act));
   else
     MGFLD_ENQ(launch_solve(n, NR, n_act * NS, w.dinv, w.lower, w.upper, w.rhs, w.x, c.precision, w.list_act, s,
                            cnt_act));

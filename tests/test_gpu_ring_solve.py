@@ -44,3 +44,29 @@ def test_group_edges(M, n_r, n_e):
 @pytest.mark.parametrize('n_e', [1, 2, 5, 6, 7, 9, 11, 14, 16, 17, 19, 21, 23, 24, 25, 30, 31, 32])
 def test_block_sizes(M, n_e):
     _check(M, SP.strong(n_ray=3, n_r=21, n_e=n_e, kabs=1e12, kscat=1e13, nes=2.0))
+
+
+@pytest.mark.parametrize('n_e,pair', [(13, False), (10, False), (5, True), (20, True)])
+def test_a_failed_factor_stays_with_its_ray(M, n_e, pair):
+    """A ray whose blocks cannot be eliminated (a NaN temperature in one zone) is done again with
+    partial pivoting, fails on its own and leaves the other rays' results as they are without it."""
+    inp = SP.strong(n_ray=3, n_r=11, n_e=n_e, kabs=1e12, kscat=1e13, nes=2.0, pair=1.0 if pair else 0.0)
+    got = []
+    for poison in (False, True):
+        T0 = np.array(inp['T0'])
+        if poison:
+            T0[1, 4] = np.nan
+        st = M.Stepper(inp, M.MGFLD_MIXED, tol=1e-11, max_iter=60)
+        psi, ye, T = st.state_to_device(inp['psi0'], inp['ye0'], T0)
+        code = st.step(psi, ye, T)
+        assert code == (M.MGFLD_ENAN if poison else M.MGFLD_OK)
+        got.append((psi.cpu().numpy(), st.report['ray_status'].cpu().numpy()))
+    assert got[1][1].tolist() == [M.MGFLD_OK, M.MGFLD_ENAN, M.MGFLD_OK]
+    for ray in (0, 2):
+        assert np.array_equal(got[0][0][ray], got[1][0][ray])
+
+
+@pytest.mark.parametrize('n_r', [1, 2, 5, 9])
+@pytest.mark.parametrize('n_e', [3, 4, 13, 16, 18, 20, 23, 24])
+def test_pair_block_sizes(M, n_e, n_r):
+    _check(M, SP.strong(n_ray=2, n_r=n_r, n_e=n_e, kabs=1e12, kscat=1e13, nes=2.0, pair=1.0))
