@@ -579,7 +579,7 @@ static mgfld_status adjoint_step(const Prob &p, const mgfld_state *s0, const mgf
   k_adj_rhsY<<<nb(Z, 128), 128, 0, s>>>(p, w, a, s1->psi, s1->ye, io->ye_bar, io->T_bar, s0->T, hw);
   k_adj_assembleT<<<nb(F, B), B, 0, s>>>(p, w, a, s1->psi);
   ADJ_CUDA(cudaGetLastError());
-  ADJ_CUDA(launch_factor(p.n, p.n_r, p.n_ray * NS, w.diag, 0, w.lower, w.upper, w.dinv, MGFLD_FP64, nullptr, s));
+  ADJ_CUDA(launch_factor(p.n, p.n_r, p.n_ray * NS, w.diag, w.lower, w.upper, w.dinv, MGFLD_FP64, nullptr, s));
   const int max_sweeps = io->max_sweeps > 0 ? io->max_sweeps : 30;
   const double tol = io->sweep_tol > 0.0 ? io->sweep_tol : 1e-15;
   mgfld_status st = MGFLD_ENOCONV;

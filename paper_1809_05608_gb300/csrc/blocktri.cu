@@ -13,11 +13,7 @@
 // which bounds these latency-limited kernels, is half as long, and there are twice as many
 // independent instruction streams; the arithmetic is unchanged.
 //
-// Thread mapping (FP64): one thread per block row, the two halves of SPC/2 systems per CTA
-// so that SPC * NP is a multiple of 32 and every lane of every FMA instruction does work.
-// Rows and columns beyond the real group count n (<= NP) are padded with the identity.
-// The pivot search, pivot-row broadcast and the natural-order inverse go through
-// shared memory; the inverse of each zone is streamed to the caller's factor buffer.
+// The FP64 elimination is in factor64.cu, the substitution with these factors in solve.cu.
 #include "async.cuh"
 #include "mgfld_internal.cuh"
 
@@ -32,154 +28,13 @@ struct Pack {
   static constexpr int THREADS = SPC * NP;
 };
 
-// 32-bit pivot-search key of row r: the upper word of |x| (sign cleared; non-negative IEEE
-// values order like their bit patterns) with its 5 lowest bits replaced by 31 - r.  One integer
-// max over the keys then finds the largest |x| to 15 mantissa bits, ties going to the lowest
-// row, and the winner's row is 31 - (key & 31).  Rows already used as pivots carry -1.
-__device__ inline int pivot_key(double x, int r) {
-  const unsigned hi = (unsigned)((unsigned long long)__double_as_longlong(x) >> 32) & 0x7fffffffu;
-  return (int)((hi & ~31u) | (unsigned)(31 - r));
-}
-
-template <int NP>
-__device__ inline int max_key(const int *__restrict__ c) {
-  static_assert(NP % 4 == 0, "padded block sizes are multiples of 4");
-  int m[NP / 4];
-#pragma unroll
-  for (int j = 0; j < NP / 4; ++j) {
-    const int4 v = reinterpret_cast<const int4 *>(c)[j];
-    m[j] = max(max(v.x, v.y), max(v.z, v.w));
-  }
-#pragma unroll
-  for (int w = 1; w < NP / 4; w *= 2)
-#pragma unroll
-    for (int j = 0; j + w < NP / 4; j += 2 * w) m[j] = max(m[j], m[j + w]);
-  return m[0];
-}
-
 // Map the j-th system of the launch to a global (ray, species) system index.
 __device__ inline long system_of(long j, const int *ray_list) {
   return ray_list ? (long)ray_list[j / NS] * NS + (j % NS) : j;
 }
 
-template <typename T> __device__ inline T to_t(double v);
-template <> __device__ inline double to_t<double>(double v) { return v; }
-template <> __device__ inline float to_t<float>(double v) { return (float)v; }
-
-// FP64 block-Thomas elimination (one thread per block row, SPC systems per CTA).  Per pivot
-// step: barrier; every row reads the NP candidate keys of its system (NP/4 vector loads, a
-// depth-log2 max tree); the pivot row publishes itself; barrier; every row forms its multiplier
-// with one FMA and updates its NP entries.  The entry of the next pivot column is updated
-// first and its key published at once, so that the next search only waits for that one FMA
-// while the other NP - 1 drain through the FP64 pipe.
-// CTAs per SM the FP64 factor is compiled for (its register budget).
-#ifndef MGFLD_FP64_MINB
-#define MGFLD_FP64_MINB 4
-#endif
-
-template <int NP, typename TIn>
-__global__ void __launch_bounds__(Pack<NP>::THREADS, NP <= 20 ? MGFLD_FP64_MINB : 1)
-k_factor(int n, int n_r, int n_sys, const TIn *__restrict__ diag, const double *__restrict__ lower,
-         const double *__restrict__ upper, double *__restrict__ dinv, const int *__restrict__ ray_list,
-         const int *__restrict__ n_dev) {
-  constexpr int SPC = Pack<NP>::SPC;
-  __shared__ double tile[SPC][NP][NP + 1];           // natural-order inverse of the previous zone
-  __shared__ __align__(16) double prow[SPC][NP];     // pivot row of the current step
-  __shared__ __align__(16) int cand[SPC][NP];        // pivot-search keys
-  __shared__ double ushr[SPC][NP];                   // coupling to the next zone: the column scaling of its Schur term
-  __shared__ int pivrow[SPC][NP];                    // row chosen at each step
-  __shared__ double pinv[SPC];                       // 1 / pivot of the current step
-
-  const int s = threadIdx.x / NP, r = threadIdx.x % NP;
-  const int half = s & 1;                            // 0: zones 0..m top-down, 1: zones n_r-1..m+1 bottom-up
-  const int n_sys_e = listed_sys(n_sys, n_dev, NS);
-  if ((long)blockIdx.x * (SPC / 2) >= n_sys_e) return;   // the whole CTA
-  const long jsys = (long)blockIdx.x * (SPC / 2) + (s >> 1);
-  const bool valid = jsys < n_sys_e;
-  const long sys = valid ? system_of(jsys, ray_list) : 0;
-  const int m = n_r / 2;
-  const int len = half == 0 ? m + 1 : n_r - 1 - m;   // zones of this half; all threads step m + 1 times
-
-  // Each zone's rows are loaded when the zone starts: an FP64 zone step holds the pipe for far
-  // longer than a memory round trip, and the registers of a prefetch would cost resident CTAs.
-  for (int j = 0; j <= m; ++j) {
-    const bool active = j < len;                     // inactive (bottom half, j >= len): dummy identity
-    const int i = half == 0 ? j : n_r - 1 - j;
-    const bool real = valid && active && r < n;
-    const size_t zrow = ((size_t)sys * n_r + (real ? i : 0)) * n + r;   // (sys, i, r)
-    double a[NP];
-#pragma unroll
-    for (int c = 0; c < NP; ++c) a[c] = (real && c < n) ? (double)diag[zrow * n + c] : ((c == r) ? 1.0 : 0.0);
-    const double lr = (real && j > 0) ? (half == 0 ? lower[zrow] : upper[zrow]) : 0.0;
-    if (j > 0 && active) {
-#pragma unroll
-      for (int c = 0; c < NP; ++c) a[c] = fma(-(lr * tile[s][r][c]), ushr[s][c], a[c]);
-    }
-    if (half == 0 && j == m && n_r - 1 > m) {
-      // Middle zone: also subtract the bottom-up half's term diag(u_m) D''^{-1}_{m+1} diag(l_{m+1})
-      // (that half finished at step len - 1 < m; its tile and coupling are kept).
-      const double um = real ? upper[zrow] : 0.0;
-#pragma unroll
-      for (int c = 0; c < NP; ++c) a[c] = fma(-(um * tile[s + 1][r][c]), ushr[s + 1][c], a[c]);
-    }
-
-    // Gauss-Jordan inversion in place with partial pivoting (implicit row exchanges).
-    bool used = false;
-    int my_step = 0;
-    cand[s][r] = pivot_key(a[0], r);
-#pragma unroll
-    for (int pstep = 0; pstep < NP; ++pstep) {
-      __syncthreads();
-      const int best = 31 - (max_key<NP>(cand[s]) & 31);
-      const bool me = (r == best);
-      if (me) {
-        // The pivot entry was updated first in the previous step, so its reciprocal is
-        // formed while the rest of this row is still in the FP64 pipe.
-        pinv[s] = recip(a[pstep]);
-#pragma unroll
-        for (int c = 0; c < NP; c += 2)
-          *reinterpret_cast<double2 *>(&prow[s][c]) = make_double2(a[c], a[c + 1]);
-        pivrow[s][pstep] = r;
-        used = true;
-        my_step = pstep;
-      }
-      __syncthreads();
-      const double inv = pinv[s];
-      // Uniform update for every row: a -= f * pivot_row, with f chosen so that the pivot row
-      // itself becomes pivot_row / pivot (f = 1 - 1/pivot): one FMA either way.  The pivot
-      // column itself is overwritten below, so its update is skipped.
-      const double f = fma(me ? -1.0 : a[pstep], inv, me ? 1.0 : 0.0);
-      if (pstep + 1 < NP) {
-        a[pstep + 1] = fma(-f, prow[s][pstep + 1], a[pstep + 1]);
-        cand[s][r] = used ? -1 : pivot_key(a[pstep + 1], r);
-      }
-      // the rest of the pivot row read from shared memory as it is used (16-byte pieces)
-#pragma unroll
-      for (int c = 0; c < NP; c += 2) {
-        const double2 v = *reinterpret_cast<const double2 *>(&prow[s][c]);
-        if (c != pstep + 1 && c != pstep) a[c] = fma(-f, v.x, a[c]);
-        if (c + 1 != pstep + 1 && c + 1 != pstep) a[c + 1] = fma(-f, v.y, a[c + 1]);
-      }
-      a[pstep] = me ? inv : -f;
-    }
-    // Row r now holds row my_step of the inverse, with column c belonging to input row pivrow[c].
-    __syncthreads();
-    if (active) {
-#pragma unroll
-      for (int c = 0; c < NP; ++c) tile[s][my_step][pivrow[s][c]] = a[c];
-      ushr[s][r] = real ? (half == 0 ? upper[zrow] : lower[zrow]) : 0.0;
-    }
-    __syncthreads();
-    if (real) {
-      double *out = dinv + zrow * n;
-#pragma unroll
-      for (int c = 0; c < NP; ++c)
-        if (c < n) out[c] = tile[s][r][c];
-    }
-  }
-}
-
-// FP64 forward and back substitution with the twisted factors (one thread per block row, the
+// FP64 substitution with factors that a caller of the C ABI holds off the 16-byte boundaries that the
+// ring-fed one (solve.cu) needs; the same operations in the same order (one thread per block row, the
 // two halves of each system in the same CTA, stepping together): forward g_i = Dinv_i (r_i -
 // l_i g_{i-1}) for i < m and h_i = Dinv_i (r_i - u_i h_{i+1}) for i > m, the middle
 // x_m = Dinv_m (r_m - l_m g_{m-1} - u_m h_{m+1}), then back outward from m.  The forward results
@@ -272,10 +127,10 @@ k_solve(int n, int n_r, int n_sys, const double *__restrict__ dinv, const double
 }
 
 // ---------------------------------------------------------------------------------------
-// Thread-per-row elimination and substitution for systems of any block width up to 64 rows
-// (the coupled nu / antinu blocks of the pair process: 2 n_e rows; the substitution in FP64 only), with
+// Thread-per-row elimination of systems of any block width up to 64 rows
+// (the coupled nu / antinu blocks of the pair process: 2 n_e rows), in FP64 or FP32, with
 // `spr` systems per ray (the launch's j-th system is system j % spr of ray ray_list[j / spr]).
-// Same algorithm and thread mapping as k_factor / k_solve above: partial pivoting through integer
+// Same algorithm and thread mapping as k_factor above: partial pivoting through integer
 // keys (6 row bits for blocks wider than 32), the next zone's rows fetched one zone ahead, the
 // pivot row read from shared memory where it is used; shared memory sized at launch.
 template <int NP, typename T>
@@ -426,94 +281,6 @@ k_factor_rows(int n, int n_r, int n_sys, int spr, const TIn *__restrict__ diag, 
       for (int c = 0; c < NP; ++c)
         if (c < n) out[c] = tile[s][r][c];
     }
-  }
-}
-
-// FP64 substitution with those factors (twisted, as k_solve); the forward results are kept in x until
-// the backward sweep replaces them.
-template <int NP>
-__global__ void __launch_bounds__(RowCta<NP, double>::THREADS)
-k_solve_rows(int n, int n_r, int n_sys, int spr, const double *__restrict__ dinv, const double *__restrict__ lower,
-             const double *__restrict__ upper, const double *rhs, double *x, const int *__restrict__ ray_list,
-             const int *__restrict__ n_dev) {
-  using T = double;
-  constexpr int SPC = RowCta<NP, double>::SPC;
-  __shared__ T v[SPC][NP];
-  __shared__ T mid[SPC / 2][NP];
-  const int s = threadIdx.x / NP, r = threadIdx.x % NP;
-  const int half = s & 1, sl = s >> 1;
-  const int n_sys_e = listed_sys(n_sys, n_dev, spr);
-  if ((long)blockIdx.x * (SPC / 2) >= n_sys_e) return;   // the whole CTA
-  const long jsys = (long)blockIdx.x * (SPC / 2) + sl;
-  const bool valid = jsys < n_sys_e;
-  const long sys = valid ? system_of_spr(jsys, ray_list, spr) : 0;
-  const bool realr = valid && r < n;
-  const size_t base = (size_t)sys * n_r * n;
-  const int m = n_r / 2, B = n_r - 1 - m;
-  const int F = half == 0 ? m : B;
-  const T zero = T(0);
-  auto rowdot = [&](int z, bool real) {
-    const T *src = dinv + (base + (size_t)z * n + r) * n;
-    T acc0 = zero, acc1 = zero;
-    if (real) {
-#pragma unroll
-      for (int c = 0; c < NP; c += 2) {
-        if (c < n) acc0 = fma(src[c], v[s][c], acc0);
-        if (c + 1 < n) acc1 = fma(src[c + 1], v[s][c + 1], acc1);
-      }
-    }
-    return acc0 + acc1;
-  };
-  T prev = zero;
-  for (int j = 0; j < m; ++j) {
-    const bool act = j < F;
-    const bool real = realr && act;
-    const int z = half == 0 ? j : n_r - 1 - j;
-    const size_t zr = base + (size_t)(real ? z : 0) * n + r;
-    const T c = (real && j > 0) ? (half == 0 ? lower[zr] : upper[zr]) : zero;
-    const T b = real ? rhs[zr] : zero;
-    v[s][r] = real ? b - c * prev : zero;
-    __syncthreads();
-    const T g = rowdot(z, real);
-    if (real) {
-      x[zr] = g;
-      prev = g;
-    }
-    __syncthreads();
-  }
-  if (half == 1) mid[sl][r] = B > 0 ? prev : zero;
-  __syncthreads();
-  if (half == 0) {
-    const size_t zr = base + (size_t)m * n + r;
-    const T l = (realr && m > 0) ? lower[zr] : zero;
-    const T u = (realr && m < n_r - 1) ? upper[zr] : zero;
-    v[s][r] = realr ? rhs[zr] - l * prev - u * mid[sl][r] : zero;
-  }
-  __syncthreads();
-  if (half == 0) {
-    const T xm = rowdot(m, realr);
-    if (realr) x[base + (size_t)m * n + r] = xm;
-    prev = xm;
-  }
-  __syncthreads();
-  if (half == 0) mid[sl][r] = prev;
-  __syncthreads();
-  if (half == 1) prev = mid[sl][r];
-  for (int j = 0; j < m; ++j) {
-    const bool act = j < F;
-    const bool real = realr && act;
-    const int z = half == 0 ? m - 1 - j : m + 1 + j;
-    const size_t zr = base + (size_t)(real ? z : 0) * n + r;
-    const T c = real ? (half == 0 ? upper[zr] : lower[zr]) : zero;
-    v[s][r] = real ? c * prev : zero;
-    __syncthreads();
-    const T acc = rowdot(z, real);
-    if (real) {
-      const T xi = x[zr] - acc;
-      x[zr] = xi;
-      prev = xi;
-    }
-    __syncthreads();
   }
 }
 
@@ -1079,21 +846,6 @@ k_solve_w32(int n, int n_r, int n_sys, const float *__restrict__ dinv, const dou
 }
 
 template <int NP>
-static cudaError_t run_factor(int n, int n_r, int n_sys, const void *diag, int diag_fp32, const double *lower,
-                              const double *upper, void *dinv, const int *ray_list, cudaStream_t s,
-                              const int *n_dev) {
-  constexpr int SPS = Pack<NP>::SPC / 2;             // systems per CTA
-  const unsigned grid = (unsigned)((n_sys + SPS - 1) / SPS);
-  if (diag_fp32)
-    k_factor<NP, float><<<grid, Pack<NP>::THREADS, 0, s>>>(n, n_r, n_sys, (const float *)diag, lower, upper,
-                                                           (double *)dinv, ray_list, n_dev);
-  else
-    k_factor<NP, double><<<grid, Pack<NP>::THREADS, 0, s>>>(n, n_r, n_sys, (const double *)diag, lower, upper,
-                                                            (double *)dinv, ray_list, n_dev);
-  return cudaGetLastError();
-}
-
-template <int NP>
 static cudaError_t run_solve(int n, int n_r, int n_sys, const void *dinv, const double *lower,
                              const double *upper, const double *rhs, double *x, const int *ray_list,
                              cudaStream_t s, const int *n_dev) {
@@ -1104,28 +856,16 @@ static cudaError_t run_solve(int n, int n_r, int n_sys, const void *dinv, const 
   return cudaGetLastError();
 }
 
-cudaError_t launch_factor(int n, int n_r, int n_sys, const void *diag, int diag_fp32, const double *lower,
-                          const double *upper, void *dinv, int precision, const int *ray_list,
-                          cudaStream_t s, const int *n_dev) {
+cudaError_t launch_factor(int n, int n_r, int n_sys, const double *diag, const double *lower, const double *upper,
+                          void *dinv, int precision, const int *ray_list, cudaStream_t s, const int *n_dev) {
   if (n_sys == 0) return cudaSuccess;
-  if (precision == MGFLD_MIXED) {
-    if (diag_fp32) {
-      MGFLD_DISPATCH_NP(n, constexpr int W = fw_wpc<NP>();
-                        const unsigned grid = (unsigned)((n_sys + W / 2 - 1) / (W / 2));
-                        k_factor_w32<NP, float, double><<<grid, W * 32, 0, s>>>(
-                            n, n_r, n_sys, (const float *)diag, lower, upper, (float *)dinv, ray_list, n_dev);
-                        return cudaGetLastError())
-    } else {
-      MGFLD_DISPATCH_NP(n, constexpr int W = fw_wpc<NP>();
-                        const unsigned grid = (unsigned)((n_sys + W / 2 - 1) / (W / 2));
-                        k_factor_w32<NP, double, double><<<grid, W * 32, 0, s>>>(
-                            n, n_r, n_sys, (const double *)diag, lower, upper, (float *)dinv, ray_list, n_dev);
-                        return cudaGetLastError())
-    }
-  } else {
-    MGFLD_DISPATCH_NP(n, return (run_factor<NP>(n, n_r, n_sys, diag, diag_fp32, lower, upper, dinv,
-                                                        ray_list, s, n_dev)))
-  }
+  if (precision != MGFLD_MIXED)
+    return launch_factor64(n, n_r, n_sys, diag, lower, upper, (double *)dinv, ray_list, s, n_dev);
+  MGFLD_DISPATCH_NP(n, constexpr int W = fw_wpc<NP>();
+                    const unsigned grid = (unsigned)((n_sys + W / 2 - 1) / (W / 2));
+                    k_factor_w32<NP, double, double><<<grid, W * 32, 0, s>>>(n, n_r, n_sys, diag, lower, upper,
+                                                                             (float *)dinv, ray_list, n_dev);
+                    return cudaGetLastError())
 }
 
 template <int NP, typename TIn, typename T>
@@ -1181,17 +921,6 @@ cudaError_t launch_factor_rows(int nb, int n_r, int n_sys, int spr, const void *
   }
 }
 
-cudaError_t launch_solve_rows(int nb, int n_r, int n_sys, int spr, const double *dinv, const double *lower,
-                              const double *upper, const double *rhs, double *x, const int *ray_list, cudaStream_t s,
-                              const int *n_dev) {
-  if (n_sys == 0) return cudaSuccess;
-  if (nb > 48) return cudaErrorInvalidValue;
-  MGFLD_DISPATCH_NPW(nb, using C = RowCta<NP, double>;
-                     k_solve_rows<NP><<<(unsigned)((n_sys + C::SPC / 2 - 1) / (C::SPC / 2)), C::THREADS, 0, s>>>(
-                         nb, n_r, n_sys, spr, dinv, lower, upper, rhs, x, ray_list, n_dev);
-                     return cudaGetLastError())
-}
-
 cudaError_t launch_factor_f32(int n, int n_r, int n_sys, const float *diag, const float *lower32,
                               const float *upper32, float *dinv, int *bad, const int *ray_list, cudaStream_t s,
                               const int *n_dev) {
@@ -1218,7 +947,10 @@ cudaError_t launch_solve(int n, int n_r, int n_sys, const void *dinv, const doub
     MGFLD_DISPATCH_NP(n, k_solve_w32<NP><<<grid, kWarpsPerCta * 32, 0, s>>>(n, n_r, n_sys, (const float *)dinv,
                                                                           lower, upper, rhs, x, ray_list, n_dev);
                          return cudaGetLastError())
+  } else if (((uintptr_t)dinv & 15u) == 0) {
+    return launch_solve_ring64(n, n_r, n_sys, NS, (const double *)dinv, lower, upper, rhs, x, ray_list, nullptr, s, n_dev);
   } else {
+    // a caller's factors off the 16-byte boundaries that bulk copies start on
     MGFLD_DISPATCH_NP(n, return (run_solve<NP>(n, n_r, n_sys, dinv, lower, upper, rhs, x, ray_list, s, n_dev)))
   }
 }

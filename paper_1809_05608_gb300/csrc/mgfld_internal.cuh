@@ -17,6 +17,7 @@ namespace mgfld {
 
 constexpr int NS = 4;                       // nu_e, nubar_e, nu_mu/tau, nubar_mu/tau
 constexpr int MAX_NE = 32;
+constexpr int kSMs = 152;                   // of the GB300
 constexpr double kC = 2.99792458e10;        // cm/s
 constexpr double kHC = 1.23984198e-10;      // MeV cm
 constexpr double kPi = 3.14159265358979323846;
@@ -252,15 +253,21 @@ cudaError_t launch_assemble(const Prob &p, const Ws &w, const double *psi, void 
                             double *lower, double *upper, double *rhs, const int *list, int n_list,
                             const int *jac_flag, cudaStream_t s, double *src_out = nullptr, int first = 0,
                             const int *n_dev = nullptr);
-cudaError_t launch_factor(int n, int n_r, int n_sys, const void *diag, int diag_fp32, const double *lower,
-                          const double *upper, void *dinv, int precision, const int *ray_list,
-                          cudaStream_t s, const int *n_dev = nullptr);
+cudaError_t launch_factor(int n, int n_r, int n_sys, const double *diag, const double *lower, const double *upper,
+                          void *dinv, int precision, const int *ray_list, cudaStream_t s, const int *n_dev = nullptr);
+// The FP64 elimination (factor64.cu).
+cudaError_t launch_factor64(int n, int n_r, int n_sys, const double *diag, const double *lower, const double *upper,
+                            double *dinv, const int *ray_list, cudaStream_t s, const int *n_dev = nullptr);
 // The FP32 substitution of the outer iteration (blocks, couplings and vectors in the workspace,
 // rhs != x; spr systems per ray, n <= 48 for the pair systems' spr = 2): the right-hand sides are scaled into
 // rhs32 first.  Sets *err on a bounded-wait timeout.
 cudaError_t launch_solve_ring(int n, int n_r, int n_sys, int spr, const void *dinv, const float *lower32, const float *upper32,
                               const double *rhs, float *rhs32, double *x, float *g32, const int *ray_list,
                               int *sys_exp, int *err, cudaStream_t s, const int *n_dev = nullptr);
+// The FP64 substitution (dinv on a 16-byte boundary; rhs and x may be one array; err or null).
+cudaError_t launch_solve_ring64(int n, int n_r, int n_sys, int spr, const double *dinv, const double *lower,
+                                const double *upper, const double *rhs, double *x, const int *ray_list, int *err,
+                                cudaStream_t s, const int *n_dev = nullptr);
 // Per system (spr per ray): the power of two k that brings max |rhs| into [1/2, 1), and rhs 2^k in FP32.
 cudaError_t launch_sysmax(int n, int n_r, int n_sys, const double *rhs, const int *ray_list, int spr, int *sys_exp,
                           float *rhs32, cudaStream_t s, const int *n_dev = nullptr);
@@ -431,15 +438,12 @@ cudaError_t launch_assemble_pair(const Prob &p, const Ws &w, const double *psi, 
                                  const int *jac_flag, cudaStream_t s, double *src_out, int first,
                                  const int *n_dev = nullptr);
 
-// Factor and FP64 substitution of systems of block width nb <= 48 with spr systems per ray (the
-// coupled nu / antinu pair systems: nb = 2 n, spr = 2); the factor in FP64 or FP32 (fp32: float
+// Factor of systems of block width nb <= 48 with spr systems per ray (the
+// coupled nu / antinu pair systems: nb = 2 n, spr = 2), in FP64 or FP32 (fp32: float
 // blocks, couplings and factors; bad: scratch of n_sys ints).
 cudaError_t launch_factor_rows(int nb, int n_r, int n_sys, int spr, const void *diag, const void *lower,
                                const void *upper, void *dinv, int fp32, int *bad, const int *ray_list, cudaStream_t s,
                                const int *n_dev = nullptr);
-cudaError_t launch_solve_rows(int nb, int n_r, int n_sys, int spr, const double *dinv, const double *lower,
-                              const double *upper, const double *rhs, double *x, const int *ray_list, cudaStream_t s,
-                              const int *n_dev = nullptr);
 cudaError_t launch_solve(int n, int n_r, int n_sys, const void *dinv, const double *lower,
                          const double *upper, const double *rhs, double *x, int precision,
                          const int *ray_list, cudaStream_t s, const int *n_dev = nullptr);

@@ -114,10 +114,13 @@ __device__ inline void fma4(const float *a, const float *v, float *s) {
   const float2 hi = __ffma2_rn(make_float2(a[2], a[3]), make_float2(v[2], v[3]), make_float2(s[2], s[3]));
   s[0] = lo.x; s[1] = lo.y; s[2] = hi.x; s[3] = hi.y;
 }
+// (FP64: two sums, of the even and of the odd columns, in ascending order)
 __device__ inline void fma4(const double *a, const double *v, double *s) {
 #pragma unroll
-  for (int c = 0; c < 4; ++c) s[c] = fma(a[c], v[c], s[c]);
+  for (int c = 0; c < 4; ++c) s[c & 1] = fma(a[c], v[c], s[c & 1]);
 }
+__device__ inline float sum4(const float *s) { return (s[0] + s[1]) + (s[2] + s[3]); }
+__device__ inline double sum4(const double *s) { return s[0] + s[1]; }
 // The result in the caller's units: FP32 sweeps ran on a right-hand side scaled by 2^-k.  An ordinary
 // value is moved to FP64 and scaled by its bit pattern; the others (and every value where 2^k takes
 // FP32's range out of FP64's, which its 11-bit exponent allows) go through f2d_exp2.
@@ -283,7 +286,7 @@ k_solve_ring(int n, int n_r, int n_sys, int spr, const T *__restrict__ dinv, con
       for (int p = 0; p < RPL; ++p) fma4(&a[p][c], v, s[p]);
     }
 #pragma unroll
-    for (int p = 0; p < RPL; ++p) out[p] = (s[p][0] + s[p][1]) + (s[p][2] + s[p][3]);
+    for (int p = 0; p < RPL; ++p) out[p] = sum4(s[p]);
   };
   int tog = 0;                                              // broadcast buffer of the next step (odd K)
   auto broadcast = [&](int buf, const T *val) {
@@ -466,6 +469,22 @@ cudaError_t launch_solve_ring(int n, int n_r, int n_sys, int spr, const void *di
   }
   MGFLD_DISPATCH_NP(n, return (run_ring<NP, 1, float>(n, n_r, n_sys, spr, f, lower32, upper32, rhs32, x, g32, ray_list,
                                                       sys_exp, err, s, n_dev)))
+}
+
+// FP64 factors (dinv on a 16-byte boundary; rhs and x may be one array; err or null).  Bound by the FP64
+// units with 20 of 32 lanes at work: per substitution at 64 / 256 rays of 512 x 20 1770 -> 495 us /
+// 1834 -> 1634 us, one ray of 64 x 12 115 -> 45 us (a thread per row and CTA barriers before).
+cudaError_t launch_solve_ring64(int n, int n_r, int n_sys, int spr, const double *dinv, const double *lower,
+                                const double *upper, const double *rhs, double *x, const int *ray_list, int *err,
+                                cudaStream_t s, const int *n_dev) {
+  if (n_sys == 0) return cudaSuccess;
+  if (spr != NS) {
+    if (n > 48) return cudaErrorInvalidValue;
+    MGFLD_DISPATCH_NPW(n, return (run_ring<NP, (NP > 16 ? 2 : 1), double>(n, n_r, n_sys, spr, dinv, lower, upper, rhs, x, x,
+                                                                          ray_list, nullptr, err, s, n_dev)))
+  }
+  MGFLD_DISPATCH_NP(n, return (run_ring<NP, 1, double>(n, n_r, n_sys, spr, dinv, lower, upper, rhs, x, x, ray_list,
+                                                       nullptr, err, s, n_dev)))
 }
 
 }  // namespace mgfld

@@ -839,19 +839,16 @@ static cudaError_t enqueue_iteration(const StepCall &c, int it, int n_act, int n
       MGFLD_ENQ(launch_factor_f32(n, NR, nf * NS, (const float *)w.diag, w.lower32, w.upper32, (float *)w.dinv,
                                   w.sscale, flist, s, cnt_ref));
     else
-      MGFLD_ENQ(launch_factor(n, NR, nf * NS, w.diag, 0, w.lower, w.upper, w.dinv, c.precision, flist, s, cnt_ref));
+      MGFLD_ENQ(launch_factor(n, NR, nf * NS, w.diag, w.lower, w.upper, w.dinv, c.precision, flist, s, cnt_ref));
     if (prof) prof->end(MGFLD_PROF_FACTOR, 1);
   }
   if (prof) prof->begin(MGFLD_PROF_SOLVE);
   if (tl.mixed)
     MGFLD_ENQ(launch_solve_ring(pair ? 2 * n : n, NR, n_act * (pair ? 2 : NS), pair ? 2 : NS, w.dinv, w.lower32, w.upper32,
                                 w.rhs, w.rhs32, w.x, w.g32, w.list_act, w.sscale, w.counters + 3, s, cnt_act));
-  else if (pair)
-    MGFLD_ENQ(launch_solve_rows(2 * n, NR, n_act * 2, 2, (const double *)w.dinv, w.lower, w.upper, w.rhs, w.x,
-                                w.list_act, s, cnt_act));
   else
-    MGFLD_ENQ(launch_solve(n, NR, n_act * NS, w.dinv, w.lower, w.upper, w.rhs, w.x, c.precision, w.list_act, s,
-                           cnt_act));
+    MGFLD_ENQ(launch_solve_ring64(pair ? 2 * n : n, NR, n_act * (pair ? 2 : NS), pair ? 2 : NS, (const double *)w.dinv,
+                                  w.lower, w.upper, w.rhs, w.x, w.list_act, w.counters + 3, s, cnt_act));
   if (prof) prof->end(MGFLD_PROF_SOLVE, 1);
   if (prof) prof->begin(MGFLD_PROF_UPDATE);
   if (!pair && n % 2 == 0 && ((uintptr_t)c.st.psi & 15u) == 0)
@@ -1093,7 +1090,7 @@ mgfld_status mgfld_factor(const mgfld_dims *dims, const mgfld_system *sys, int p
   if (!dims_ok(dims) || !sys || !sys->diag || !sys->lower || !sys->upper || !factor ||
       (precision != MGFLD_FP64 && precision != MGFLD_MIXED))
     return MGFLD_EINVAL;
-  MGFLD_CUDA(launch_factor(dims->n_e, dims->n_r, dims->n_ray * NS, sys->diag, 0, sys->lower, sys->upper,
+  MGFLD_CUDA(launch_factor(dims->n_e, dims->n_r, dims->n_ray * NS, sys->diag, sys->lower, sys->upper,
                            factor, precision, nullptr, (cudaStream_t)stream));
   return MGFLD_OK;
 }
