@@ -9,6 +9,7 @@
 //                                                              (Eq. d8, Phi_1 = 0; Phi_in[k,k'] = Phi_out[k',k])
 // and, when the ray is flagged for a new factorisation, the dense row dG_k/dpsi_k' of the
 // diagonal block plus the diagonal couplings to zones i-1 and i+1 (Eq. a62ae).
+#include "async.cuh"
 #include "mgfld_internal.cuh"
 
 namespace mgfld {
@@ -304,16 +305,30 @@ cudaError_t launch_src_mixed(const Prob &p, const Ws &w, const double *psi, doub
 // as the later passes form it (G = psi (D0 + j + gain - lp) - (b0 + j + gain) - couplings) and,
 // where the ray takes new factors, the FP32 Jacobian rows.
 //
-// A block takes whole zones (Z zones of NS n rows, Z NS n <= 256), stages their scaled kernels
-// and the corrections of its rows in shared memory, and runs the two dot products of a row as
+// A block takes a few whole zones of NS n rows (ff_zpb), stages their scaled kernels (asynchronous
+// copies) and the corrections of its rows in shared memory, and runs the two dot products of a row as
 // one sequence of packed FP32x2 operations (the gain and the loss sums side by side).  Rows are
 // threads in the order (zone, species, group) of k_assemble.
-__host__ __device__ inline int ff_zpb(int n) { return (256 / (NS * n)) > 0 ? 256 / (NS * n) : 1; }
-__host__ __device__ inline int ff_ld(int n) { return (n % 2 == 0) ? n + 1 : n; }      // odd row stride in float4
+//
+// What bounds it: 12 FP64 additions and multiply-adds a row (two thirds of the FP64 units' time), the
+// 14 KB a zone that pass through DRAM (0.6 of its bandwidth) and the issue slots (0.6), on a chain of
+// staging, group maxima and row loads whose latency several blocks per SM have to cover.  So: blocks
+// of whole warps, as few as that allows, between barriers; the group count a compile-time constant
+// (a third of the instructions were its divisions, loop control and addressing); the staging without
+// registers; one shared-memory atomic per warp and group.  Measured per pass at 1024 / 32 rays of
+// 512 x 20: 2.12 -> 1.45 ms / 83 -> 59 us; at 173 rays of 301 x 13: 134 -> 114 us (three zones a block,
+// 7.5 warps, and a run-time group count before).
+__host__ __device__ constexpr int ff_zpb(int n) {
+  // the most zones that fill whole warps (5 of them for two zones of 20 groups); else about 128 threads
+  for (int z = 256 / (NS * n); z > 0; --z)
+    if (z * NS * n % 32 == 0) return z;
+  return 128 / (NS * n) > 0 ? 128 / (NS * n) : 1;
+}
+__host__ __device__ constexpr int ff_ld(int n) { return (n % 2 == 0) ? n + 1 : n; }      // odd row stride in float4
 static inline size_t ff_smem(int n) {
   const int z = ff_zpb(n), rows = z * NS * n;
   return sizeof(float4) * (size_t)z * n * ff_ld(n) + sizeof(int2) * (size_t)z * n + sizeof(float2) * rows +
-         2 * sizeof(unsigned) * (size_t)z * NS + sizeof(long long) * (size_t)z;
+         sizeof(unsigned) * (size_t)z * NS + sizeof(long long) * (size_t)z;
 }
 
 // Knuth's two-sum of the two lanes of a pair: s + b -> s, returning its rounding error; the
@@ -343,17 +358,20 @@ __device__ __noinline__ void nes_sums_fp64(const double *__restrict__ fin, const
   *lp = b;
 }
 
-// CTAs of 256 threads per SM the residual kernel is compiled for (its register budget).
+// CTAs of 256 threads per SM the residual kernel is compiled for (its register budget: 40 registers; at
+// 1024 rays 6048 us for four passes with 32, 5819 with 40, 5809 with 48).
 #ifndef MGFLD_FF_MINB
-#define MGFLD_FF_MINB 7
+#define MGFLD_FF_MINB 6
 #endif
 
+// NC: the group count, when the kernel is compiled for it (0: any).
+template <int NC>
 __global__ void __launch_bounds__(256, MGFLD_FF_MINB)
 k_resid_ff(Prob p, Ws w, const double *__restrict__ psi, float *__restrict__ diag, double *__restrict__ lower,
            double *__restrict__ upper, double *__restrict__ rhs, const int *__restrict__ list, int n_list,
            const int *__restrict__ jac_flag, double tolmin, const int *__restrict__ n_dev) {
   extern __shared__ __align__(16) unsigned char ff_sm[];
-  const int n = p.n, ld = ff_ld(n), zpb = ff_zpb(n);
+  const int n = NC ? NC : p.n, ld = ff_ld(n), zpb = NC ? ff_zpb(NC ? NC : 1) : (int)(blockDim.x / (NS * n));
   const unsigned zrows = (unsigned)(NS * n), bt = (unsigned)zpb * zrows, nn = (unsigned)(n * n);
   // (16-byte pieces first, then 8-byte, then 4-byte: every array aligned to its element)
   float4 *tile = reinterpret_cast<float4 *>(ff_sm);                       // [zpb][n][ld]
@@ -361,7 +379,6 @@ k_resid_ff(Prob p, Ws w, const double *__restrict__ psi, float *__restrict__ dia
   int2 *rsc = reinterpret_cast<int2 *>(dff + bt);                          // [zpb][n]
   long long *zoff = reinterpret_cast<long long *>(rsc + (size_t)zpb * n);  // [zpb]: zone index ray n_r + i
   unsigned *gmx = reinterpret_cast<unsigned *>(zoff + zpb);                // [zpb NS]: max |dpsi| (upper words)
-  unsigned *gpx = gmx + (size_t)zpb * NS;                                  // [zpb NS]: max |psi|
   const unsigned per_ray = (unsigned)p.n_r * zrows;
   const unsigned total = (unsigned)listed(n_list, n_dev) * per_ray;
   const unsigned b0 = blockIdx.x * bt;
@@ -394,18 +411,23 @@ k_resid_ff(Prob p, Ws w, const double *__restrict__ psi, float *__restrict__ dia
     const unsigned gz = gz0 + threadIdx.x, zr = gz / p.n_r;
     zoff[threadIdx.x] = (long long)list[zr] * p.n_r + (gz - zr * p.n_r);
   }
-  if (threadIdx.x < (unsigned)zpb * NS) gmx[threadIdx.x] = gpx[threadIdx.x] = 0u;
+  if (threadIdx.x < (unsigned)zpb * NS) gmx[threadIdx.x] = 0u;
   __syncthreads();
   for (unsigned zs = 0; zs < nzb; ++zs) {
     const float4 *src = w.nesff + (size_t)zoff[zs] * nn;
     float4 *dst = tile + (size_t)zs * n * ld;
-    for (unsigned e = threadIdx.x; e < nn; e += bt) dst[e + e / (unsigned)n * (unsigned)(ld - n)] = src[e];
+    for (unsigned e = threadIdx.x; e < nn; e += bt) cp_async16(dst + e + e / (unsigned)n * (unsigned)(ld - n), src + e);
     if (threadIdx.x < (unsigned)n) rsc[zs * n + threadIdx.x] = w.nessc[(size_t)zoff[zs] * n + threadIdx.x];
   }
+  cp_async_commit();
   // the corrections of the block's (zone, species) groups, each scaled by its group's largest
-  if (in) {
-    atomicMax(&gmx[grp], abs_hi_word(dx));
-    atomicMax(&gpx[grp], abs_hi_word(pk));
+  // (the lanes of a warp that share a group reduce first)
+  {
+    const int lane = threadIdx.x & 31, kk = (int)(threadIdx.x - grp * (unsigned)n);
+    const int lo = max(lane - kk, 0), hi = min(lane + n - 1 - kk, 31);
+    const unsigned seg = (0xffffffffu >> (31 - hi)) & (0xffffffffu << lo);
+    const unsigned mx = __reduce_max_sync(seg & __activemask(), abs_hi_word(dx));
+    if (lane == lo) atomicMax(&gmx[grp], mx);
   }
   __syncthreads();
   const int sgrp = scale_of_max(gmx[grp]);
@@ -415,6 +437,7 @@ k_resid_ff(Prob p, Ws w, const double *__restrict__ psi, float *__restrict__ dia
     const float d = d2f_exp2(dx, sgrp);
     dff[threadIdx.x] = make_float2(d, -d);
   }
+  cp_async_wait_all();
   __syncthreads();
   if (!in) return;
 
@@ -422,31 +445,48 @@ k_resid_ff(Prob p, Ws w, const double *__restrict__ psi, float *__restrict__ dia
   const unsigned zs = threadIdx.x / zrows;
   double gain, lp;
   // the pairs while the group's last correction is at most 2^-6 (1.6 %) of max(max |psi|, tolmin),
-  // by exponents (the same decision for every row of the group)
-  if ((int)(gmx[grp] >> 20) + 6 <= (int)(max(gpx[grp], abs_hi_word(tolmin)) >> 20)) {
+  // by exponents (the same decision for every row of the group; the group's psi is looked at only
+  // where the floor does not decide)
+  const int need = (int)(gmx[grp] >> 20) + 6;
+  bool small = need <= (int)(abs_hi_word(tolmin) >> 20);
+  if (!small) {
+    unsigned mp = 0;
+    for (int kp = 0; kp < n; ++kp) mp = max(mp, abs_hi_word(ps[kp]));
+    small = need <= (int)(mp >> 20);
+  }
+  if (small) {
     const float4 *fr = tile + ((size_t)zs * n + k) * ld;
     const float2 *dr = dff + (size_t)grp * n;
-    // (gain, loss) lanes; two running sums (even and odd k') for two independent dependency chains
-    float2 s0 = make_float2(0.f, 0.f), s1 = s0, e0 = s0, e1 = s0;
-    auto term = [&](int kp, float2 &sum, float2 &err) {
+    // (gain, loss) lanes; two running sums (even and odd k') for two independent dependency chains,
+    // their errors in two parts (what adds to the sum: the kernels' lo part and the sums' rounding;
+    // what takes from it: the products' rounding, negated as its FMA forms it)
+    float2 s0 = make_float2(0.f, 0.f), s1 = s0, p0 = s0, p1 = s0, m0 = s0, m1 = s0;
+    auto term = [&](int kp, float2 &sum, float2 &plus, float2 &minus) {
       const float4 f = fr[kp];                       // (in hi, in lo, out hi, out lo)
       const float2 d = dr[kp];                       // (d, -d)
       const float2 fh = make_float2(f.x, f.z), fl = make_float2(f.y, f.w);
       const float2 dh = make_float2(d.x, d.x), nd = make_float2(d.y, d.y);
       const float2 pr = __fmul2_rn(fh, dh);
-      const float2 ex = __ffma2_rn(fh, dh, __fmul2_rn(fh, nd));          // exact product error
-      const float2 cr = __fmul2_rn(fl, dh);                              // the kernels' lo part
-      const float2 e = two_sum2(sum, pr);
-      err = __fadd2_rn(err, __fadd2_rn(__fadd2_rn(ex, cr), e));
+      minus = __fadd2_rn(minus, __ffma2_rn(fh, nd, pr));                 // the rounded product minus the product
+      plus = __fadd2_rn(__ffma2_rn(fl, dh, plus), two_sum2(sum, pr));
     };
-    int kp = 0;
-    for (; kp + 1 < n; kp += 2) {
-      term(kp, s0, e0);
-      term(kp + 1, s1, e1);
+    if (NC) {
+#pragma unroll
+      for (int kp = 0; kp < NC; ++kp) {
+        if (kp % 2 == 0) term(kp, s0, p0, m0);
+        else term(kp, s1, p1, m1);
+      }
+    } else {
+      int kp = 0;
+      for (; kp + 1 < n; kp += 2) {
+        term(kp, s0, p0, m0);
+        term(kp + 1, s1, p1, m1);
+      }
+      if (kp < n) term(kp, s0, p0, m0);
     }
-    if (kp < n) term(kp, s0, e0);
     const float2 e01 = two_sum2(s0, s1);
-    const float2 er = __fadd2_rn(__fadd2_rn(e0, e1), e01);
+    const float2 neg = make_float2(-1.f, -1.f);
+    const float2 er = __ffma2_rn(__fadd2_rn(m0, m1), neg, __fadd2_rn(__fadd2_rn(p0, p1), e01));
     const float2 sm = s0;
     const int2 sc = rsc[zs * n + k];
     const int ug = -(sc.x + sgrp), ul = -(sc.y + sgrp);
@@ -459,13 +499,13 @@ k_resid_ff(Prob p, Ws w, const double *__restrict__ psi, float *__restrict__ dia
   w.g0[g] = gain;
   w.l0[g] = lp;
 
-  const double j = w.jbuf[g];
-  const double dg = ((w.cdiag[g] + j) + gain) - lp;
-  double G = fma(pk, dg, -((w.cb[g] + j) + gain));
-  const double c_up = w.cup[g], c_low = w.clow[g];
-  if (i < last) G = fma(-c_up, ps[k + n], G);
-  if (i > 0) G = fma(-c_low, ps[k - (ptrdiff_t)n], G);
-  rhs[g] = -G;
+  const double jn = w.jbuf[g], cd = w.cdiag[g], cb = w.cb[g], c_up = w.cup[g], c_low = w.clow[g];
+  const double jg = jn + gain;
+  const double dg = (cd + jg) - lp;
+  double b = fma(-pk, dg, cb + jg);                  // -G
+  if (i < last) b = fma(c_up, ps[k + n], b);
+  if (i > 0) b = fma(c_low, ps[k - (ptrdiff_t)n], b);
+  rhs[g] = b;
 
   if (!jac_flag || !jac_flag[ray]) return;
   // a new FP32 Jacobian row for the ray (as k_assemble writes it)
@@ -480,6 +520,13 @@ k_resid_ff(Prob p, Ws w, const double *__restrict__ psi, float *__restrict__ dia
   w.upper32[g] = d2f_exp2(-c_up, 0);
 }
 
+// The kernel compiled for the group count (the 8 to 24 groups of transport grids), or the general one.
+template <int NC>
+static auto resid_ff_kernel(int n) {
+  if constexpr (NC < 8) return k_resid_ff<0>;
+  else return n == NC ? k_resid_ff<NC> : resid_ff_kernel<NC - 1>(n);
+}
+
 cudaError_t launch_resid_ff(const Prob &p, const Ws &w, const double *psi, float *diag, double *lower,
                             double *upper, double *rhs, const int *list, int n_list, const int *jac_flag,
                             double tolmin, cudaStream_t s, const int *n_dev) {
@@ -487,12 +534,13 @@ cudaError_t launch_resid_ff(const Prob &p, const Ws &w, const double *psi, float
   if (zones == 0) return cudaSuccess;
   const int zpb = ff_zpb(p.n);
   const size_t sm = ff_smem(p.n);
+  const auto kern = resid_ff_kernel<24>(p.n);
   if (sm > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(k_resid_ff, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
   }
-  k_resid_ff<<<(unsigned)((zones + zpb - 1) / zpb), zpb * NS * p.n, sm, s>>>(p, w, psi, diag, lower, upper, rhs,
-                                                                            list, n_list, jac_flag, tolmin, n_dev);
+  kern<<<(unsigned)((zones + zpb - 1) / zpb), zpb * NS * p.n, sm, s>>>(p, w, psi, diag, lower, upper, rhs, list, n_list,
+                                                                      jac_flag, tolmin, n_dev);
   return cudaGetLastError();
 }
 

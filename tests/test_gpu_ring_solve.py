@@ -24,8 +24,8 @@ def M():
     return mgfld
 
 
-def _check(M, inp):
-    st = M.Stepper(inp, M.MGFLD_MIXED, tol=1e-11, max_iter=60)
+def _check(M, inp, tol=1e-11):
+    st = M.Stepper(inp, M.MGFLD_MIXED, tol=tol, max_iter=60)
     psi, ye, T = st.state_to_device(inp['psi0'], inp['ye0'], inp['T0'])
     assert st.step(psi, ye, T) == M.MGFLD_OK
     ref = O.step(inp['problem'], inp['psi0'], inp['ye0'], inp['T0'])
@@ -44,6 +44,15 @@ def test_group_edges(M, n_r, n_e):
 @pytest.mark.parametrize('n_e', [1, 2, 5, 6, 7, 9, 11, 14, 16, 17, 19, 21, 23, 24, 25, 30, 31, 32])
 def test_block_sizes(M, n_e):
     _check(M, SP.strong(n_ray=3, n_r=21, n_e=n_e, kabs=1e12, kscat=1e13, nes=2.0))
+
+
+@pytest.mark.parametrize('n_e', [7, 8, 9, 10, 12, 13, 15, 18, 20, 22, 24, 25])
+def test_incremental_residual(M, n_e):
+    """The later residual passes for group counts that the kernel is compiled for and their neighbours,
+    with a last block of fewer zones; from an empty state, so that the first corrections are as large as
+    the occupations and their sums are formed again."""
+    inp = SP.strong(n_ray=3, n_r=7, n_e=n_e, kabs=1e13, kscat=1e13, nes=5.0)
+    _check(M, dict(inp, psi0=1e-3 * inp['psi0']))
 
 
 @pytest.mark.parametrize('n_e,pair', [(13, False), (10, False), (5, True), (20, True)])
