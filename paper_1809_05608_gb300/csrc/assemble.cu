@@ -316,8 +316,9 @@ cudaError_t launch_src_mixed(const Prob &p, const Ws &w, const double *psi, doub
 // of whole warps, as few as that allows, between barriers; the group count a compile-time constant
 // (a third of the instructions were its divisions, loop control and addressing); the staging without
 // registers; one shared-memory atomic per warp and group.  Measured per pass at 1024 / 32 rays of
-// 512 x 20: 2.12 -> 1.45 ms / 83 -> 59 us; at 173 rays of 301 x 13: 134 -> 114 us (three zones a block,
-// 7.5 warps, and a run-time group count before).
+// 512 x 20: 2.12 -> 1.40 ms / 83 -> 57 us; at 173 rays of 301 x 13: 134 -> 104 us (three zones a block,
+// 7.5 warps, and a run-time group count before).  The (gain, loss) pairs of the kernels and the corrections
+// lie in shared memory as the packed operations take them (5819 -> 5583 us for four passes).
 __host__ __device__ constexpr int ff_zpb(int n) {
   // the most zones that fill whole warps (5 of them for two zones of 20 groups); else about 128 threads
   for (int z = 256 / (NS * n); z > 0; --z)
@@ -327,7 +328,7 @@ __host__ __device__ constexpr int ff_zpb(int n) {
 __host__ __device__ constexpr int ff_ld(int n) { return (n % 2 == 0) ? n + 1 : n; }      // odd row stride in float4
 static inline size_t ff_smem(int n) {
   const int z = ff_zpb(n), rows = z * NS * n;
-  return sizeof(float4) * (size_t)z * n * ff_ld(n) + sizeof(int2) * (size_t)z * n + sizeof(float2) * rows +
+  return sizeof(float4) * (size_t)z * n * ff_ld(n) + sizeof(int2) * (size_t)z * n + sizeof(float4) * rows +
          sizeof(unsigned) * (size_t)z * NS + sizeof(long long) * (size_t)z;
 }
 
@@ -359,7 +360,7 @@ __device__ __noinline__ void nes_sums_fp64(const double *__restrict__ fin, const
 }
 
 // CTAs of 256 threads per SM the residual kernel is compiled for (its register budget: 40 registers; at
-// 1024 rays 6048 us for four passes with 32, 5819 with 40, 5809 with 48).
+// 1024 rays 6878 us for four passes with 36, 5583 with 40, 5768 with 48).
 #ifndef MGFLD_FF_MINB
 #define MGFLD_FF_MINB 6
 #endif
@@ -375,7 +376,7 @@ k_resid_ff(Prob p, Ws w, const double *__restrict__ psi, float *__restrict__ dia
   const unsigned zrows = (unsigned)(NS * n), bt = (unsigned)zpb * zrows, nn = (unsigned)(n * n);
   // (16-byte pieces first, then 8-byte, then 4-byte: every array aligned to its element)
   float4 *tile = reinterpret_cast<float4 *>(ff_sm);                       // [zpb][n][ld]
-  float2 *dff = reinterpret_cast<float2 *>(tile + (size_t)zpb * n * ld);   // [bt]: (d, -d)
+  float4 *dff = tile + (size_t)zpb * n * ld;                               // [bt]: (d, d, -d, -d)
   int2 *rsc = reinterpret_cast<int2 *>(dff + bt);                          // [zpb][n]
   long long *zoff = reinterpret_cast<long long *>(rsc + (size_t)zpb * n);  // [zpb]: zone index ray n_r + i
   unsigned *gmx = reinterpret_cast<unsigned *>(zoff + zpb);                // [zpb NS]: max |dpsi| (upper words)
@@ -435,7 +436,7 @@ k_resid_ff(Prob p, Ws w, const double *__restrict__ psi, float *__restrict__ dia
     // the correction of the mixed path comes from the FP32 substitution (an FP32 value times a
     // power of two), so its scaled FP32 form is exact (the lo part of split_ff is zero)
     const float d = d2f_exp2(dx, sgrp);
-    dff[threadIdx.x] = make_float2(d, -d);
+    dff[threadIdx.x] = make_float4(d, d, -d, -d);
   }
   cp_async_wait_all();
   __syncthreads();
@@ -456,16 +457,15 @@ k_resid_ff(Prob p, Ws w, const double *__restrict__ psi, float *__restrict__ dia
   }
   if (small) {
     const float4 *fr = tile + ((size_t)zs * n + k) * ld;
-    const float2 *dr = dff + (size_t)grp * n;
+    const float4 *dr = dff + (size_t)grp * n;
     // (gain, loss) lanes; two running sums (even and odd k') for two independent dependency chains,
     // their errors in two parts (what adds to the sum: the kernels' lo part and the sums' rounding;
     // what takes from it: the products' rounding, negated as its FMA forms it)
     float2 s0 = make_float2(0.f, 0.f), s1 = s0, p0 = s0, p1 = s0, m0 = s0, m1 = s0;
     auto term = [&](int kp, float2 &sum, float2 &plus, float2 &minus) {
-      const float4 f = fr[kp];                       // (in hi, in lo, out hi, out lo)
-      const float2 d = dr[kp];                       // (d, -d)
-      const float2 fh = make_float2(f.x, f.z), fl = make_float2(f.y, f.w);
-      const float2 dh = make_float2(d.x, d.x), nd = make_float2(d.y, d.y);
+      const float4 f = fr[kp], d = dr[kp];           // (in hi, out hi, in lo, out lo), (d, d, -d, -d)
+      const float2 fh = make_float2(f.x, f.y), fl = make_float2(f.z, f.w);
+      const float2 dh = make_float2(d.x, d.y), nd = make_float2(d.z, d.w);
       const float2 pr = __fmul2_rn(fh, dh);
       minus = __fadd2_rn(minus, __ffma2_rn(fh, nd, pr));                 // the rounded product minus the product
       plus = __fadd2_rn(__ffma2_rn(fl, dh, plus), two_sum2(sum, pr));

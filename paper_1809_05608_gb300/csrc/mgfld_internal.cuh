@@ -110,7 +110,7 @@ struct Ws {
   double *rsum;             // [ray][zone][k] row sums of phout: sum_k' phout (1 - psi_k') = rsum - phout.psi
   float *phin32, *phd32;    // FP32 copies for the Jacobian of the mixed path
   // MIXED: the NES kernels as pairs of FP32 values (hi + lo, ~48 bits), each row scaled by a power
-  // of two: nesff[k][k'] = (phin hi, phin lo, phout hi, phout lo) of phin[k][k'] 2^sin_k and
+  // of two: nesff[k][k'] = (phin hi, phout hi, phin lo, phout lo) of phin[k][k'] 2^sin_k and
   // phout[k][k'] 2^sout_k, nessc[k] = (sin_k, sout_k); the later residual passes add the
   // kernels times the last correction to the kept sums in this form (FP32 pipe).
   float4 *nesff;

@@ -242,7 +242,7 @@ __global__ void k_phi(Prob p, Ws w, const double *__restrict__ T, int zpb) {
       w.phin32[base + e] = vf;
       w.phd32[base + e] = __fsub_rn(vf, d2f_exp2(o, 0));
       const float2 fa = split_ff(v, rsc[zz * 2 * n + k]), fb = split_ff(o, rsc[zz * 2 * n + n + k]);
-      w.nesff[base + e] = make_float4(fa.x, fa.y, fb.x, fb.y);
+      w.nesff[base + e] = make_float4(fa.x, fb.x, fa.y, fb.y);
     } else {
       w.phd[base + e] = v - o;
     }
