@@ -11,51 +11,56 @@ __device__ inline long listed_system(long j, const int *ray_list, int spr) {
   return ray_list ? (long)ray_list[j / spr] * spr + (j % spr) : j;
 }
 
-// The power-of-two scaling of one system's right-hand side for the FP32 substitution: k such that
-// max |rhs| 2^k lies in [1/2, 1) (from the largest exponent, so the maximum is taken over the
-// upper words of the bit patterns: integer pipe only), and the FP32 copy rhs 2^k.  All threads of
-// the block call it.
-__device__ inline void sysmax_scale(const double *__restrict__ rhs, int cnt, int *__restrict__ sys_exp,
-                                    float *__restrict__ rhs32) {
-  __shared__ unsigned red[256];
-  __shared__ int kexp_s;
-  unsigned m = 0u;
-  for (int e = threadIdx.x; e < cnt; e += blockDim.x)
-    m = max(m, (unsigned)(__double_as_longlong(rhs[e]) >> 32) & 0x7fffffffu);
-  red[threadIdx.x] = m;
-  __syncthreads();
-  for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) red[threadIdx.x] = max(red[threadIdx.x], red[threadIdx.x + h]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    const int e = (int)(red[0] >> 20);
-    const int k = (e > 0 && e < 0x7ff) ? 1022 - e : 0;
-    *sys_exp = k;
-    kexp_s = k;
-  }
-  __syncthreads();
-  const int k = kexp_s;
-  for (int e = threadIdx.x; e < cnt; e += blockDim.x) rhs32[e] = d2f_exp2(rhs[e], k);
-}
-
-// Per-system power-of-two scaling of the FP32 solve: k with max |rhs| 2^k in [0.5, 1) (the
-// exponent field of the maximum), then the scaled right-hand side rounded to FP32 once, so that
-// the substitution reads FP32 values.  One CTA per listed system (spr systems per ray); its n_r x n
-// right-hand side is contiguous (coalesced loads; the second pass reads it from L2).
-__global__ void k_sysmax(int n, int n_r, const double *__restrict__ rhs, const int *__restrict__ ray_list, int spr,
-                         int *__restrict__ sys_exp, float *__restrict__ rhs32, const int *__restrict__ n_dev) {
+// Per-system power-of-two scaling of the FP32 solve: k such that max |rhs| 2^k lies in [1/2, 1) (from
+// the largest exponent, so the maximum is taken over the upper words of the bit patterns: integer pipe
+// only), then the scaled right-hand side rounded to FP32 once, so that the substitution reads FP32
+// values.  One CTA per listed system (spr systems per ray); its cnt = n_r x n right-hand side is
+// contiguous.  A thread keeps its first kKeep entries in registers between the two uses (whole systems
+// up to 16384 entries), all their loads in flight at once; 256 threads where that holds the system, so that
+// short ones leave room for more CTAs.  Measured at 32 / 1024 rays of 512 x 20: 25 -> 7 us / 175 ->
+// 107 us; at 173 rays of 301 x 13: 17 -> 9 us (256 threads, one load after another, the second pass
+// from L2 before).
+constexpr int kKeep = 16;
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS)
+k_sysmax(int cnt, const double *__restrict__ rhs, const int *__restrict__ ray_list, int spr, int *__restrict__ sys_exp,
+         float *__restrict__ rhs32, const int *__restrict__ n_dev) {
   if ((int)blockIdx.x >= listed_sys(gridDim.x, n_dev, spr)) return;   // the whole block
-  const size_t base = (size_t)listed_system(blockIdx.x, ray_list, spr) * n_r * n;
-  sysmax_scale(rhs + base, n_r * n, sys_exp + blockIdx.x, rhs32 + base);
+  const size_t base = (size_t)listed_system(blockIdx.x, ray_list, spr) * cnt;
+  __shared__ unsigned red[32];
+  double v[kKeep];
+#pragma unroll
+  for (int j = 0; j < kKeep; ++j) {
+    const int e = threadIdx.x + j * THREADS;
+    v[j] = e < cnt ? rhs[base + e] : 0.0;
+  }
+  unsigned m = 0u;
+#pragma unroll
+  for (int j = 0; j < kKeep; ++j) m = max(m, abs_hi_word(v[j]));
+  for (int e = threadIdx.x + kKeep * THREADS; e < cnt; e += THREADS) m = max(m, abs_hi_word(rhs[base + e]));
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  const unsigned wm = (threadIdx.x & 31) < THREADS / 32 ? red[threadIdx.x & 31] : 0u;
+  const int k = scale_of_max(__reduce_max_sync(0xffffffffu, wm));
+  if (threadIdx.x == 0) sys_exp[blockIdx.x] = k;
+#pragma unroll
+  for (int j = 0; j < kKeep; ++j) {
+    const int e = threadIdx.x + j * THREADS;
+    if (e < cnt) rhs32[base + e] = d2f_exp2(v[j], k);
+  }
+  for (int e = threadIdx.x + kKeep * THREADS; e < cnt; e += THREADS) rhs32[base + e] = d2f_exp2(rhs[base + e], k);
 }
 
 cudaError_t launch_sysmax(int n, int n_r, int n_sys, const double *rhs, const int *ray_list, int spr, int *sys_exp,
                           float *rhs32, cudaStream_t s, const int *n_dev) {
-  k_sysmax<<<n_sys, 256, 0, s>>>(n, n_r, rhs, ray_list, spr, sys_exp, rhs32, n_dev);
+  const int cnt = n * n_r;
+  if (cnt <= 256 * kKeep)
+    k_sysmax<256><<<n_sys, 256, 0, s>>>(cnt, rhs, ray_list, spr, sys_exp, rhs32, n_dev);
+  else
+    k_sysmax<1024><<<n_sys, 1024, 0, s>>>(cnt, rhs, ray_list, spr, sys_exp, rhs32, n_dev);
   return cudaGetLastError();
 }
-
 
 // ---------------------------------------------------------------------------------------
 // Ring-fed substitution, one CTA per system: warp 0 takes the top-down half (zones 0..m-1, then the
