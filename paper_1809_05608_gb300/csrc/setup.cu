@@ -90,6 +90,10 @@ __global__ void k_zone(Prob p, Ws w, const double *__restrict__ ye, const double
 // forms each entry pair from its product with the chain's own two multiplications (a = cw_k' P,
 // then a P: down-scattering (out, in) = (a, a P), up-scattering (in, out) = (a, a P)), so the
 // values are those of the chains, bit for bit, from one staged FP64 per entry.
+// The group count is a compile-time constant for 8 to 24 groups (two divisions an entry in the copy-out
+// otherwise), and the row scales of the mixed path come from integer sums of the factors' upper words:
+// 897 -> 783 us at 256 rays of 512 x 20 in FP64, 3544 -> 3338 us at 1024 in the mixed path, whose FP64 units
+// (about 6 instructions an entry) and 16 KB a zone to HBM bound it.
 static inline int phi_threads_per_zone(int n) { return (n + 1) / 2; }
 static inline size_t phi_zone_bytes(int n) {
   return sizeof(double) * ((size_t)n * (n + 1) + 2 * (size_t)n) + sizeof(int) * 2 * (size_t)n;
@@ -115,6 +119,13 @@ static inline size_t phi_smem_bytes(int n) { return (size_t)phi_zones_per_block(
 struct PhiRowMax {
   unsigned in_a, out_a, in_b, out_b;
 };
+// The upper word of a product of two positive values from theirs, up to the carry of the mantissas: the
+// product of the values it stands for is between 1 and 1.125 times it (an integer addition in place of a
+// multiplication that only serves the row scales; 0 where the product is below the normal range).
+__device__ inline unsigned hi_product(unsigned a, unsigned b) {
+  const unsigned s = a + b;
+  return a && b && s > 0x3ff00000u ? s - 0x3ff00000u : 0u;
+}
 __device__ inline void phi_chains(int n, int t, const double *gap, const double *cw, double *sp, int ld, bool want_max,
                                   double &rs_a, double &rs_b, PhiRowMax &mx) {
   const int ka = t, kb = n - 1 - t;                     // ka <= kb; equal for the middle row of odd n
@@ -134,8 +145,8 @@ __device__ inline void phi_chains(int n, int t, const double *gap, const double 
     P *= gap[kp + 1];                                   // e^{-(eps_k - eps_kp)/T}
     const double o = cw[kp] * P;                        // down-scattering k -> kp
     if (first) { pa[kp] = P; rsa += o; } else { pb[kp] = P; rsb += o; }
-    if (want_max) {
-      const unsigned ho = abs_hi_word(o), hv = abs_hi_word(o * P);   // in: cw e^{-2(eps_k - eps_kp)/T}
+    if (want_max) {                                     // in: cw e^{-2(eps_k - eps_kp)/T}
+      const unsigned ho = hi_product(abs_hi_word(cw[kp]), abs_hi_word(P)), hv = hi_product(ho, abs_hi_word(P));
       if (first) { mx.out_a = max(mx.out_a, ho); mx.in_a = max(mx.in_a, hv); }
       else { mx.out_b = max(mx.out_b, ho); mx.in_b = max(mx.in_b, hv); }
     }
@@ -153,7 +164,7 @@ __device__ inline void phi_chains(int n, int t, const double *gap, const double 
     const double o = v * Q;                             // up-scattering k -> kp
     if (first) { pb[kp] = Q; rsb += o; } else { pa[kp] = Q; rsa += o; }
     if (want_max) {
-      const unsigned ho = abs_hi_word(o), hv = abs_hi_word(v);
+      const unsigned hv = hi_product(abs_hi_word(cw[kp]), abs_hi_word(Q)), ho = hi_product(hv, abs_hi_word(Q));
       if (first) { mx.out_b = max(mx.out_b, ho); mx.in_b = max(mx.in_b, hv); }
       else { mx.out_a = max(mx.out_a, ho); mx.in_a = max(mx.in_a, hv); }
     }
@@ -179,9 +190,11 @@ __device__ inline void phi_zone_consts(const Ws &w, int n, int t, int H, double 
   }
 }
 
+// NC: the group count, when the kernel is compiled for it (0: any).
+template <int NC>
 __global__ void k_phi(Prob p, Ws w, const double *__restrict__ T, int zpb) {
   extern __shared__ double smem[];
-  const int n = p.n, H = (n + 1) / 2, ld = n + 1;
+  const int n = NC ? NC : p.n, H = (n + 1) / 2, ld = n + 1;
   double *gapm = smem;                                   // [zpb][n]  e^{-(eps_m - eps_{m-1})/T}
   double *cwm = gapm + (size_t)zpb * n;                   // [zpb][n]  C w_m = C W_m / a^3
   double *sp = cwm + (size_t)zpb * n;                     // [zpb][n][n + 1]  running products
@@ -249,6 +262,13 @@ __global__ void k_phi(Prob p, Ws w, const double *__restrict__ T, int zpb) {
   }
 }
 
+// The kernel compiled for the group count (the 8 to 24 groups of transport grids), or the general one.
+template <int NC>
+static auto phi_kernel(int n) {
+  if constexpr (NC < 8) return k_phi<0>;
+  else return n == NC ? k_phi<NC> : phi_kernel<NC - 1>(n);
+}
+
 // The NES sums of one (zone, group) row for the four species, sum_k' phin_k' psi_k' and
 // sum_k' phout_k' psi_k' (psi of species q at ps0 + q qs), each row entry loaded once for all
 // species; every sum runs over k' in ascending order.  The kernels that call it are bound by
@@ -313,7 +333,7 @@ __global__ void k_jlam(Prob p, Ws w, const double *__restrict__ psi, const doubl
     const double j = kap * e1;
     w.jbuf[g] = j;
     const double kt = kap + j + ksc + gain[q] + (rs - lp[q]);
-    const double y = rsqrt(kt);            // sqrt(lambda): the edge mean free path is a product
+    const double y = w.phin32 ? rsqrt_h(kt) : rsqrt(kt);      // sqrt(lambda): the edge mean free path is a product
     w.kinv[g] = kt;
     w.slam[g] = y;
     w.lam[g] = y * y;
@@ -326,63 +346,90 @@ __global__ void k_jlam(Prob p, Ws w, const double *__restrict__ psi, const doubl
 // Neutrinosphere radius per (ray, q, k): where the optical depth integrated inward from
 // the outer edge reaches 2/3 (linear inside the zone), else the centre edge; then the
 // outer ghost ratio of Eq. a62af with R_nu clamped to the last zone centre.
-// One warp per (ray, q, k): lane c sums the optical depth of the c-th chunk of zones counted
-// from the outer edge, an exclusive warp scan gives each chunk the depth above it, each lane
-// looks for the crossing inside its chunk, and the outermost crossing wins.
+// One block per (ray, q), a thread per (chunk of zones, group): thread (c, k) sums the optical depth of
+// the c-th of 32 chunks of zones counted from the outer edge, a warp per group forms the exclusive
+// prefix over the chunks (the depth above each), the threads whose chunk can hold the crossing look
+// for it there, and the outermost crossing wins.  The threads of a chunk read consecutive groups of the
+// same zones, whole rows of them, and share the zone widths.  Bound by one FP64 multiply-add and one
+// read of 1/lambda an element; measured at 1024 / 32 rays of 512 x 20: 569 -> 171 us / 32 -> 13 us
+// (a warp per (ray, q, k) before, whose lanes read zones 16 rows apart, twice, and formed every width).
 // With a ray list (the outer iteration at the n+1 coefficients) only the listed rays are done.
-__global__ void k_nusphere(Prob p, Ws w, const int *__restrict__ list, int n_list, const int *__restrict__ n_dev) {
+constexpr int kChunks = 32, kMaxWidths = 2048;
+// KEPT: the zone widths in shared memory (n_r <= kMaxWidths).
+template <bool KEPT>
+__global__ void __launch_bounds__(kChunks * MAX_NE)
+k_nusphere(Prob p, Ws w, const int *__restrict__ list, int n_list, const int *__restrict__ n_dev) {
+  extern __shared__ double width[];                // [n_r], up to kMaxWidths zones
+  __shared__ double part[kChunks * MAX_NE], cand[kChunks * MAX_NE];
+  __shared__ int first[MAX_NE];
   const unsigned full = 0xffffffffu;
   const int n = p.n;
-  const int per_ray = NS * n;
-  int t = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (t >= (list ? listed(n_list, n_dev) : p.n_ray) * per_ray) return;   // whole warps leave together
-  if (list) {
-    const int rl = t / per_ray;
-    t = list[rl] * per_ray + (t - rl * per_ray);
-  }
-  const int k = t % n, q = (t / n) % NS, ray = t / (n * NS);
+  const int rl = (int)(blockIdx.x / NS), q = (int)(blockIdx.x % NS);
+  if (rl >= (list ? listed(n_list, n_dev) : p.n_ray)) return;      // the whole block
+  const int ray = list ? list[rl] : rl;
+  const int t = (int)threadIdx.x, c = t / n, k = t - c * n;
   const double *re = p.r_edge + (size_t)ray * (p.n_r + 1);
   const size_t off = ((size_t)ray * NS + q) * p.n_r * n + k;
   const double *kt = w.kinv + off;                 // 1/lambda, so the scan needs no division
-  const int L = (p.n_r + 31) / 32;                 // zones per chunk
-  const int top = p.n_r - 1 - lane * L;            // outermost zone of this lane's chunk
+  const int L = (p.n_r + kChunks - 1) / kChunks;   // zones per chunk
+  const int top = p.n_r - 1 - c * L;               // outermost zone of this chunk
   const int cnt = top < 0 ? 0 : (top + 1 < L ? top + 1 : L);
+  if (KEPT) {
+    for (int i = t; i < p.n_r; i += (int)blockDim.x) width[i] = re[i + 1] - re[i];
+    __syncthreads();
+  }
+  auto dr = [&](int i) { return KEPT ? width[i] : re[i + 1] - re[i]; };
   double s = 0.0;
-  for (int j = 0; j < cnt; ++j) {
-    const int i = top - j;
-    s += (re[i + 1] - re[i]) * kt[(size_t)i * n];
-  }
-  // exclusive prefix over lanes (outer chunks first)
-  double above = s;
+#pragma unroll 8
+  for (int j = 0; j < cnt; ++j) s += dr(top - j) * kt[(size_t)(top - j) * n];
+  part[t] = s;
+  if (t < n) first[t] = kChunks;
+  __syncthreads();
+  {
+    // exclusive prefix over the chunks (outer ones first) of group `wk`, lane = chunk; n warps
+    const int wk = t >> 5, lane = t & 31;
+    const double v0 = part[lane * n + wk];
+    double above = v0;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const double v = __shfl_up_sync(full, above, o);
-    if (lane >= o) above += v;
+    for (int o = 1; o < 32; o <<= 1) {
+      const double v = __shfl_up_sync(full, above, o);
+      if (lane >= o) above += v;
+    }
+    __syncwarp();
+    part[lane * n + wk] = above - v0;
   }
-  double tau_out = above - s;
-  double rnu = 0.0;
-  bool hit = false;
-  for (int j = 0; j < cnt; ++j) {
+  __syncthreads();
+  double tau_out = part[t];
+  // (no crossing where the whole chunk stays below by more than the rounding of its sum)
+  const bool look = !(tau_out + s < kTauNu * (1.0 - 1e-9));
+  for (int j = 0; look && j < cnt; ++j) {
     const int i = top - j;
-    const double dtau = (re[i + 1] - re[i]) * kt[(size_t)i * n];
+    const double dtau = dr(i) * kt[(size_t)i * n];
     if (dbits(tau_out + dtau) >= dbits(kTauNu)) {          // depths >= 0: compared on the integer pipe
-      rnu = re[i + 1] - (kTauNu - tau_out) * w.lam[off + (size_t)i * n];
-      hit = true;
+      cand[t] = re[i + 1] - (kTauNu - tau_out) * w.lam[off + (size_t)i * n];
+      atomicMin(&first[k], c);
       break;
     }
     tau_out += dtau;
   }
-  const unsigned hits = __ballot_sync(full, hit);
-  const int src = hits ? __ffs(hits) - 1 : 0;
-  rnu = hits ? __shfl_sync(full, rnu, src) : re[0];
-  if (lane == 0) {
-    w.rnu[t] = rnu;
+  __syncthreads();
+  if (c == 0) {
+    const int hit = first[k];
+    const double rnu = hit < kChunks ? cand[hit * n + k] : re[0];
+    const int g = (ray * NS + q) * n + k;
+    w.rnu[g] = rnu;
     const double rI = 0.5 * (re[p.n_r - 1] + re[p.n_r]);
     const double rg = 2.0 * re[p.n_r] - rI;
     const double rn = fmin(rnu, rI);
-    w.ghost[t] = (rI * rI - 0.25 * rn * rn) / (rg * rg - 0.25 * rn * rn);
+    w.ghost[g] = (rI * rI - 0.25 * rn * rn) / (rg * rg - 0.25 * rn * rn);
   }
+}
+
+static void launch_nusphere(const Prob &p, const Ws &w, int rays, const int *list, const int *n_dev, cudaStream_t s) {
+  if (p.n_r <= kMaxWidths)
+    k_nusphere<true><<<rays * NS, kChunks * p.n, sizeof(double) * p.n_r, s>>>(p, w, list, rays, n_dev);
+  else
+    k_nusphere<false><<<rays * NS, kChunks * p.n, 0, s>>>(p, w, list, rays, n_dev);
 }
 
 // alpha_{i+1/2} = A_{i+1/2} D_{i+1/2} / a_{i+1/2}^2 with D = lambda_e F / (3 (R_{i+1} - R_i)),
@@ -519,7 +566,7 @@ __global__ void k_lam_iter(Prob p, Ws w, const double *__restrict__ psi, const i
     const size_t g = (((size_t)ray * NS + q) * p.n_r + i) * n + k;
     const double kap = scaled(p, p.kabs, g, q, k), ksc = scaled(p, p.kscat, g, q, k);
     const double kt = kap + w.jbuf[g] + ksc + gain[q] + (rs - lp[q]);
-    const double y = rsqrt(kt);
+    const double y = w.phin32 ? rsqrt_h(kt) : rsqrt(kt);
     w.g0[g] = gain[q];
     w.l0[g] = lp[q];
     w.kinv[g] = kt;
@@ -606,14 +653,15 @@ cudaError_t launch_setup(const Prob &p, const Ws &w, const double *psi, const do
   {
     const int zpb = phi_zones_per_block(p.n);
     const size_t sm = phi_smem_bytes(p.n);
+    const auto kern = phi_kernel<24>(p.n);
     if (sm > 48 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(k_phi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (e != cudaSuccess) return e;
     }
-    k_phi<<<nblk(nz, zpb), zpb * phi_threads_per_zone(p.n), sm, s>>>(p, w, T, zpb);
+    kern<<<nblk(nz, zpb), zpb * phi_threads_per_zone(p.n), sm, s>>>(p, w, T, zpb);
   }
   k_jlam<<<nblk(nzk, B), B, 0, s>>>(p, w, psi, T);
-  k_nusphere<<<nblk((size_t)p.n_ray * NS * p.n * 32, B), B, 0, s>>>(p, w, nullptr, 0, nullptr);   // a warp per (ray, q, k)
+  launch_nusphere(p, w, p.n_ray, nullptr, nullptr, s);
   k_edges<<<nblk(nall, B), B, 0, s>>>(p, w, w.psi_n, nullptr, 0, nullptr);
   if (p.u) k_shock<<<nblk(nall, B), B, 0, s>>>(p, w, w.psi_n);
   if (p.pair && w.pmake) {
@@ -630,7 +678,7 @@ cudaError_t launch_coef_iterate(const Prob &p, const Ws &w, const double *psi, c
   const size_t nzk = (size_t)n_list * p.n_r * p.n;
   const size_t nall = nzk * NS;
   k_lam_iter<<<nblk(nzk, B), B, 0, s>>>(p, w, psi, list, n_list, n_dev);
-  k_nusphere<<<nblk((size_t)n_list * NS * p.n * 32, B), B, 0, s>>>(p, w, list, n_list, n_dev);
+  launch_nusphere(p, w, n_list, list, n_dev, s);
   k_edges<<<nblk(nall, B), B, 0, s>>>(p, w, psi, list, n_list, n_dev);
   return cudaGetLastError();
 }
