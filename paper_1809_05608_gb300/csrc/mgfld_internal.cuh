@@ -402,23 +402,6 @@ __device__ inline double recip2(double d) {
   return fma(x, fma(-d, x, 1.0), x);
 }
 
-// 1/sqrt(d) within about an ulp: an FP32 seed from the mantissa and the parity of the exponent (integer
-// and FP32 pipes) and one third-order step of Householder's iteration, y + y e (1/2 + 3/8 e) with
-// e = 1 - d y^2, whose error is of the order of the cube of the seed's (five FP64 instructions; the
-// library's takes about twice as many).  Zero, negative, subnormal and non-finite d: the library's.
-__device__ inline double rsqrt_h(double d) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(d);
-  const int e = (int)(b >> 52);                                 // (the sign counts as a huge exponent)
-  if (e == 0 || e >= 0x7ff) return rsqrt(d);
-  const int odd = (e - 1023) & 1, h = (e - 1023 - odd) >> 1;
-  const float m = __uint_as_float((unsigned)(127 + odd) << 23 | (unsigned)((b >> 29) & 0x7fffff));
-  const unsigned rb = __float_as_uint(rsqrtf(m));               // in (1/2, 1]
-  const double y = __longlong_as_double((long long)(((unsigned long long)((int)(rb >> 23) + 896 - h) << 52) |
-                                                    ((unsigned long long)(rb & 0x7fffff) << 29)));
-  const double r = fma(-(d * y), y, 1.0);
-  return fma(y * r, fma(0.375, r, 0.5), y);
-}
-
 // Order keys of doubles for comparisons on the integer pipe: the bit pattern of a non-negative
 // value orders like the value, so two non-negative values compare by their patterns (dbits); ord_key
 // maps every non-NaN value to an integer of the same order (-0 just below +0).

@@ -333,7 +333,7 @@ __global__ void k_jlam(Prob p, Ws w, const double *__restrict__ psi, const doubl
     const double j = kap * e1;
     w.jbuf[g] = j;
     const double kt = kap + j + ksc + gain[q] + (rs - lp[q]);
-    const double y = w.phin32 ? rsqrt_h(kt) : rsqrt(kt);      // sqrt(lambda): the edge mean free path is a product
+    const double y = rsqrt(kt);            // sqrt(lambda): the edge mean free path is a product
     w.kinv[g] = kt;
     w.slam[g] = y;
     w.lam[g] = y * y;
@@ -566,7 +566,7 @@ __global__ void k_lam_iter(Prob p, Ws w, const double *__restrict__ psi, const i
     const size_t g = (((size_t)ray * NS + q) * p.n_r + i) * n + k;
     const double kap = scaled(p, p.kabs, g, q, k), ksc = scaled(p, p.kscat, g, q, k);
     const double kt = kap + w.jbuf[g] + ksc + gain[q] + (rs - lp[q]);
-    const double y = w.phin32 ? rsqrt_h(kt) : rsqrt(kt);
+    const double y = rsqrt(kt);
     w.g0[g] = gain[q];
     w.l0[g] = lp[q];
     w.kinv[g] = kt;
