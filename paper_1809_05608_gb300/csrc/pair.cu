@@ -15,76 +15,86 @@
 
 namespace mgfld {
 
-// Shared memory of k_pair per zone: e^{-eps/T} and eps^2 d eps of each group, and the flux
-// factor and cone edge (Eqs. d17, d22) of every species and group.
-__host__ __device__ inline size_t pair_zone_doubles(int n) { return (size_t)(2 + 3 * NS) * n; }
-static inline int pair_zones_per_block(int n) {
-  const int z = 256 / (NS * n);
-  return z < 1 ? 1 : z;
-}
-
-// One thread per (zone, species q, group k): row k of species q's weighted annihilation kernel
+// The pair kernels of every zone, threads (zone, species q, group k): species q's weighted annihilation kernel
 //   pkill[q][k][k'] = C w_k' chi_q(k, k') Phi^a,
-// and (q = 0) row k of the weighted creation kernel, shared by the species,
+// and the weighted creation kernel, shared by the species,
 //   pmake[k][k'] = C w_k' Phi^p(eps_k, eps_k') = C w_k' Phi^a e^{-eps_k/T} e^{-eps_k'/T},
-// with its row sum.  chi = min(chi_1, chi_2) (Eq. d21): chi_1 = 1 - eta eta' / 6 (Eq. d16, the
+// with its row sums.  chi = min(chi_1, chi_2) (Eq. d21): chi_1 = 1 - eta eta' / 6 (Eq. d16, the
 // flux factors eta of species q at eps_k and of its partner at eps_k', the input eta1 clamped to
 // [0, 1]), chi_2 = (8 + (mu mu' - 3)(1 + mu)(1 + mu')) / 8 (Eq. d19) with the cone edges
 // mu = max(sign(x) sqrt|x|, -1), x = 1 - (R_nu / R_i)^2 (Eqs. d17, d22), R_nu each species' and
-// group's neutrinosphere at psi^n and R_i the zone centre.
+// group's neutrinosphere at psi^n and R_i the zone centre.  chi_q(k, k') = chi_qbar(k', k), so it is
+// formed once per pair of species into shared memory (chi_2 = 1 + (m mu' - 3 m8) (1 + mu') with m = mu m8,
+// m8 = (1 + mu) / 8), and the kernels leave from there with consecutive threads on consecutive
+// columns.  Bound by the FP64 units; measured at 256 rays of 512 x 20: 4412 -> 2630 us (a thread per
+// row, which formed chi of both species and stored its row 160 bytes from the next thread's, before).
+static inline int pair_zones_per_block(int n) {
+  // whole warps where some number of zones gives them
+  for (int z = 256 / (NS * n); z > 0; --z)
+    if (z * NS * n % 32 == 0) return z;
+  return 256 / (NS * n) > 0 ? 256 / (NS * n) : 1;
+}
+// per zone: e^{-eps/T} and weights, the flux factors, mu and 1 + mu of every species, chi of both pairs,
+// e^{-eps/T} e^{-eps'/T}
+__host__ __device__ inline size_t pair_zone_doubles(int n) { return (size_t)(2 + 3 * NS) * n + 3 * (size_t)n * (n + 1); }
+
 __global__ void k_pair(Prob p, Ws w, const double *__restrict__ T, int zpb) {
   extern __shared__ double sm[];
-  const int n = p.n, per = NS * n;
+  const int n = p.n, per = NS * n, ld = n + 1;
   const int zl = threadIdx.x / per, rem = threadIdx.x % per, q = rem / n, k = rem % n;
   const unsigned nz = (unsigned)(p.n_ray * p.n_r);
   const unsigned zi = blockIdx.x * (unsigned)zpb + zl;
   const bool live = zl < zpb && zi < nz;
   double *ez = sm + (size_t)(live ? zl : 0) * pair_zone_doubles(n);
-  double *wl = ez + n, *eta = wl + n, *mu = eta + NS * n, *mu1 = mu + NS * n;
-  int ray = 0, i = 0;
+  double *wl = ez + n, *eta = wl + n, *mu = eta + NS * n, *mu1 = mu + NS * n, *chi = mu1 + NS * n;
+  double *mk = chi + 2 * (size_t)n * ld;
   if (live) {
-    ray = (int)(zi / (unsigned)p.n_r);
-    i = (int)(zi - (unsigned)ray * p.n_r);
+    const int ray = (int)(zi / (unsigned)p.n_r), i = (int)(zi - (unsigned)ray * p.n_r);
     const double inv_a = 1.0 / lapse_at(p, ray, i);
     if (q == 0) {
       ez[k] = exp(-(w.E[k] * inv_a) / T[zi]);
       wl[k] = kCNes * p.pair[zi] * (w.W[k] * inv_a * inv_a * inv_a);
     }
     const size_t g = (((size_t)ray * NS + q) * p.n_r + i) * n + k;
-    eta[q * n + k] = p.eta1 ? fmin(fmax(p.eta1[g], 0.0), 1.0) : 0.0;
+    eta[rem] = p.eta1 ? fmin(fmax(p.eta1[g], 0.0), 1.0) : 0.0;
     const double *re = p.r_edge + (size_t)ray * (p.n_r + 1);
     const double rc = 0.5 * (re[i] + re[i + 1]);
     const double rr = w.rnu[((size_t)ray * NS + q) * n + k] / rc;
     const double x = 1.0 - rr * rr;
     const double m = fmax(x > 0.0 ? sqrt(x) : (x < 0.0 ? -sqrt(-x) : 0.0), -1.0);
-    mu[q * n + k] = m;
-    mu1[q * n + k] = 1.0 + m;
+    mu[rem] = m;
+    mu1[rem] = 1.0 + m;
+  }
+  __syncthreads();
+  if (live) {
+    // chi of the even species of the pair, row k, every other column; every fourth column of e e'
+    const int pp = q >> 1, qe = 2 * pp, qb = qe + 1;
+    double *row = chi + ((size_t)pp * n + k) * ld;
+    if (p.pair_chi) {
+      const double e6 = eta[qe * n + k] / 6.0, m8 = 0.125 * mu1[qe * n + k], m = mu[qe * n + k] * m8, m3 = -3.0 * m8;
+      for (int kp = q & 1; kp < n; kp += 2) {
+        const double c1 = fma(-e6, eta[qb * n + kp], 1.0);
+        const double c2 = fma(fma(m, mu[qb * n + kp], m3), mu1[qb * n + kp], 1.0);
+        row[kp] = ord_key(c1) < ord_key(c2) ? c1 : c2;        // the minimum, on the integer pipe
+      }
+    } else {
+      for (int kp = q & 1; kp < n; kp += 2) row[kp] = 1.0;
+    }
+    const double ek = ez[k];
+    for (int kp = q; kp < n; kp += NS) mk[(size_t)k * ld + kp] = ek * ez[kp];
   }
   __syncthreads();
   if (!live) return;
-  const int qb = q ^ 1;
-  double *kill = w.pkill + (((size_t)zi * NS + q) * n + k) * n;
-  if (p.pair_chi) {
-    // the factors of this row taken out of the loop: chi_1 = 1 - (eta / 6) eta', and
-    // chi_2 = 1 + (mu mu' - 3) ((1 + mu) / 8) (1 + mu') (the 1/8 exact)
-    const double e6 = eta[q * n + k] / 6.0, mt = mu[q * n + k], m8 = 0.125 * mu1[q * n + k];
-    for (int kp = 0; kp < n; ++kp) {
-      const double c1 = fma(-e6, eta[qb * n + kp], 1.0);
-      const double c2 = fma(fma(mt, mu[qb * n + kp], -3.0) * m8, mu1[qb * n + kp], 1.0);
-      kill[kp] = wl[kp] * fmin(c1, c2);
-    }
-  } else {
-    for (int kp = 0; kp < n; ++kp) kill[kp] = wl[kp];
-  }
+  // column k of every row (consecutive threads: consecutive columns)
+  const double wk = wl[k];
+  const double *x = chi + (size_t)(q >> 1) * n * ld + ((q & 1) ? k * ld : k);
+  const int xs = (q & 1) ? 1 : ld;
+  double *kill = w.pkill + ((size_t)zi * NS + q) * n * n + k, *make = w.pmake + (size_t)zi * n * n + k;
+  for (int r = 0; r < n; ++r) kill[(size_t)r * n] = wk * x[r * xs];
+  for (int r = q; r < n; r += NS) make[(size_t)r * n] = wk * mk[(size_t)r * ld + k];
   if (q == 0) {
-    double *make = w.pmake + ((size_t)zi * n + k) * n;
-    const double ek = ez[k];
     double ms = 0.0;
-    for (int kp = 0; kp < n; ++kp) {
-      const double v = wl[kp] * (ek * ez[kp]);
-      make[kp] = v;
-      ms += v;
-    }
+    for (int kp = 0; kp < n; ++kp) ms += wl[kp] * mk[(size_t)k * ld + kp];
     w.pmsum[(size_t)zi * n + k] = ms;
   }
 }
@@ -93,6 +103,10 @@ cudaError_t launch_pair(const Prob &p, const Ws &w, const double *T, cudaStream_
   const int zpb = pair_zones_per_block(p.n);
   const size_t nz = (size_t)p.n_ray * p.n_r;
   const size_t sm = sizeof(double) * zpb * pair_zone_doubles(p.n);
+  if (sm > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(k_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+  }
   k_pair<<<(unsigned)((nz + zpb - 1) / zpb), zpb * NS * p.n, sm, s>>>(p, w, T, zpb);
   return cudaGetLastError();
 }
@@ -104,7 +118,8 @@ cudaError_t launch_pair(const Prob &p, const Ws &w, const double *T, cudaStream_
 // S += (1 - psi_k) make - psi_k kill.  Row (s n + k) of the zone's 2 n x 2 n block: the species'
 // own NES block with the diagonal, and the partner's columns
 //   dG_k / d psibar_k' = (1 - psi_k) pmake[k][k'] + psi_k pkill[k][k'].
-// src_out: the converged sources (psi layout) for Eq. a62b and the ledgers.
+// src_out (FP64): the converged sources (psi layout) for Eq. a62b and the ledgers.  Bound by the
+// FP64 multiply-adds of the sums, 4 n a row: 1.95 ms a pass at 256 rays of 512 x 20.
 template <typename TD>
 __global__ void k_assemble_pair(Prob p, Ws w, const double *__restrict__ psi, TD *__restrict__ diag,
                                 double *__restrict__ lower, double *__restrict__ upper, double *__restrict__ rhs,
@@ -146,6 +161,7 @@ __global__ void k_assemble_pair(Prob p, Ws w, const double *__restrict__ psi, TD
       lp += fout[kp] * pv;
     }
   }
+  constexpr bool MIXED = sizeof(TD) == 4;
   const double *mk = w.pmake + (zi * n + k) * n;
   const double *kl = w.pkill + ((zi * NS + q) * n + k) * n;
   double mb = 0.0, kb = 0.0;
@@ -155,11 +171,21 @@ __global__ void k_assemble_pair(Prob p, Ws w, const double *__restrict__ psi, TD
     kb = fma(kl[kp], v, kb);
   }
   const double make = w.pmsum[zi * n + k] - mb, kill = kb;
+  const double j = w.jbuf[g];
+  if (MIXED) {
+    // the sums kept for the final sources (k_src_pair; the pair sums in the storage of 1/lambda and lambda,
+    // which the neutrinosphere scan has consumed)
+    if (!first) {
+      w.g0[g] = gain;
+      w.l0[g] = lp;
+    }
+    w.kinv[g] = mb;
+    w.lam[g] = kb;
+  }
   const double loss = w.rsum[zi * n + k] - lp;
   const double kap = scaled(p, p.kabs, g, q, k);
-  const double j = w.jbuf[g];
   const double S = j * (1.0 - pk) - kap * pk + ((1.0 - pk) * gain - pk * loss) + ((1.0 - pk) * make - pk * kill);
-  if (src_out) {
+  if (!MIXED && src_out) {
     src_out[g] = S;
     return;
   }
@@ -176,6 +202,7 @@ __global__ void k_assemble_pair(Prob p, Ws w, const double *__restrict__ psi, TD
   if (jac_flag && !jac_flag[ray]) return;
   const double jdiag = al_out * (1.0 - gh) + al_in;
   const double dg = inv_acdt + pre * jdiag + j + kap + (gain + loss) + (make + kill);
+  const double c_low = pre * al_in, c_up = i < last ? pre * al_out : 0.0;
   TD *row = diag + gc * n2;
   const int own = sq * n, part = (1 - sq) * n;
   if (sizeof(TD) == 4 && w.phin32) {
@@ -200,13 +227,60 @@ __global__ void k_assemble_pair(Prob p, Ws w, const double *__restrict__ psi, TD
     }
     for (int kp = 0; kp < n; ++kp) row[part + kp] = TD(fma(pk, kl[kp] - mk[kp], mk[kp]));
   }
-  const double c_low = pre * al_in, c_up = i < last ? pre * al_out : 0.0;
   lower[gc] = -c_low;
   upper[gc] = -c_up;
   if (w.lower32) {
     w.lower32[gc] = d2f_exp2(-c_low, 0);
     w.upper32[gc] = d2f_exp2(-c_up, 0);
   }
+}
+
+// The converged sources of the mixed path, as k_src_mixed forms them: the sums of the ray's last residual
+// plus the kernels times the last, sub-tolerance correction in FP32 (the kernels' leading 24 bits), a
+// thread per (zone, species, group), the block's corrections staged as FP32.
+constexpr int kSrcPairThreads = 256;
+__global__ void __launch_bounds__(kSrcPairThreads)
+k_src_pair(Prob p, Ws w, const double *__restrict__ psi, double *__restrict__ src) {
+  extern __shared__ float xs[];                              // the block's zones, [zone][species][group]
+  const int n = p.n, n2 = 2 * n;
+  const unsigned zrows = (unsigned)(NS * n), zpb = blockDim.x / zrows;
+  const unsigned total = (unsigned)(p.n_ray * p.n_r);
+  const unsigned zs = threadIdx.x / zrows, zi = blockIdx.x * zpb + zs, e = threadIdx.x - zs * zrows;
+  const int q = (int)(e / (unsigned)n), k = (int)(e - (unsigned)q * n);
+  const bool in = zi < total;
+  const unsigned ray = in ? zi / (unsigned)p.n_r : 0, i = in ? zi - ray * (unsigned)p.n_r : 0;
+  if (in)
+    xs[threadIdx.x] = (float)w.x[(((size_t)ray * 2 + (q >> 1)) * p.n_r + i) * n2 + (size_t)(q & 1) * n + k];
+  __syncthreads();
+  if (!in) return;
+  const size_t g = (((size_t)ray * NS + q) * p.n_r + i) * n + k, zr = ((size_t)zi * n + k) * n;
+  const float *fi = w.phin32 + zr, *fd = w.phd32 + zr;
+  const double *mk = w.pmake + zr, *kl = w.pkill + (((size_t)zi * NS + q) * n + k) * n;
+  const float *dx = xs + zs * zrows + (size_t)q * n, *dy = xs + zs * zrows + (size_t)(q ^ 1) * n;
+  float dg = 0.f, dl = 0.f, dm = 0.f, dk = 0.f;
+  for (int kp = 0; kp < n; ++kp) {
+    const float d = dx[kp], a = fi[kp], y = dy[kp];
+    dg = fmaf(a, d, dg);
+    dl = fmaf(a - fd[kp], d, dl);
+    dm = fmaf(d2f_exp2(mk[kp], 0), y, dm);
+    dk = fmaf(d2f_exp2(kl[kp], 0), y, dk);
+  }
+  const double pk = psi[g], q1 = 1.0 - pk;
+  const float pf = d2f_exp2(pk, 0);
+  // (1 - psi) (dgain - dmake) + psi (dlp - dkill): the FP32 part of the sources
+  const float corr = fmaf(1.f - pf, dg - dm, pf * (dl - dk));
+  const double kap = scaled(p, p.kabs, g, q, k);
+  const double up = w.g0[g] + (w.pmsum[(size_t)zi * n + k] - w.kinv[g]);
+  const double down = (w.rsum[(size_t)zi * n + k] - w.l0[g]) + w.lam[g];
+  double S = fma(q1, up, fma(-pk, down, (double)corr));
+  S = fma(w.jbuf[g], q1, fma(-kap, pk, S));
+  src[g] = S;
+}
+
+cudaError_t launch_src_pair(const Prob &p, const Ws &w, const double *psi, double *src, cudaStream_t s) {
+  const unsigned zrows = (unsigned)(NS * p.n), zpb = kSrcPairThreads / zrows, zones = (unsigned)(p.n_ray * p.n_r);
+  k_src_pair<<<(zones + zpb - 1) / zpb, zpb * zrows, sizeof(float) * zpb * zrows, s>>>(p, w, psi, src);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_assemble_pair(const Prob &p, const Ws &w, const double *psi, void *diag, int diag_fp32,
