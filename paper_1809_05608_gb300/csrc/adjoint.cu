@@ -123,8 +123,6 @@ __device__ inline double omega(const Prob &p, const Ws &w, int q, int k, double 
 __global__ void k_adj_zone1(Prob p, Ws w, AdjWs a, const double *__restrict__ ye1, const double *__restrict__ Tn) {
   const size_t zi = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (zi >= (size_t)p.n_ray * p.n_r) return;
-  const int n = p.n;
-  const int ray = (int)(zi / p.n_r), i = (int)(zi % p.n_r);
   const double *z = w.zone + zi * ZC_N;
   const double T = Tn[zi];
   double mu1, dmu1, mun, dmun;
@@ -137,44 +135,93 @@ __global__ void k_adj_zone1(Prob p, Ws w, AdjWs a, const double *__restrict__ ye
   za[ZA_DMUN] = dmun;
   za[ZA_MUTN] = log(w.ye_n[zi] / (1.0 - w.ye_n[zi])) + p.eos.log_gn_gp;
   za[ZA_MUY] = 0.0;
-  const double inv_a = z[ZC_INV_A];
-  for (int q = 0; q < NS; ++q) {
-    const size_t g0 = (((size_t)ray * NS + q) * p.n_r + i) * n;
-    for (int k = 0; k < n; ++k) {
-      const double sc = p.scale ? p.scale[q * n + k] : 1.0;
-      bool live;
-      a.j1[g0 + k] = emissivity(p.kabs[g0 + k] * sc, species_mu(q, mu1), w.E[k] * inv_a, T, live);
-    }
-  }
 }
 
-// b_psi = psi_bar + sum_k omega_k dS_k/dpsi_k' at x (transposed source Jacobian).
-__global__ void k_adj_rhs(Prob p, Ws w, AdjWs a, const double *__restrict__ psi1, const double *__restrict__ psib1,
-                          const double *__restrict__ Tb1, double hw) {
-  const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (size_t)p.n_ray * NS * p.n_r * p.n) return;
-  const Elem e = elem_of(p, t);
-  const int n = p.n;
-  const double *z = w.zone + e.zi * ZC_N;
+// The blocks of the element kernels: whole zones, a thread per (zone, group), whole warps where some number
+// of zones gives them.
+constexpr int kAdjThreads = 256;
+static inline int adj_zones(int n) {
+  for (int z = kAdjThreads / n; z > 0; --z)
+    if (z * n % 32 == 0) return z;
+  return kAdjThreads / n;
+}
+
+// The psi half of the system, a thread per (zone, group k) for the four species, which share the entries
+// of the NES kernels: the emissivity at Ye^{n+1} (one exponential for the species with mu = 0); the transposed
+// diagonal blocks (row k of D^T = column k of D) and couplings of J_psi^T; and
+// b_psi = psi_bar + sum_k' omega_k' dS_k'/dpsi_k at x (transposed source Jacobian), which takes the same
+// entries of D.  psi and the two weight vectors omega (nu_e and its antiparticle have one, the others the
+// other) of the block's zones are staged in shared memory.  Bound by the FP64 units, 4 multiply-adds per
+// entry of D; measured at 64 rays of 512 x 20: 1820 -> 763 us (in three kernels with a thread per element, which formed
+// omega and the entries again for each, before).
+__global__ void __launch_bounds__(kAdjThreads)
+k_adj_system(Prob p, Ws w, AdjWs a, const double *__restrict__ psi1, const double *__restrict__ psib1,
+             const double *__restrict__ Tb1, const double *__restrict__ Tn, double hw, int zpb) {
+  extern __shared__ double sm[];                           // per zone: psi [NS][n], omega [2][n]
+  const int n = p.n, last = p.n_r - 1;
+  const unsigned zl = threadIdx.x / (unsigned)n, zu = blockIdx.x * (unsigned)zpb + zl;
+  const int k = (int)(threadIdx.x - zl * (unsigned)n);
+  const bool in = zu < (unsigned)(p.n_ray * p.n_r);
+  const size_t zi = in ? zu : 0;
+  const int ray = (int)(zi / (unsigned)p.n_r), i = (int)(zi - (size_t)ray * p.n_r);
+  const size_t qs = (size_t)p.n_r * n, g0 = ((size_t)ray * NS * p.n_r + i) * n + k, zrow = zi * n;
+  double *ps = sm + (size_t)zl * (NS + 2) * n, *oms = ps + NS * n;
+  const double *z = w.zone + zi * ZC_N;
   const double inv_a = z[ZC_INV_A];
-  const double rho = p.rho[e.zi];
-  const double Tb = Tb1 ? Tb1[e.zi] : 0.0;
-  const double hcoef = in_gain(p, e.ray, e.i) ? hw * (-z[ZC_ACDT] * z[ZC_VOL] * kFourPiHC3) : 0.0;
-  const double *ps = psi1 + (t - e.k);
-  const size_t zrow = e.zi * n;
-  double acc = 0.0, gain = 0.0, lp = 0.0;
-  for (int k = 0; k < n; ++k) {
-    const double om = omega(p, w, e.q, k, inv_a, z, rho, Tb, hcoef);
-    acc += om * (w.phin[(zrow + k) * n + e.k] - ps[k] * w.phd[(zrow + k) * n + e.k]);
-    gain += w.phin[(zrow + e.k) * n + k] * ps[k];
-    lp += w.phout[(zrow + e.k) * n + k] * ps[k];
+  const double rho = p.rho[zi];
+  const double Tb = Tb1 ? Tb1[zi] : 0.0;
+  const double hcoef = in_gain(p, ray, i) ? hw * (-z[ZC_ACDT] * z[ZC_VOL] * kFourPiHC3) : 0.0;
+  const double om_e = omega(p, w, 0, k, inv_a, z, rho, Tb, hcoef);
+  const double om_x = omega(p, w, 2, k, inv_a, z, rho, Tb, hcoef);
+  if (in) {
+#pragma unroll
+    for (int q = 0; q < NS; ++q) ps[q * n + k] = psi1[g0 + q * qs];
+    oms[k] = om_e;
+    oms[n + k] = om_x;
   }
-  const double loss = w.rsum[zrow + e.k] - lp;
-  const double sc = p.scale ? p.scale[e.q * n + e.k] : 1.0;
-  const double kap = p.kabs[t] * sc;
-  const double om_k = omega(p, w, e.q, e.k, inv_a, z, rho, Tb, hcoef);
-  acc -= om_k * (a.j1[t] + kap + gain + loss);
-  a.b[t] = (psib1 ? psib1[t] : 0.0) + acc;
+  __syncthreads();
+  if (!in) return;
+  double acc[NS], gain[NS], lp[NS], dk[NS];
+#pragma unroll
+  for (int q = 0; q < NS; ++q) acc[q] = gain[q] = lp[q] = dk[q] = 0.0;
+  double *row = w.diag + g0 * n;
+  for (int m = 0; m < n; ++m) {
+    const double cin = w.phin[(zrow + m) * n + k], cd = w.phd[(zrow + m) * n + k];
+    const double fin = w.phin[(zrow + k) * n + m], fout = w.phout[(zrow + k) * n + m];
+#pragma unroll
+    for (int q = 0; q < NS; ++q) {
+      const double pm = ps[q * n + m];
+      const double t = fma(-pm, cd, cin);                  // -D[m][k] off the diagonal
+      acc[q] = fma(oms[(q >> 1) * n + m], t, acc[q]);
+      gain[q] = fma(fin, pm, gain[q]);
+      lp[q] = fma(fout, pm, lp[q]);
+      row[q * qs * n + m] = -t;
+      if (m == k) dk[q] = t;
+    }
+  }
+  const double T = Tn[zi], eps = w.E[k] * inv_a, mu1 = a.zadj[zi * 8 + ZA_MU1];
+  const double rs = w.rsum[zrow + k], pre = z[ZC_PRE];
+  const double pre_l = i > 0 ? w.zone[(zi - 1) * ZC_N + ZC_PRE] : 0.0;
+  const double pre_r = i < last ? w.zone[(zi + 1) * ZC_N + ZC_PRE] : 0.0;
+  double e1 = 0.0;
+#pragma unroll
+  for (int q = 0; q < NS; ++q) {
+    const size_t g = g0 + q * qs;
+    bool live;
+    if (q < 3) e1 = emissivity(1.0, species_mu(q, mu1), eps, T, live);
+    const double kap = scaled(p, p.kabs, g, q, k);
+    const double j1 = kap * e1, loss = rs - lp[q];
+    a.j1[g] = j1;
+    const double al_out = w.alpha[g];
+    const double al_in = i > 0 ? w.alpha[g - n] : 0.0;
+    const double gh = (i == last) ? w.ghost[((size_t)ray * NS + q) * n + k] : 0.0;
+    const double dg = z[ZC_INV_ACDT] + pre * (al_out * (1.0 - gh) + al_in) + j1 + kap + gain[q] + loss;
+    row[q * qs * n + k] = dg - dk[q];
+    // J^T couples zone i to i-1 through upper_{i-1} and to i+1 through lower_{i+1}.
+    w.lower[g] = -pre_l * al_in;
+    w.upper[g] = -pre_r * al_out;
+    a.b[g] = (psib1 ? psib1[g] : 0.0) + (acc[q] - (q < 2 ? om_e : om_x) * (j1 + kap + gain[q] + loss));
+  }
 }
 
 // Ye part of the right-hand side and the Ye diagonal of J.
@@ -211,37 +258,6 @@ __global__ void k_adj_rhsY(Prob p, Ws w, AdjWs a, const double *__restrict__ psi
   const double mu_nn = z[ZC_MUB] * (E.g2_is_5_2 ? yn1 * sqrt(yn1) : pow(yn1, E.g2 - 1.0));
   za[ZA_BY] = (yeb1 ? yeb1[zi] : 0.0) + sb - Tb * (mu_e - mu_nn) / E.ec;     // d e_cold/dYe = mu_e - mu_nn
   za[ZA_DYY] = z[ZC_INV_ACDT] + cy * sd;
-}
-
-// Transposed diagonal blocks (row k of D^T = column k of D) and couplings of J_psi^T.
-__global__ void k_adj_assembleT(Prob p, Ws w, AdjWs a, const double *__restrict__ psi1) {
-  const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (size_t)p.n_ray * NS * p.n_r * p.n) return;
-  const Elem e = elem_of(p, t);
-  const int n = p.n, last = p.n_r - 1;
-  const double *z = w.zone + e.zi * ZC_N;
-  const double *ps = psi1 + (t - e.k);
-  const size_t zrow = e.zi * n;
-  double gain = 0.0, lp = 0.0;
-  for (int k = 0; k < n; ++k) {
-    gain += w.phin[(zrow + e.k) * n + k] * ps[k];
-    lp += w.phout[(zrow + e.k) * n + k] * ps[k];
-  }
-  const double loss = w.rsum[zrow + e.k] - lp;
-  const double sc = p.scale ? p.scale[e.q * n + e.k] : 1.0;
-  const double kap = p.kabs[t] * sc;
-  const double al_out = w.alpha[t];
-  const double al_in = e.i > 0 ? w.alpha[t - n] : 0.0;
-  const double gh = (e.i == last) ? w.ghost[((size_t)e.ray * NS + e.q) * n + e.k] : 0.0;
-  const double pre = z[ZC_PRE];
-  const double dg = z[ZC_INV_ACDT] + pre * (al_out * (1.0 - gh) + al_in) + a.j1[t] + kap + gain + loss;
-  double *row = w.diag + t * n;
-  for (int kp = 0; kp < n; ++kp)                       // D[kp][k] = -(phin - psi_kp phd)[kp][k]
-    row[kp] = -(w.phin[(zrow + kp) * n + e.k] - ps[kp] * w.phd[(zrow + kp) * n + e.k]);
-  row[e.k] += dg;
-  // J^T couples zone i to i-1 through upper_{i-1} and to i+1 through lower_{i+1}.
-  w.lower[t] = e.i > 0 ? -w.zone[(e.zi - 1) * ZC_N + ZC_PRE] * w.alpha[t - n] : 0.0;
-  w.upper[t] = e.i < last ? -w.zone[(e.zi + 1) * ZC_N + ZC_PRE] * al_out : 0.0;
 }
 
 // rhs_psi = b_psi - (dG_Y/dpsi)^T mu_Y.
@@ -442,74 +458,107 @@ __global__ void k_adj_rnu(Prob p, Ws w, AdjWs a) {
 }
 
 // Parameter gradients per element (ray, q, i, k): psi^n (time term, flux coefficients, mean
-// free path through the NES sums), and the contributions to the scale, T^n and Ye^n gradients.
-__global__ void k_adj_params(Prob p, Ws w, AdjWs a, const double *__restrict__ psi1, const double *__restrict__ Tn,
-                             const double *__restrict__ Tb1, double hw, double *__restrict__ psib_out) {
-  const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (size_t)p.n_ray * NS * p.n_r * p.n) return;
-  const Elem e = elem_of(p, t);
+// free path through the NES sums), and the contributions to the scale, T^n and Ye^n gradients; a thread per
+// (zone, group) for the four species, which share the NES kernels and their T-derivatives
+//   d phout[k][m]/dT = phout eo(k,m)/T^2,  d phin[k][m]/dT = phin eo(m,k)/T^2
+// and, for the two with mu = 0, the exponential.  What the sums over a zone's row take of each element (psi and
+// 1 - psi of both states and the gradient with respect to 1/lambda) is formed once into shared memory.  Bound
+// by the FP64 units, 5 multiply-adds per entry and species; measured at 64 rays of 512 x 20: 4344 -> 942 us (a
+// thread per element before, which formed all of it for each entry, with a division).
+__global__ void __launch_bounds__(kAdjThreads)
+k_adj_params(Prob p, Ws w, AdjWs a, const double *__restrict__ psi1, const double *__restrict__ Tn,
+             const double *__restrict__ Tb1, double hw, double *__restrict__ psib_out, int zpb) {
+  extern __shared__ double sm[];                           // per zone: five [NS][n] and eps [n]
   const int n = p.n;
-  const double *z = w.zone + e.zi * ZC_N;
-  const double *za = a.zadj + e.zi * 8;
-  const double inv_a = z[ZC_INV_A], inv_a3 = inv_a * inv_a * inv_a;
-  const double T = Tn[e.zi], T2 = T * T, capT = kExpCap * T;
-  const size_t zrow = e.zi * n;
-  const size_t r0 = t - e.k;                        // (ray, q, i, 0)
-  // kappa_t gradient of this zone-species row (the mean free path is 1/kappa_t)
-  const double lam = w.lam[t];
-  const double ktb_self = -lam * lam * a.lamb[t];
-  // psi^n gradient: time term + flux coefficients + sum_k ktb_k d kappa_t,k / d psi^n_k' (= phd[k][k'])
-  double pn = w.x[t] * z[ZC_INV_ACDT] + a.psinb[t];
-  for (int k = 0; k < n; ++k) {
-    const double lk = w.lam[r0 + k];
-    pn += (-lk * lk * a.lamb[r0 + k]) * w.phd[(zrow + k) * n + e.k];
+  const unsigned zl = threadIdx.x / (unsigned)n, zu = blockIdx.x * (unsigned)zpb + zl;
+  const int k = (int)(threadIdx.x - zl * (unsigned)n);
+  const bool in = zu < (unsigned)(p.n_ray * p.n_r);
+  const size_t zi = in ? zu : 0;
+  const int ray = (int)(zi / (unsigned)p.n_r), i = (int)(zi - (size_t)ray * p.n_r);
+  const size_t qs = (size_t)p.n_r * n, g0 = ((size_t)ray * NS * p.n_r + i) * n + k, zrow = zi * n;
+  const int nn = NS * n;
+  double *p1 = sm + (size_t)zl * (5 * NS + 1) * n, *o1 = p1 + nn, *pn = o1 + nn, *on = pn + nn, *kt = on + nn,
+         *es = kt + nn;
+  const double *z = w.zone + zi * ZC_N;
+  const double inv_a = z[ZC_INV_A];
+  const double eps = w.E[k] * inv_a;
+  if (in) {
+#pragma unroll
+    for (int q = 0; q < NS; ++q) {
+      const size_t g = g0 + q * qs;
+      const double x1 = psi1[g], xn = w.psi_n[g], lam = w.lam[g];
+      p1[q * n + k] = x1;
+      o1[q * n + k] = 1.0 - x1;
+      pn[q * n + k] = xn;
+      on[q * n + k] = 1.0 - xn;
+      kt[q * n + k] = -lam * lam * a.lamb[g];              // the mean free path is 1/kappa_t
+    }
+    es[k] = eps;
   }
-  psib_out[t] = pn;
-  // weights of dS/dp: theta (source in G_psi and in the outputs), theta_ae (abs/em in G_Y)
-  const double rho = p.rho[e.zi];
-  const double Tb = Tb1 ? Tb1[e.zi] : 0.0;
-  const double hcoef = in_gain(p, e.ray, e.i) ? hw * (-z[ZC_ACDT] * z[ZC_VOL] * kFourPiHC3) : 0.0;
-  const double theta = w.x[t] + omega(p, w, e.q, e.k, inv_a, z, rho, Tb, hcoef);
-  const double wk = w.W[e.k] * inv_a3;
-  const double cy = kFourPiHC3 * p.eos.mb / rho;
-  const double theta_ae = -za[ZA_MUY] * cy * lepton_sign(e.q) * wk;
-  const double eps = w.E[e.k] * inv_a;
-  const double kin = p.kabs[t], ksin = p.kscat[t];
-  const double pk = psi1[t];
-  // at x: emissivity j1 = kappa e^{x1}, x1 = (mu_q(Ye1, T) - eps)/T
-  const double m1 = species_mu(e.q, za[ZA_MU1]);
-  const bool live1 = m1 - eps < capT;
-  const double ex1 = live1 ? exp((m1 - eps) / T) : exp(kExpCap);
-  const double dSae_ds = (ex1 * (1.0 - pk) - pk) * kin;                 // d S_ae / d s
-  const double muT1 = e.q == 0 ? za[ZA_MUT1] : (e.q == 1 ? -za[ZA_MUT1] : 0.0);
-  const double dx1dT = live1 ? muT1 / T - (m1 - eps) / T2 : 0.0;
-  const double dSae_dT = (1.0 - pk) * a.j1[t] * dx1dT;
-  // at psi^n: emissivity j_n and the NES rates of the mean free path
-  const double mn = species_mu(e.q, z[ZC_MU]);
-  const bool liven = mn - eps < capT;
-  const double exn = liven ? exp((mn - eps) / T) : exp(kExpCap);
-  const double muTn = e.q == 0 ? za[ZA_MUTN] : (e.q == 1 ? -za[ZA_MUTN] : 0.0);
-  const double dxndT = liven ? muTn / T - (mn - eps) / T2 : 0.0;
-  const double dkt_ds = kin * (1.0 + exn) + ksin;
-  double dkt_dT = w.jbuf[t] * dxndT;
-  // T-derivatives of the NES kernels: d phout[k][m]/dT = phout eo(k,m)/T^2, d phin[k][m]/dT = phin eo(m,k)/T^2
-  double g1 = 0.0, l1 = 0.0;
-  const double *ps1 = psi1 + r0;
-  const double *psn = w.psi_n + r0;
+  __syncthreads();
+  if (!in) return;
+  // sk: sum_m ktb_m d kappa_t,m / d psi^n_k (= phd[m][k]); g1, l1, dk: T-derivatives (times T^2) of the gain and
+  // loss at x and of the NES rates of the mean free path at psi^n
+  double sk[NS], g1[NS], l1[NS], dk[NS];
+#pragma unroll
+  for (int q = 0; q < NS; ++q) sk[q] = g1[q] = l1[q] = dk[q] = 0.0;
   for (int m = 0; m < n; ++m) {
-    const double em = w.E[m] * inv_a;
-    const double eo_km = nes_exponent(eps, em, m <= e.k);
-    const double eo_mk = nes_exponent(em, eps, e.k <= m);
-    const double fin = w.phin[(zrow + e.k) * n + m] * eo_mk;
-    const double fout = w.phout[(zrow + e.k) * n + m] * eo_km;
-    g1 += fin * ps1[m];
-    l1 += fout * (1.0 - ps1[m]);
-    dkt_dT += (fin * psn[m] + fout * (1.0 - psn[m])) / T2;
+    const double hd = w.phd[(zrow + m) * n + k];
+    const double fin = w.phin[(zrow + k) * n + m] * nes_exponent(es[m], eps, k <= m);
+    const double fout = w.phout[(zrow + k) * n + m] * nes_exponent(eps, es[m], m <= k);
+#pragma unroll
+    for (int q = 0; q < NS; ++q) {
+      sk[q] = fma(kt[q * n + m], hd, sk[q]);
+      g1[q] = fma(fin, p1[q * n + m], g1[q]);
+      l1[q] = fma(fout, o1[q * n + m], l1[q]);
+      dk[q] = fma(fin, pn[q * n + m], fma(fout, on[q * n + m], dk[q]));
+    }
   }
-  const double dSnes_dT = ((1.0 - pk) * g1 - pk * l1) / T2;
-  a.sS[t] = (theta + theta_ae) * dSae_ds + ktb_self * dkt_ds;
-  a.tT[t] = theta * (dSae_dT + dSnes_dT) + theta_ae * dSae_dT + ktb_self * dkt_dT;
-  a.yY[t] = (e.q < 2 && liven) ? ktb_self * w.jbuf[t] * lepton_sign(e.q) * za[ZA_DMUN] / T : 0.0;
+  const double *za = a.zadj + zi * 8;
+  const double T = Tn[zi], capT = kExpCap * T, inv_T = 1.0 / T, inv_T2 = inv_T * inv_T;
+  const double rho = p.rho[zi];
+  const double Tb = Tb1 ? Tb1[zi] : 0.0;
+  const double hcoef = in_gain(p, ray, i) ? hw * (-z[ZC_ACDT] * z[ZC_VOL] * kFourPiHC3) : 0.0;
+  const double om_e = omega(p, w, 0, k, inv_a, z, rho, Tb, hcoef);
+  const double om_x = omega(p, w, 2, k, inv_a, z, rho, Tb, hcoef);
+  const double wk = w.W[k] * (inv_a * inv_a * inv_a);
+  const double ae = -za[ZA_MUY] * (kFourPiHC3 * p.eos.mb / rho) * wk;
+  double ex1 = 0.0, exn = 0.0, x1 = 0.0, xn = 0.0;
+  bool live1 = false, liven = false;
+#pragma unroll
+  for (int q = 0; q < NS; ++q) {
+    const size_t g = g0 + q * qs;
+    // emissivities kappa e^x, x = (mu_q(Ye, T) - eps)/T, at x and at psi^n
+    if (q < 3) {
+      const double d1 = species_mu(q, za[ZA_MU1]) - eps, dn = species_mu(q, z[ZC_MU]) - eps;
+      live1 = d1 < capT;
+      liven = dn < capT;
+      x1 = d1 / T;
+      ex1 = exp(live1 ? x1 : kExpCap);
+      if (q == 2) {
+        xn = x1;
+        exn = ex1;
+      } else {
+        xn = dn / T;
+        exn = exp(liven ? xn : kExpCap);
+      }
+    }
+    const double muT1 = q == 0 ? za[ZA_MUT1] : (q == 1 ? -za[ZA_MUT1] : 0.0);
+    const double muTn = q == 0 ? za[ZA_MUTN] : (q == 1 ? -za[ZA_MUTN] : 0.0);
+    // weights of dS/dp: theta (source in G_psi and in the outputs), theta_ae (abs/em in G_Y)
+    const double mu = w.x[g], theta = mu + (q < 2 ? om_e : om_x), theta_ae = lepton_sign(q) * ae;
+    const double kin = p.kabs[g], jn = w.jbuf[g];
+    const double pk = p1[q * n + k], qk = o1[q * n + k], ktb = kt[q * n + k];
+    const double dSae_ds = (ex1 * qk - pk) * kin;          // d S_ae / d s
+    const double dSae_dT = qk * a.j1[g] * (live1 ? (muT1 - x1) * inv_T : 0.0);
+    const double dSnes_dT = (qk * g1[q] - pk * l1[q]) * inv_T2;
+    const double dkt_ds = kin * (1.0 + exn) + p.kscat[g];
+    const double dkt_dT = jn * (liven ? (muTn - xn) * inv_T : 0.0) + dk[q] * inv_T2;
+    psib_out[g] = mu * z[ZC_INV_ACDT] + a.psinb[g] + sk[q];
+    a.sS[g] = (theta + theta_ae) * dSae_ds + ktb * dkt_ds;
+    a.tT[g] = theta * (dSae_dT + dSnes_dT) + theta_ae * dSae_dT + ktb * dkt_dT;
+    a.yY[g] = (q < 2 && liven) ? ktb * jn * lepton_sign(q) * za[ZA_DMUN] * inv_T : 0.0;
+  }
 }
 
 // Per zone: T^n and Ye^n gradients.
@@ -575,9 +624,10 @@ static mgfld_status adjoint_step(const Prob &p, const mgfld_state *s0, const mgf
   const double hw = io->heat_weight;
   ADJ_CUDA(launch_setup(p, w, s0->psi, s0->ye, s0->T, s));
   k_adj_zone1<<<nb(Z, 128), 128, 0, s>>>(p, w, a, s1->ye, s0->T);
-  k_adj_rhs<<<nb(F, B), B, 0, s>>>(p, w, a, s1->psi, io->psi_bar, io->T_bar, hw);
+  const int zpb = adj_zones(p.n), zb = zpb * p.n;
+  const size_t sm_zone = sizeof(double) * zb;              // one value per thread of a block
+  k_adj_system<<<nb(Z, zpb), zb, (NS + 2) * sm_zone, s>>>(p, w, a, s1->psi, io->psi_bar, io->T_bar, s0->T, hw, zpb);
   k_adj_rhsY<<<nb(Z, 128), 128, 0, s>>>(p, w, a, s1->psi, s1->ye, io->ye_bar, io->T_bar, s0->T, hw);
-  k_adj_assembleT<<<nb(F, B), B, 0, s>>>(p, w, a, s1->psi);
   ADJ_CUDA(cudaGetLastError());
   ADJ_CUDA(launch_factor(p.n, p.n_r, p.n_ray * NS, w.diag, w.lower, w.upper, w.dinv, MGFLD_FP64, nullptr, s));
   const int max_sweeps = io->max_sweeps > 0 ? io->max_sweeps : 30;
@@ -622,7 +672,8 @@ static mgfld_status adjoint_step(const Prob &p, const mgfld_state *s0, const mgf
   ADJ_CUDA(launch_solve(p.n, p.n_r, p.n_ray * NS, w.dinv, w.lower, w.upper, w.rhs, w.x, MGFLD_FP64, nullptr, s));
   k_adj_flux<<<nb(F, B), B, 0, s>>>(p, w, a, s1->psi);
   k_adj_rnu<<<nb((size_t)p.n_ray * NS * p.n, 128), 128, 0, s>>>(p, w, a);
-  k_adj_params<<<nb(F, B), B, 0, s>>>(p, w, a, s1->psi, s0->T, io->T_bar, hw, io->psi_bar_out);
+  k_adj_params<<<nb(Z, zpb), zb, (5 * NS + 1) * sm_zone, s>>>(p, w, a, s1->psi, s0->T, io->T_bar, hw,
+                                                                  io->psi_bar_out, zpb);
   k_adj_zoneout<<<nb(Z, 128), 128, 0, s>>>(p, w, a, io->T_bar, io->T_bar_out, io->ye_bar_out);
   if (io->scale_bar) k_adj_scale<<<NS * p.n, 256, 0, s>>>(p, a, io->scale_bar);
   ADJ_CUDA(cudaGetLastError());
