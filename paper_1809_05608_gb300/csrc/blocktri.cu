@@ -514,7 +514,7 @@ k_factor_w32(int n, int n_r, int n_sys, const TIn *__restrict__ diag, const TC *
 // ---------------------------------------------------------------------------------------
 // FP32 factor of the outer iteration with two block rows per lane (the mixed path's zone blocks,
 // M-matrices: no row exchanges).  L = NP/2 lanes hold a half-system, lane m rows m and m + L, and a
-// warp holds S = 32 / L half-systems (three at NP = 20, one at the pair systems' NP = 40); warp 0 of a
+// warp holds S = 32 / L half-systems (three at NP = 20); warp 0 of a
 // CTA takes the top-down halves and warp 1 the bottom-up halves of the same S systems.  Every pivot row
 // is read from shared memory once per lane for its two rows, so a broadcast serves twice the rows and S
 // systems at once: the shared-memory traffic per system, which bounds a one-row-per-lane kernel, drops
@@ -527,10 +527,8 @@ k_factor_w32(int n, int n_r, int n_sys, const TIn *__restrict__ diag, const TC *
 // zone ahead.  A zone whose 2 x 2 pivot block is singular or not finite leaves its inverse non-finite;
 // where the launch keeps flags, its system is done again with partial pivoting (without them the outer
 // iteration reports ENAN for the ray).
-// Bound by the latency of the pivot chain.  Measured at 256 rays of 512 x 20 with the pair process (512
-// systems of 40-row blocks) 2.8 ms, against 8.0 ms for one row per thread with CTA barriers and partial
-// pivoting (k_factor_rows); at 173 rays of 301 x 13 (padded to 16) 0.44 ms, against 0.57 ms for one
-// row per lane.
+// Bound by the issue slots of the row updates; measured at 1024 rays of 512 x 20: 2.05 ms.  (Publishing the next
+// pivots before the other row is updated, as k_factor_wide does, spills here: 2.50 ms.)
 template <int NP>
 struct Row2 {
   static constexpr int L = NP / 2;                 // lanes per half-system
@@ -540,12 +538,8 @@ struct Row2 {
 };
 
 // CTAs per SM the two-rows-per-lane factor is compiled for (its register budget).
-#ifndef MGFLD_ROW2_MINB
-#define MGFLD_ROW2_MINB 9
-#endif
-
 template <int NP>
-__host__ __device__ constexpr int row2_minb() { return NP <= 20 ? MGFLD_ROW2_MINB : (NP <= 32 ? 6 : 4); }
+__host__ __device__ constexpr int row2_minb() { return NP <= 20 ? 9 : 6; }
 
 // FULL: n = NP, rows in 16-byte pieces; otherwise rows and columns beyond n are padded with the
 // identity.  spr: systems per ray.  FLAG: bad[listed system] is set to whether a pivot block was
@@ -763,6 +757,228 @@ k_factor_row2(int n_, int n_r, int n_sys, int spr, const float *__restrict__ dia
   }
 }
 
+// The same factor, a warp per half-system, for launches that leave most of the chip idle and for the pair systems:
+// lane (g, m) holds C columns of the R rows m, m + L, ..., the columns dealt to G groups of L lanes (three groups
+// of 8, 8 and 4 columns of two rows at NP = 20, of 16, 16 and 8 columns of four rows at NP = 40), so that a
+// pivot costs a lane a third of the row updates; the multipliers' two columns come from their group by shuffles.
+// The rows that hold the next pivots are updated and published first, the others while those stores are
+// under way.  Every entry takes the same operations in the same order as in k_factor_row2: the same inverses.
+// Bound by the latency of the pivot chain; measured against k_factor_row2 (512 zones): 32 rays of 20 groups
+// 609 -> 325 us, 256 rays 900 -> 689 us, 173 rays of 301 x 13 431 -> 318 us, 256 rays of 40-row pair systems
+// 2.83 -> 2.26 ms (one row per thread with CTA barriers and partial pivoting, k_factor_rows: 8.0 ms).
+template <int NP>
+struct Wide {
+  static constexpr int R = NP > 32 ? 4 : 2;                    // rows per lane
+  static constexpr int L = NP / R;                             // lanes per column group
+  static constexpr int G0 = 32 / L < NP / 4 ? 32 / L : NP / 4;
+  static constexpr int C = ((NP + G0 - 1) / G0 + 3) / 4 * 4;   // columns per lane
+  static constexpr int G = (NP + C - 1) / C;                   // column groups
+  static constexpr int W = G * C;                              // padded row
+};
+
+template <int NP, bool FULL, bool FLAG>
+__global__ void __launch_bounds__(64)
+k_factor_wide(int n_, int n_r, int n_sys, int spr, const float *__restrict__ diag, const float *__restrict__ lower,
+              const float *__restrict__ upper, float *__restrict__ dinv, const int *__restrict__ ray_list,
+              int *__restrict__ bad, const int *__restrict__ n_dev) {
+  using Q = Wide<NP>;
+  constexpr int R = Q::R, L = Q::L, C = Q::C, G = Q::G, W = Q::W;
+  static_assert(NP % 4 == 0 && L % 2 == 0 && L * G <= 32, "pivot pairs in one lane pair, rows in 16-byte pieces");
+  const int n = FULL ? NP : n_;
+  // (columns from NP to W stay zero throughout)
+  __shared__ __align__(16) float rows[2][NP][W];           // the next zone's rows, per warp
+  __shared__ __align__(16) float cpl[2][2][NP];            // its couplings (to the previous / next zone)
+  __shared__ __align__(16) float prow[2][2][2][W];         // per warp, double-buffered pivot row pairs
+  __shared__ __align__(16) float ucol[2][W];               // column scaling of the next zone's Schur term
+  __shared__ int okb;                                      // the bottom-up half's pivots were fine
+  const int half = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool act = lane < L * G;                           // the other lanes repeat the first group's and store nothing
+  const int cg = act ? lane / L : 0, mm = lane % L, c0 = cg * C;
+  const long jsys = blockIdx.x;
+  if (jsys >= listed_sys(n_sys, n_dev, spr)) return;       // the whole CTA
+  const size_t sys = (size_t)system_of_spr(jsys, ray_list, spr);
+  const int m = n_r / 2;
+  const int len = half == 0 ? m + 1 : n_r - 1 - m;
+  auto zone = [&](int j) { return half == 0 ? j : n_r - 1 - j; };
+  if (act) {
+    // what no copy touches: the identity, without couplings
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int r = mm + i * L;
+#pragma unroll
+      for (int c = 0; c < C; ++c)
+        if (r >= n || c0 + c >= n) rows[half][r][c0 + c] = c0 + c == r ? 1.f : 0.f;
+      if (cg == 0 && r >= n) cpl[half][0][r] = cpl[half][1][r] = 0.f;
+    }
+    if (mm == 0) {
+#pragma unroll
+      for (int c = 0; c < C; ++c) ucol[half][c0 + c] = 0.f;
+    }
+  }
+  __syncwarp();
+  auto issue = [&](int j) {                                // rows and couplings of zone j
+    if (act && j < len) {
+      const size_t zb = (sys * n_r + zone(j)) * n;
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        const int r = mm + i * L;
+        if (FULL || r < n) {
+          const float *src = diag + (zb + r) * n + c0;
+          float *dst = &rows[half][r][c0];
+          if (FULL) {
+#pragma unroll
+            for (int c = 0; c < C; c += 4)
+              if (c0 + c < NP) cp_async16(dst + c, src + c);
+          } else if (n % 2 == 0) {
+            for (int c = 0; c < C && c0 + c < n; c += 2) cp_async8(dst + c, src + c);
+          } else {
+            for (int c = 0; c < C && c0 + c < n; ++c) cp_async4(dst + c, src + c);
+          }
+          if (cg == 0) {
+            cp_async4(&cpl[half][0][r], (half == 0 ? lower : upper) + zb + r);
+            cp_async4(&cpl[half][1][r], (half == 0 ? upper : lower) + zb + r);
+          }
+        }
+      }
+    }
+    cp_async_commit();
+  };
+  float (*midt)[W] = rows[1];                              // the bottom-up warp's last inverse
+  float a[R][C];
+  bool ok = true;
+  issue(0);
+  for (int j = 0; j < len; ++j) {
+    cp_async_wait_all();
+    __syncwarp();
+    // the zone's rows minus the Schur term of the previous zone
+    float u[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const float l = cpl[half][0][mm + i * L];
+      u[i] = cpl[half][1][mm + i * L];
+#pragma unroll
+      for (int c = 0; c < C; c += 4) {
+        float4 x = *reinterpret_cast<const float4 *>(&rows[half][mm + i * L][c0 + c]);
+        if (j > 0) {
+          const float4 v = *reinterpret_cast<const float4 *>(&ucol[half][c0 + c]);
+          x.x = fmaf(-(l * a[i][c]), v.x, x.x);
+          x.y = fmaf(-(l * a[i][c + 1]), v.y, x.y);
+          x.z = fmaf(-(l * a[i][c + 2]), v.z, x.z);
+          x.w = fmaf(-(l * a[i][c + 3]), v.w, x.w);
+        }
+        a[i][c] = x.x; a[i][c + 1] = x.y; a[i][c + 2] = x.z; a[i][c + 3] = x.w;
+      }
+    }
+    __syncwarp();                                          // every lane has read the rows, couplings and ucol
+    issue(j + 1);
+    if (half == 0 && j == m) {
+      // middle zone: wait for the bottom-up half and subtract its term diag(u_m) D''^{-1}_{m+1} diag(l_{m+1})
+      asm volatile("bar.sync 1, 64;" ::: "memory");
+      if (n_r - 1 > m) {
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          const float lc = ucol[1][c0 + c];
+#pragma unroll
+          for (int i = 0; i < R; ++i) a[i][c] = fmaf(-(u[i] * midt[mm + i * L][c0 + c]), lc, a[i][c]);
+        }
+      }
+    }
+    // rows p and p + 1 to the pivot buffer
+    auto publish = [&](int p) {
+      if (act && (mm == p % L || mm == p % L + 1)) {
+        float *dst = &prow[half][(p / 2) & 1][mm - p % L][c0];
+        const float (&x)[C] = a[p / L];
+#pragma unroll
+        for (int c = 0; c < C; c += 4) *reinterpret_cast<float4 *>(dst + c) = make_float4(x[c], x[c + 1], x[c + 2], x[c + 3]);
+      }
+    };
+    publish(0);
+#pragma unroll
+    for (int b = 0; b < NP / 2; ++b) {
+      const int p = 2 * b, pl = p % L, pg = p / C, pc = p % C;
+      const float (*pb)[W] = prow[half][b & 1];
+      // columns p and p + 1 of this lane's rows, from the group that holds them
+      float xp[R], yp[R];
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        xp[i] = __shfl_sync(0xffffffffu, a[i][pc], pg * L + mm);
+        yp[i] = __shfl_sync(0xffffffffu, a[i][pc + 1], pg * L + mm);
+      }
+      __syncwarp();
+      const float2 q0 = *reinterpret_cast<const float2 *>(&pb[0][p]);
+      const float2 q1 = *reinterpret_cast<const float2 *>(&pb[1][p]);
+      float4 v0[C / 4], v1[C / 4];
+#pragma unroll
+      for (int c = 0; c < C; c += 4) {
+        v0[c / 4] = *reinterpret_cast<const float4 *>(&pb[0][c0 + c]);
+        v1[c / 4] = *reinterpret_cast<const float4 *>(&pb[1][c0 + c]);
+      }
+      const float det = fmaf(q0.x, q1.y, -(q0.y * q1.x));
+      const float idet = rcp_nr(det);
+      if (FLAG) ok = ok && fabsf(idet) < INFINITY;
+      const float i00 = q1.y * idet, i01 = -q0.y * idet, i10 = -q1.x * idet, i11 = q0.x * idet;
+      // one row: minus its two multipliers times the pivot rows; what its columns p and p + 1 become is minus the
+      // multipliers (x, y) P^{-1}, in the owners' rows P^{-1}
+      auto update = [&](int i) {
+        float f0 = fmaf(xp[i], i00, yp[i] * i10), f1 = fmaf(xp[i], i01, yp[i] * i11);
+        float z0 = -f0, z1 = -f1;
+        if (i == p / L && mm == pl) { z0 = i00; z1 = i01; f0 = 1.f - i00; f1 = -i01; }
+        if (i == p / L && mm == pl + 1) { z0 = i10; z1 = i11; f0 = -i10; f1 = 1.f - i11; }
+        float (&x)[C] = a[i];
+#pragma unroll
+        for (int c = 0; c < C; c += 4) {
+          const float4 v = v0[c / 4], t = v1[c / 4];
+          float2 lo = __ffma2_rn(make_float2(-f0, -f0), make_float2(v.x, v.y), make_float2(x[c], x[c + 1]));
+          float2 hi = __ffma2_rn(make_float2(-f0, -f0), make_float2(v.z, v.w), make_float2(x[c + 2], x[c + 3]));
+          lo = __ffma2_rn(make_float2(-f1, -f1), make_float2(t.x, t.y), lo);
+          hi = __ffma2_rn(make_float2(-f1, -f1), make_float2(t.z, t.w), hi);
+          x[c] = lo.x; x[c + 1] = lo.y; x[c + 2] = hi.x; x[c + 3] = hi.y;
+        }
+        if (cg == pg) {
+          x[pc] = z0;
+          x[pc + 1] = z1;
+        }
+      };
+      const int next = b + 1 < NP / 2 ? (p + 2) / L : 0;     // the slot of the next pivots
+      update(next);
+      if (b + 1 < NP / 2) publish(p + 2);
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+        if (i != next) update(i);
+    }
+    if (act) {
+      const size_t zb = (sys * n_r + zone(j)) * n;
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        const int r = mm + i * L;
+        float *o = dinv + (zb + r) * n + c0;
+        if (FULL) {
+#pragma unroll
+          for (int c = 0; c < C; c += 4)
+            if (c0 + c < NP) *reinterpret_cast<float4 *>(o + c) = make_float4(a[i][c], a[i][c + 1], a[i][c + 2], a[i][c + 3]);
+        } else if (r < n) {
+#pragma unroll
+          for (int c = 0; c < C; ++c)
+            if (c0 + c < n) o[c] = a[i][c];
+        }
+        if (cg == 0) ucol[half][r] = u[i];
+        if (half == 1 && j == len - 1) {
+#pragma unroll
+          for (int c = 0; c < C; ++c) midt[r][c0 + c] = a[i][c];
+        }
+      }
+    }
+    __syncwarp();
+  }
+  cp_async_wait_all();
+  if (half == 1) {
+    if (FLAG && lane == 0) okb = ok;                       // (read after the barrier, the top half's last zone)
+    asm volatile("bar.sync 1, 64;" ::: "memory");
+  } else if (FLAG && lane == 0) {
+    bad[jsys] = !(ok && okb);
+  }
+}
+
 // Forward/back substitution with the twisted FP32 factors, two warps per system (the top-down
 // and bottom-up halves), lane r owning block row r; the halves meet at the middle zone m through
 // shared memory and a two-warp named barrier.
@@ -885,14 +1101,27 @@ static cudaError_t run_factor_rows(int nb, int n_r, int n_sys, int spr, const TI
 }
 
 template <int NP>
-static cudaError_t run_factor_row2(int n, int n_r, int n_sys, int spr, const float *diag, const float *lower,
+static cudaError_t run_factor_gj(int n, int n_r, int n_sys, int spr, const float *diag, const float *lower,
                                    const float *upper, float *dinv, const int *ray_list, int *bad, cudaStream_t s,
                                    const int *n_dev) {
-  constexpr int S = Row2<NP>::S;
-  const unsigned grid = (unsigned)((n_sys + S - 1) / S);
-  const auto kern = n == NP ? (bad ? k_factor_row2<NP, true, true> : k_factor_row2<NP, true, false>)
-                            : k_factor_row2<NP, false, true>;
-  kern<<<grid, 64, 0, s>>>(n, n_r, n_sys, spr, diag, lower, upper, dinv, ray_list, bad, n_dev);
+  // A warp per half-system up to about four half-systems on each of the 4 kSMs warp schedulers (two of small
+  // blocks, of which k_factor_row2 takes five to sixteen a warp), and for the pair systems' wide blocks at any
+  // number.  Both sides, wide / row2, 256 zones: 1216 systems of 12 groups 186 / 173 us, 608 128 / 148 us; of 16
+  // groups 1216 247 / 259 us; of 24 groups 1216 521 / 578 us; 512 zones of 20 groups: 1024 689 / 900 us, 1536 1092 /
+  // 1035 us, 4096 2330 / 2048 us; 128 zones of 40-row blocks: 1536 1661 / 2060 us.
+  if constexpr (NP <= 32) {
+    if (n_sys > (NP < 16 ? 4 : 8) * kSMs) {
+      constexpr int S = Row2<NP>::S;
+      const unsigned grid = (unsigned)((n_sys + S - 1) / S);
+      const auto kern = n == NP ? (bad ? k_factor_row2<NP, true, true> : k_factor_row2<NP, true, false>)
+                                : k_factor_row2<NP, false, true>;
+      kern<<<grid, 64, 0, s>>>(n, n_r, n_sys, spr, diag, lower, upper, dinv, ray_list, bad, n_dev);
+      return cudaGetLastError();
+    }
+  }
+  const auto kern = n == NP ? (bad ? k_factor_wide<NP, true, true> : k_factor_wide<NP, true, false>)
+                            : k_factor_wide<NP, false, true>;
+  kern<<<n_sys, 64, 0, s>>>(n, n_r, n_sys, spr, diag, lower, upper, dinv, ray_list, bad, n_dev);
   return cudaGetLastError();
 }
 
@@ -910,7 +1139,7 @@ cudaError_t launch_factor_rows(int nb, int n_r, int n_sys, int spr, const void *
     const float *d = (const float *)diag, *l = (const float *)lower, *u = (const float *)upper;
     float *out = (float *)dinv;
     MGFLD_DISPATCH_NPW(nb, {
-      const cudaError_t e = run_factor_row2<NP>(nb, n_r, n_sys, spr, d, l, u, out, ray_list, bad, s, n_dev);
+      const cudaError_t e = run_factor_gj<NP>(nb, n_r, n_sys, spr, d, l, u, out, ray_list, bad, s, n_dev);
       if (e != cudaSuccess) return e;
       return (run_factor_rows<NP, float, float>(nb, n_r, n_sys, spr, d, l, u, out, ray_list, bad, s, n_dev));
     })
@@ -926,12 +1155,12 @@ cudaError_t launch_factor_f32(int n, int n_r, int n_sys, const float *diag, cons
                               const int *n_dev) {
   if (n_sys == 0) return cudaSuccess;
   if (n % 4 == 0) {
-    MGFLD_DISPATCH_NP(n, return (run_factor_row2<NP>(n, n_r, n_sys, NS, diag, lower32, upper32, dinv, ray_list, nullptr,
+    MGFLD_DISPATCH_NP(n, return (run_factor_gj<NP>(n, n_r, n_sys, NS, diag, lower32, upper32, dinv, ray_list, nullptr,
                                                      s, n_dev)))
   }
   // padded blocks; a system whose pivots failed again with partial pivoting
   MGFLD_DISPATCH_NP(n, {
-    const cudaError_t e = run_factor_row2<NP>(n, n_r, n_sys, NS, diag, lower32, upper32, dinv, ray_list, bad, s, n_dev);
+    const cudaError_t e = run_factor_gj<NP>(n, n_r, n_sys, NS, diag, lower32, upper32, dinv, ray_list, bad, s, n_dev);
     if (e != cudaSuccess) return e;
     constexpr int NW = (NP + 7) / 8 * 8;
     return (run_factor_rows<NW, float, float>(n, n_r, n_sys, NS, diag, lower32, upper32, dinv, ray_list, bad, s, n_dev));
