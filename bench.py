@@ -206,13 +206,16 @@ class ClockSampler:
 # ------------------------------------------------------------------------- traffic record
 
 def traffic_record(kernel):
-    """DRAM bytes per launch of `kernel` from the committed ncu summary, or None when the
-    kernel source changed since the counters were taken."""
+    """DRAM bytes per pass of `kernel` (its key in the committed ncu summary), or None when the
+    kernel sources changed since the counters were taken."""
     path = os.path.join(ROOT, 'profiles', 'ncu_traffic.txt')
     if not os.path.exists(path):
         return None
-    src = open(os.path.join(ROOT, 'paper_1809_05608_gb300', 'csrc', 'blocktri.cu'), 'rb').read()
-    src += open(os.path.join(ROOT, 'paper_1809_05608_gb300', 'csrc', 'assemble.cu'), 'rb').read()
+    src = b''
+    for name in ('blocktri.cu', 'assemble.cu', 'solve.cu', 'factor64.cu'):
+        source = os.path.join(ROOT, 'paper_1809_05608_gb300', 'csrc', name)
+        if os.path.exists(source):
+            src += open(source, 'rb').read()
     digest = hashlib.sha256(src).hexdigest()[:16]
     for line in open(path):
         parts = line.split()
@@ -364,8 +367,8 @@ def roofline_for(res, inp, precision):
     per_clk = FP32_FLOP_PER_CLK_SM if fp32 else FP64_FLOP_PER_CLK_SM
     peak = per_clk * N_SM * SM_HZ / 1e12
     launches = max(prof[dom]['launches'], 1)
-    kname = {'factor': 'k_factor_row2' if fp32 else 'k_factor', 'assemble': 'k_assemble'}[dom]
-    tr = traffic_record(kname)
+    kname = {'factor': 'k_factor_row2' if fp32 else 'k_factor64', 'assemble': 'k_assemble'}[dom]
+    tr = traffic_record('k_factor' if kname == 'k_factor64' else kname)
     traffic = None
     if tr is not None:
         units_per_launch = (res['nfact'] if dom == 'factor' else res['iters']) * inp['psi0'].shape[1] / launches
@@ -396,7 +399,7 @@ def factor_roofline(res, inp):
 
 
 def solve_roofline(res, inp):
-    """HBM roofline of the mixed path's FP32 substitution (k_sysmax + k_solve_tma per solve).
+    """HBM roofline of the mixed path's FP32 substitution (k_sysmax + k_solve_ring per solve).
 
     Bytes per (zone, system) and solve: every FP32 inverse block read by the inward and by the
     outward sweep (2 N^2 x 4 B; the blocks of the workload do not stay in the 129 MB L2 between
@@ -413,7 +416,7 @@ def solve_roofline(res, inp):
     traffic = None
     if tr is not None and solves:
         traffic = tr['bytes'] / tr['units'] * (res['iters'] * n_s / solves)
-    return dict(bound='hbm', kernel='k_solve_tma', achieved=achieved, peak=PEAK_HBM_GBS, unit='GB/s',
+    return dict(bound='hbm', kernel='k_solve_ring', achieved=achieved, peak=PEAK_HBM_GBS, unit='GB/s',
                 frac=achieved / PEAK_HBM_GBS, traffic=traffic, peak_source=HBM_SOURCE,
                 bytes_per_zone_system=per_unit, kernel_ms_per_launch=prof['ms'] / max(solves, 1),
                 kernel_share=prof['ms'] / res['ms'])

@@ -33,8 +33,8 @@ __device__ inline long system_of(long j, const int *ray_list) {
   return ray_list ? (long)ray_list[j / NS] * NS + (j % NS) : j;
 }
 
-// FP64 substitution with factors that a caller of the C ABI holds off the 16-byte boundaries that the
-// ring-fed one (solve.cu) needs; the same operations in the same order (one thread per block row, the
+// FP64 substitution for many systems, and with factors that a caller of the C ABI holds off the 16-byte
+// boundaries that the ring-fed one (solve.cu) needs; the same operations in the same order (one thread per block row, the
 // two halves of each system in the same CTA, stepping together): forward g_i = Dinv_i (r_i -
 // l_i g_{i-1}) for i < m and h_i = Dinv_i (r_i - u_i h_{i+1}) for i > m, the middle
 // x_m = Dinv_m (r_m - l_m g_{m-1} - u_m h_{m+1}), then back outward from m.  The forward results
@@ -130,7 +130,7 @@ k_solve(int n, int n_r, int n_sys, const double *__restrict__ dinv, const double
 // Thread-per-row elimination of systems of any block width up to 64 rows
 // (the coupled nu / antinu blocks of the pair process: 2 n_e rows), in FP64 or FP32, with
 // `spr` systems per ray (the launch's j-th system is system j % spr of ray ray_list[j / spr]).
-// Same algorithm and thread mapping as k_factor above: partial pivoting through integer
+// Partial pivoting through integer
 // keys (6 row bits for blocks wider than 32), the next zone's rows fetched one zone ahead, the
 // pivot row read from shared memory where it is used; shared memory sized at launch.
 template <int NP, typename T>
@@ -1167,6 +1167,13 @@ cudaError_t launch_factor_f32(int n, int n_r, int n_sys, const float *diag, cons
   })
 }
 
+// FP64 substitution, up to how many systems the ring-fed one (a warp per half-system, n of its 32 lanes at work: bound
+// by latency while the FP64 units wait) is the faster one; beyond, the thread per row of k_solve keeps every lane at
+// work.  Ring / k_solve over 256 zones: 20 groups 256 systems 261 / 843 us, 1216 852 / 949, 1280 911 / 1052, 2048 1413 /
+// 1221 us; 12 groups 1280 637 / 639; 8 groups 1280 446 / 468, 2048 649 / 491; blocks of 16 and of up to 4 rows
+// (bank conflicts; few lanes) 1280 998 / 757 and 282 / 177 us.
+static inline int ring64_systems(int n) { return (n <= 4 || (n > 12 && n <= 16) ? 5 : 8) * kSMs; }
+
 cudaError_t launch_solve(int n, int n_r, int n_sys, const void *dinv, const double *lower,
                          const double *upper, const double *rhs, double *x, int precision,
                          const int *ray_list, cudaStream_t s, const int *n_dev) {
@@ -1176,10 +1183,10 @@ cudaError_t launch_solve(int n, int n_r, int n_sys, const void *dinv, const doub
     MGFLD_DISPATCH_NP(n, k_solve_w32<NP><<<grid, kWarpsPerCta * 32, 0, s>>>(n, n_r, n_sys, (const float *)dinv,
                                                                           lower, upper, rhs, x, ray_list, n_dev);
                          return cudaGetLastError())
-  } else if (((uintptr_t)dinv & 15u) == 0) {
+  } else if (n_sys <= ring64_systems(n) && ((uintptr_t)dinv & 15u) == 0) {
     return launch_solve_ring64(n, n_r, n_sys, NS, (const double *)dinv, lower, upper, rhs, x, ray_list, nullptr, s, n_dev);
   } else {
-    // a caller's factors off the 16-byte boundaries that bulk copies start on
+    // more systems, or a caller's factors off the 16-byte boundaries that bulk copies start on
     MGFLD_DISPATCH_NP(n, return (run_solve<NP>(n, n_r, n_sys, dinv, lower, upper, rhs, x, ray_list, s, n_dev)))
   }
 }
