@@ -13,7 +13,7 @@
 // which bounds these latency-limited kernels, is half as long, and there are twice as many
 // independent instruction streams; the arithmetic is unchanged.
 //
-// The FP64 elimination is in factor64.cu, the substitution with these factors in solve.cu.
+// The FP64 elimination of fewer systems is in factor64.cu, the ring-fed substitution in solve.cu.
 #include "async.cuh"
 #include "mgfld_internal.cuh"
 
@@ -31,6 +31,139 @@ struct Pack {
 // Map the j-th system of the launch to a global (ray, species) system index.
 __device__ inline long system_of(long j, const int *ray_list) {
   return ray_list ? (long)ray_list[j / NS] * NS + (j % NS) : j;
+}
+
+// Pivot-search key of a row: the value's exponent and leading mantissa bits, then the row; an integer
+// max over the keys finds the largest |x| to 15 mantissa bits, ties going to the lowest
+// row, and the winner's row is 31 - (key & 31).  Rows already used as pivots carry -1.
+__device__ inline int pivot_key(double x, int r) {
+  const unsigned hi = (unsigned)((unsigned long long)__double_as_longlong(x) >> 32) & 0x7fffffffu;
+  return (int)((hi & ~31u) | (unsigned)(31 - r));
+}
+
+template <int NP>
+__device__ inline int max_key(const int *__restrict__ c) {
+  static_assert(NP % 4 == 0, "padded block sizes are multiples of 4");
+  int m[NP / 4];
+#pragma unroll
+  for (int j = 0; j < NP / 4; ++j) {
+    const int4 v = reinterpret_cast<const int4 *>(c)[j];
+    m[j] = max(max(v.x, v.y), max(v.z, v.w));
+  }
+#pragma unroll
+  for (int w = 1; w < NP / 4; w *= 2)
+#pragma unroll
+    for (int j = 0; j + w < NP / 4; j += 2 * w) m[j] = max(m[j], m[j + w]);
+  return m[0];
+}
+
+// FP64 elimination of many systems: one thread per block row, SPC half-systems per CTA, every lane at work where
+// k_factor64 leaves some of each warp idle; the same operations on every entry, the same inverses.  Per pivot
+// step: barrier; every row reads the NP candidate keys of its system (NP/4 vector loads, a
+// depth-log2 max tree); the pivot row publishes itself; barrier; every row forms its multiplier
+// with one FMA and updates its NP entries.  The entry of the next pivot column is updated
+// first and its key published at once, so that the next search only waits for that one FMA
+// while the other NP - 1 drain through the FP64 pipe, which bounds it.
+template <int NP>
+__global__ void __launch_bounds__(Pack<NP>::THREADS, NP <= 20 ? 4 : 1)
+k_factor(int n, int n_r, int n_sys, const double *__restrict__ diag, const double *__restrict__ lower,
+         const double *__restrict__ upper, double *__restrict__ dinv, const int *__restrict__ ray_list,
+         const int *__restrict__ n_dev) {
+  constexpr int SPC = Pack<NP>::SPC;
+  __shared__ double tile[SPC][NP][NP + 1];           // natural-order inverse of the previous zone
+  __shared__ __align__(16) double prow[SPC][NP];     // pivot row of the current step
+  __shared__ __align__(16) int cand[SPC][NP];        // pivot-search keys
+  __shared__ double ushr[SPC][NP];                   // coupling to the next zone: the column scaling of its Schur term
+  __shared__ int pivrow[SPC][NP];                    // row chosen at each step
+  __shared__ double pinv[SPC];                       // 1 / pivot of the current step
+
+  const int s = threadIdx.x / NP, r = threadIdx.x % NP;
+  const int half = s & 1;                            // 0: zones 0..m top-down, 1: zones n_r-1..m+1 bottom-up
+  const int n_sys_e = listed_sys(n_sys, n_dev, NS);
+  if ((long)blockIdx.x * (SPC / 2) >= n_sys_e) return;   // the whole CTA
+  const long jsys = (long)blockIdx.x * (SPC / 2) + (s >> 1);
+  const bool valid = jsys < n_sys_e;
+  const long sys = valid ? system_of(jsys, ray_list) : 0;
+  const int m = n_r / 2;
+  const int len = half == 0 ? m + 1 : n_r - 1 - m;   // zones of this half; all threads step m + 1 times
+
+  // Each zone's rows are loaded when the zone starts: an FP64 zone step holds the pipe for far
+  // longer than a memory round trip, and the registers of a prefetch would cost resident CTAs.
+  for (int j = 0; j <= m; ++j) {
+    const bool active = j < len;                     // inactive (bottom half, j >= len): dummy identity
+    const int i = half == 0 ? j : n_r - 1 - j;
+    const bool real = valid && active && r < n;
+    const size_t zrow = ((size_t)sys * n_r + (real ? i : 0)) * n + r;   // (sys, i, r)
+    double a[NP];
+#pragma unroll
+    for (int c = 0; c < NP; ++c) a[c] = (real && c < n) ? diag[zrow * n + c] : ((c == r) ? 1.0 : 0.0);
+    const double lr = (real && j > 0) ? (half == 0 ? lower[zrow] : upper[zrow]) : 0.0;
+    if (j > 0 && active) {
+#pragma unroll
+      for (int c = 0; c < NP; ++c) a[c] = fma(-(lr * tile[s][r][c]), ushr[s][c], a[c]);
+    }
+    if (half == 0 && j == m && n_r - 1 > m) {
+      // Middle zone: also subtract the bottom-up half's term diag(u_m) D''^{-1}_{m+1} diag(l_{m+1})
+      // (that half finished at step len - 1 < m; its tile and coupling are kept).
+      const double um = real ? upper[zrow] : 0.0;
+#pragma unroll
+      for (int c = 0; c < NP; ++c) a[c] = fma(-(um * tile[s + 1][r][c]), ushr[s + 1][c], a[c]);
+    }
+
+    // Gauss-Jordan inversion in place with partial pivoting (implicit row exchanges).
+    bool used = false;
+    int my_step = 0;
+    cand[s][r] = pivot_key(a[0], r);
+#pragma unroll
+    for (int pstep = 0; pstep < NP; ++pstep) {
+      __syncthreads();
+      const int best = 31 - (max_key<NP>(cand[s]) & 31);
+      const bool me = (r == best);
+      if (me) {
+        // The pivot entry was updated first in the previous step, so its reciprocal is
+        // formed while the rest of this row is still in the FP64 pipe.
+        pinv[s] = recip(a[pstep]);
+#pragma unroll
+        for (int c = 0; c < NP; c += 2)
+          *reinterpret_cast<double2 *>(&prow[s][c]) = make_double2(a[c], a[c + 1]);
+        pivrow[s][pstep] = r;
+        used = true;
+        my_step = pstep;
+      }
+      __syncthreads();
+      const double inv = pinv[s];
+      // Uniform update for every row: a -= f * pivot_row, with f chosen so that the pivot row
+      // itself becomes pivot_row / pivot (f = 1 - 1/pivot): one FMA either way.  The pivot
+      // column itself is overwritten below, so its update is skipped.
+      const double f = fma(me ? -1.0 : a[pstep], inv, me ? 1.0 : 0.0);
+      if (pstep + 1 < NP) {
+        a[pstep + 1] = fma(-f, prow[s][pstep + 1], a[pstep + 1]);
+        cand[s][r] = used ? -1 : pivot_key(a[pstep + 1], r);
+      }
+      // the rest of the pivot row read from shared memory as it is used (16-byte pieces)
+#pragma unroll
+      for (int c = 0; c < NP; c += 2) {
+        const double2 v = *reinterpret_cast<const double2 *>(&prow[s][c]);
+        if (c != pstep + 1 && c != pstep) a[c] = fma(-f, v.x, a[c]);
+        if (c + 1 != pstep + 1 && c + 1 != pstep) a[c + 1] = fma(-f, v.y, a[c + 1]);
+      }
+      a[pstep] = me ? inv : -f;
+    }
+    // Row r now holds row my_step of the inverse, with column c belonging to input row pivrow[c].
+    __syncthreads();
+    if (active) {
+#pragma unroll
+      for (int c = 0; c < NP; ++c) tile[s][my_step][pivrow[s][c]] = a[c];
+      ushr[s][r] = real ? (half == 0 ? upper[zrow] : lower[zrow]) : 0.0;
+    }
+    __syncthreads();
+    if (real) {
+      double *out = dinv + zrow * n;
+#pragma unroll
+      for (int c = 0; c < NP; ++c)
+        if (c < n) out[c] = tile[s][r][c];
+    }
+  }
 }
 
 // FP64 substitution for many systems, and with factors that a caller of the C ABI holds off the 16-byte
@@ -1072,11 +1205,33 @@ static cudaError_t run_solve(int n, int n_r, int n_sys, const void *dinv, const 
   return cudaGetLastError();
 }
 
+// Which FP64 factor: k_factor64 splits a half-system's columns over the four warps of a CTA (the shorter chain);
+// k_factor keeps more lanes at work.  k_factor64 / k_factor over 64 zones, us: 4 rows 187 / 93 at 400 systems;
+// 8 rows 1200 systems 223 / 222, 2400 387 / 280; 12 rows 400 265 / 386, 1200 530 / 475, 2400 1085 / 739; 16 rows 400 393 /
+// 588, 1600 1406 / 1085; 24 rows 400 1183 / 1407, 800 2324 / 1927, 2400 5975 / 4762; 32 rows 800 3916 / 5331, 4000 17452 /
+// 19177.  At 20 rows both fill the SMs in whole CTAs (4 systems a CTA of k_factor, 3 halves of k_factor64, 2.6 times
+// the time a CTA): 1200 1874 / 1565, 1600 2191 / 2196, 2400 3193 / 2911, 4000 4871 / 5025.
+template <int NP>
+static bool many_rows64(long n_sys) {
+  auto up = [](long a, long b) { return (a + b - 1) / b; };
+  if (NP == 4) return true;
+  if (NP <= 16) return n_sys > 2 * kSMs * (32 / NP);         // beyond k_factor64's one row per lane
+  if (NP == 20) return 13 * up(n_sys, 4 * kSMs) < 5 * up(2 * n_sys, 3 * kSMs);
+  return NP < 32 && n_sys > 4 * kSMs;
+}
+
 cudaError_t launch_factor(int n, int n_r, int n_sys, const double *diag, const double *lower, const double *upper,
                           void *dinv, int precision, const int *ray_list, cudaStream_t s, const int *n_dev) {
   if (n_sys == 0) return cudaSuccess;
   if (precision != MGFLD_MIXED)
-    return launch_factor64(n, n_r, n_sys, diag, lower, upper, (double *)dinv, ray_list, s, n_dev);
+    MGFLD_DISPATCH_NP(n, {
+      if (!many_rows64<NP>(n_sys))
+        return launch_factor64(n, n_r, n_sys, diag, lower, upper, (double *)dinv, ray_list, s, n_dev);
+      constexpr int SPS = Pack<NP>::SPC / 2;
+      k_factor<NP><<<(unsigned)((n_sys + SPS - 1) / SPS), Pack<NP>::THREADS, 0, s>>>(n, n_r, n_sys, diag, lower, upper,
+                                                                                  (double *)dinv, ray_list, n_dev);
+      return cudaGetLastError();
+    })
   MGFLD_DISPATCH_NP(n, constexpr int W = fw_wpc<NP>();
                     const unsigned grid = (unsigned)((n_sys + W / 2 - 1) / (W / 2));
                     k_factor_w32<NP, double, double><<<grid, W * 32, 0, s>>>(n, n_r, n_sys, diag, lower, upper,
@@ -1176,7 +1331,7 @@ static inline int ring64_systems(int n) { return (n <= 4 || (n > 12 && n <= 16) 
 
 cudaError_t launch_solve(int n, int n_r, int n_sys, const void *dinv, const double *lower,
                          const double *upper, const double *rhs, double *x, int precision,
-                         const int *ray_list, cudaStream_t s, const int *n_dev) {
+                         const int *ray_list, cudaStream_t s, const int *n_dev, int *err) {
   if (n_sys == 0) return cudaSuccess;
   if (precision == MGFLD_MIXED) {
     const unsigned grid = (unsigned)((n_sys + kWarpsPerCta / 2 - 1) / (kWarpsPerCta / 2));
@@ -1184,7 +1339,7 @@ cudaError_t launch_solve(int n, int n_r, int n_sys, const void *dinv, const doub
                                                                           lower, upper, rhs, x, ray_list, n_dev);
                          return cudaGetLastError())
   } else if (n_sys <= ring64_systems(n) && ((uintptr_t)dinv & 15u) == 0) {
-    return launch_solve_ring64(n, n_r, n_sys, NS, (const double *)dinv, lower, upper, rhs, x, ray_list, nullptr, s, n_dev);
+    return launch_solve_ring64(n, n_r, n_sys, NS, (const double *)dinv, lower, upper, rhs, x, ray_list, err, s, n_dev);
   } else {
     // more systems, or a caller's factors off the 16-byte boundaries that bulk copies start on
     MGFLD_DISPATCH_NP(n, return (run_solve<NP>(n, n_r, n_sys, dinv, lower, upper, rhs, x, ray_list, s, n_dev)))

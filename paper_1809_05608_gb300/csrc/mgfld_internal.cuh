@@ -448,6 +448,6 @@ cudaError_t launch_factor_rows(int nb, int n_r, int n_sys, int spr, const void *
                                const int *n_dev = nullptr);
 cudaError_t launch_solve(int n, int n_r, int n_sys, const void *dinv, const double *lower,
                          const double *upper, const double *rhs, double *x, int precision,
-                         const int *ray_list, cudaStream_t s, const int *n_dev = nullptr);
+                         const int *ray_list, cudaStream_t s, const int *n_dev = nullptr, int *err = nullptr);
 
 }  // namespace mgfld

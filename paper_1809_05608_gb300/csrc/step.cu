@@ -846,8 +846,11 @@ static cudaError_t enqueue_iteration(const StepCall &c, int it, int n_act, int n
   if (tl.mixed)
     MGFLD_ENQ(launch_solve_ring(pair ? 2 * n : n, NR, n_act * (pair ? 2 : NS), pair ? 2 : NS, w.dinv, w.lower32, w.upper32,
                                 w.rhs, w.rhs32, w.x, w.g32, w.list_act, w.sscale, w.counters + 3, s, cnt_act));
+  else if (!pair)
+    MGFLD_ENQ(launch_solve(n, NR, n_act * NS, w.dinv, w.lower, w.upper, w.rhs, w.x, c.precision, w.list_act, s, cnt_act,
+                           w.counters + 3));
   else
-    MGFLD_ENQ(launch_solve_ring64(pair ? 2 * n : n, NR, n_act * (pair ? 2 : NS), pair ? 2 : NS, (const double *)w.dinv,
+    MGFLD_ENQ(launch_solve_ring64(2 * n, NR, n_act * 2, 2, (const double *)w.dinv,
                                   w.lower, w.upper, w.rhs, w.x, w.list_act, w.counters + 3, s, cnt_act));
   if (prof) prof->end(MGFLD_PROF_SOLVE, 1);
   if (prof) prof->begin(MGFLD_PROF_UPDATE);
