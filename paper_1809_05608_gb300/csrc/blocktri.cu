@@ -1259,6 +1259,7 @@ template <int NP>
 static cudaError_t run_factor_gj(int n, int n_r, int n_sys, int spr, const float *diag, const float *lower,
                                    const float *upper, float *dinv, const int *ray_list, int *bad, cudaStream_t s,
                                    const int *n_dev) {
+  if (n != NP && !bad) return cudaErrorInvalidValue;         // the padded kernels store flags
   // A warp per half-system up to about four half-systems on each of the 4 kSMs warp schedulers (two of small
   // blocks, of which k_factor_row2 takes five to sixteen a warp), and for the pair systems' wide blocks at any
   // number.  Both sides, wide / row2, 256 zones: 1216 systems of 12 groups 186 / 173 us, 608 128 / 148 us; of 16
@@ -1309,14 +1310,12 @@ cudaError_t launch_factor_f32(int n, int n_r, int n_sys, const float *diag, cons
                               const float *upper32, float *dinv, int *bad, const int *ray_list, cudaStream_t s,
                               const int *n_dev) {
   if (n_sys == 0) return cudaSuccess;
-  if (n % 4 == 0) {
-    MGFLD_DISPATCH_NP(n, return (run_factor_gj<NP>(n, n_r, n_sys, NS, diag, lower32, upper32, dinv, ray_list, nullptr,
-                                                     s, n_dev)))
-  }
-  // padded blocks; a system whose pivots failed again with partial pivoting
+  // padded blocks (28 rows among them, a multiple of 4 that is no padded size): with flags, and a system whose
+  // pivots failed again with partial pivoting
   MGFLD_DISPATCH_NP(n, {
-    const cudaError_t e = run_factor_gj<NP>(n, n_r, n_sys, NS, diag, lower32, upper32, dinv, ray_list, bad, s, n_dev);
-    if (e != cudaSuccess) return e;
+    const cudaError_t e = run_factor_gj<NP>(n, n_r, n_sys, NS, diag, lower32, upper32, dinv, ray_list,
+                                            n == NP ? nullptr : bad, s, n_dev);
+    if (e != cudaSuccess || n == NP) return e;
     constexpr int NW = (NP + 7) / 8 * 8;
     return (run_factor_rows<NW, float, float>(n, n_r, n_sys, NS, diag, lower32, upper32, dinv, ray_list, bad, s, n_dev));
   })
