@@ -11,6 +11,7 @@
 // diagonal block plus the diagonal couplings to zones i-1 and i+1 (Eq. a62ae).
 #include "async.cuh"
 #include "mgfld_internal.cuh"
+#include "warp.cuh"
 
 namespace mgfld {
 
@@ -422,13 +423,13 @@ k_resid_ff(Prob p, Ws w, const double *__restrict__ psi, float *__restrict__ dia
   }
   cp_async_commit();
   // the corrections of the block's (zone, species) groups, each scaled by its group's largest
-  // (the lanes of a warp that share a group reduce first)
+  // (the lanes of a warp that share a group reduce first; every thread of the block comes here, whichever lanes
+  // the loops above have let go ahead)
   {
     const int lane = threadIdx.x & 31, kk = (int)(threadIdx.x - grp * (unsigned)n);
-    const int lo = max(lane - kk, 0), hi = min(lane + n - 1 - kk, 31);
-    const unsigned seg = (0xffffffffu >> (31 - hi)) & (0xffffffffu << lo);
-    const unsigned mx = __reduce_max_sync(seg & __activemask(), abs_hi_word(dx));
-    if (lane == lo) atomicMax(&gmx[grp], mx);
+    const int live = min(32, (int)(bt - (threadIdx.x & ~31u)));
+    const unsigned mx = __reduce_max_sync(group_lanes(lane, kk, n, live), abs_hi_word(dx));
+    if (lane == max(lane - kk, 0)) atomicMax(&gmx[grp], mx);
   }
   __syncthreads();
   const int sgrp = scale_of_max(gmx[grp]);

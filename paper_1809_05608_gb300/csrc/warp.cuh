@@ -1,0 +1,15 @@
+// Which lanes take part in a warp operation, by arithmetic that the host can check.
+#pragma once
+
+namespace mgfld {
+
+// The lanes of a warp that hold rows of one group of n consecutive rows, `lane` holding row k of it and the warp
+// having `live` lanes: the members of a reduction over the group's part of the warp, known without asking which
+// lanes happen to be converged.
+__host__ __device__ constexpr unsigned group_lanes(int lane, int k, int n, int live) {
+  const int lo = lane - k > 0 ? lane - k : 0;
+  const int hi = lane - k + n < live ? lane - k + n - 1 : live - 1;
+  return (0xffffffffu >> (31 - hi)) & (0xffffffffu << lo);
+}
+
+}  // namespace mgfld

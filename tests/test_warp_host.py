@@ -1,0 +1,49 @@
+"""The arithmetic of the kernels' warp operations (csrc/warp.cuh), compiled for the host and checked there."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), 'paper_1809_05608_gb300', 'csrc')
+
+
+def _run(tmp_path, body):
+    nvcc = shutil.which('nvcc') or '/usr/local/cuda/bin/nvcc'
+    if not os.path.exists(nvcc):
+        pytest.skip('no nvcc')
+    src = tmp_path / 't.cu'
+    src.write_text('#include <cstdio>\n#include <cstdlib>\n#include "warp.cuh"\nusing namespace mgfld;\n'
+                   '#define CHECK(x) do { if (!(x)) { std::printf("line %d: %s\\n", __LINE__, #x); std::exit(1); } } '
+                   'while (0)\n' + body)
+    exe = tmp_path / 't'
+    r = subprocess.run([nvcc, '-std=c++17', '-gencode', 'arch=compute_103a,code=sm_103a', '-I', CSRC, str(src), '-o',
+                        str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_reduction_members(tmp_path):
+    """A reduction over a group's part of a warp: every lane of that part names all of it and nobody else, in blocks
+    of whole groups of every size, the last warp of the block in part."""
+    _run(tmp_path, '''
+int main() {
+  for (int n = 1; n <= 32; ++n)
+    for (int threads = n; threads <= 256; threads += n)
+      for (int t = 0; t < threads; ++t) {
+        const int warp = t / 32 * 32, live = threads - warp < 32 ? threads - warp : 32;
+        unsigned expect = 0;
+        for (int l = 0; l < live; ++l)
+          if ((warp + l) / n == t / n) expect |= 1u << l;
+        CHECK(group_lanes(t - warp, t % n, n, live) == expect);
+      }
+}
+''')
+
+
+def test_no_members_left_to_convergence():
+    """No kernel takes the lanes that happen to be converged for the members of an operation."""
+    for name in os.listdir(CSRC):
+        if name.endswith(('.cu', '.cuh')):
+            assert '__activemask' not in open(os.path.join(CSRC, name)).read(), name
