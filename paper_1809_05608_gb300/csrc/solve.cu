@@ -3,6 +3,7 @@
 
 #include "async.cuh"
 #include "mgfld_internal.cuh"
+#include "warp.cuh"
 
 namespace mgfld {
 
@@ -225,9 +226,11 @@ k_solve_ring(int n, int n_r, int n_sys, int spr, const T *__restrict__ dinv, con
     cp_async_commit();
   };
   auto wait = [&](int u) {                                  // ring use u has arrived
-    if (!ok || mbar_try_wait(&bar[u & (S - 1)], (unsigned)((u / S) & 1))) return;
-    const bool w = mbar_wait_bounded(&bar[u & (S - 1)], (unsigned)((u / S) & 1));
-    ok = __all_sync(full, w);
+    if (!ok) return;
+    unsigned long long *b = &bar[u & (S - 1)];
+    const unsigned parity = (unsigned)((u / S) & 1);
+    ok = warp_wait([&]() { return mbar_try_wait(b, parity); }, [&]() { return mbar_wait_bounded(b, parity); },
+                   [&](bool v) { return __all_sync(full, v) != 0; });
     if (!ok) {                                              // give up: flag and drain own copies
       if (r == 0) {
         if (err) atomicExch(err, 1);

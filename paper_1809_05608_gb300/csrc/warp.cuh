@@ -12,4 +12,13 @@ __host__ __device__ constexpr unsigned group_lanes(int lane, int k, int n, int l
   return (0xffffffffu >> (31 - hi)) & (0xffffffffu << lo);
 }
 
+// A wait that a whole warp goes through together: one look, then the bounded wait.  The copy may complete between
+// the looks of two lanes, so nothing but the votes tells a lane whether the others have seen it, and every lane takes
+// part in as many of them.
+template <class Look, class Bounded, class All>
+__host__ __device__ inline bool warp_wait(Look look, Bounded bounded, All all) {
+  if (all(look())) return true;
+  return all(bounded());
+}
+
 }  // namespace mgfld

@@ -47,3 +47,25 @@ def test_no_members_left_to_convergence():
     for name in os.listdir(CSRC):
         if name.endswith(('.cu', '.cuh')):
             assert '__activemask' not in open(os.path.join(CSRC, name)).read(), name
+
+
+def test_wait_keeps_the_warp_together(tmp_path):
+    """The wait of a warp whose lanes see the copy complete at different looks: every lane takes part in the same
+    votes and comes out with the same answer."""
+    _run(tmp_path, '''
+int main() {
+  // what each of 4 lanes sees at the first look and after the bounded wait
+  for (int first = 0; first < 16; ++first)
+    for (int last = 0; last < 16; ++last) {
+      const bool vote[2] = {first == 15, last == 15};
+      int votes0 = -1;
+      for (int l = 0; l < 4; ++l) {
+        int votes = 0;
+        const bool got = warp_wait([&]() { return (first >> l & 1) != 0; }, [&]() { return (last >> l & 1) != 0; },
+                                   [&](bool) { CHECK(votes < 2); return vote[votes++]; });
+        if (l == 0) votes0 = votes;
+        CHECK(votes == votes0 && got == (vote[0] || vote[1]));
+      }
+    }
+}
+''')
