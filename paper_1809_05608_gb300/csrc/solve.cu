@@ -234,7 +234,7 @@ k_solve_ring(int n, int n_r, int n_sys, int spr, const T *__restrict__ dinv, con
     if (!ok) {                                              // give up: flag and drain own copies
       if (r == 0) {
         if (err) atomicExch(err, 1);
-        for (int v = u + 1; v < min(u == 0 ? S : u + S - 1, NU); ++v)   // the uses issued
+        for (int v = u; v <= ring_last_issued(u, S, NU); ++v)   // (the one waited for among them)
           mbar_wait_bounded(&bar[v & (S - 1)], (unsigned)((v / S) & 1));
       }
       __syncwarp();

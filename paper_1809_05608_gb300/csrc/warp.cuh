@@ -21,4 +21,11 @@ __host__ __device__ inline bool warp_wait(Look look, Bounded bounded, All all) {
   return all(bounded());
 }
 
+// The last ring use whose copy has been issued when a warp waits for use u of NU, in a ring of S: the first S go out up
+// front, use u - 1's steps issue one more once they hold the last rows of use u - 2.
+__host__ __device__ constexpr int ring_last_issued(int u, int S, int NU) {
+  const int v = u == 0 ? S - 1 : u + S - 2;
+  return v < NU ? v : NU - 1;
+}
+
 }  // namespace mgfld

@@ -69,3 +69,39 @@ int main() {
     }
 }
 ''')
+
+
+def test_copies_in_flight_when_a_wait_gives_up(tmp_path):
+    """The ring uses a warp has to drain when the wait for use u gives up: the one waited for up to the last one issued,
+    in the order in which the substitution issues and waits (the top-down half with its middle zone, the
+    bottom-up half without)."""
+    _run(tmp_path, '''
+int main() {
+  for (int S = 2; S <= 4; S *= 2)
+    for (int NG = 0; NG <= 9; ++NG)
+      for (int mid = 0; mid < 2; ++mid) {
+        const int NU = 2 * NG + mid;
+        int last = -1;
+        auto issue = [&](int u) { if (u < NU) { CHECK(u == last + 1); last = u; } };
+        auto wait = [&](int u) { CHECK(ring_last_issued(u, S, NU) == last && last >= u); };
+        for (int u = 0; u < S; ++u) issue(u);
+        if (NG > 0) wait(0);
+        for (int v = 0; v < NG; ++v) {                       // inward
+          if (v > 0) issue(v - 1 + S);
+          if (v + 1 < NG) wait(v + 1);
+        }
+        int u = NG;
+        if (mid) {
+          wait(u);
+          if (u > 0) issue(u - 1 + S);
+          ++u;
+        }
+        if (NG > 0) wait(u);
+        for (int w = 0; w < NG; ++w, ++u) {                  // outward
+          if (u > 0) issue(u - 1 + S);
+          if (w + 1 < NG) wait(u + 1);
+        }
+        CHECK(last == NU - 1 || NU == 0);
+      }
+}
+''')
