@@ -433,8 +433,9 @@ cudaError_t launch_factor_f32(int n, int n_r, int n_sys, const float *diag, cons
 // and the residual / Jacobian of the coupled pair systems (blocks of 2 n rows, vectors
 // [ray][pair][zone][2 n]; src_out in the psi layout).
 cudaError_t launch_pair(const Prob &p, const Ws &w, const double *T, cudaStream_t s);
-// (the mixed path's final sources, from the kept sums of the last residual)
-cudaError_t launch_src_pair(const Prob &p, const Ws &w, const double *psi, double *src, cudaStream_t s);
+// (the mixed path's final sources, from the kept sums of the last residual where its correction is small: a ray
+// that converged to tol <= 2^-30)
+cudaError_t launch_src_pair(const Prob &p, const Ws &w, const double *psi, double *src, double tol, cudaStream_t s);
 cudaError_t launch_assemble_pair(const Prob &p, const Ws &w, const double *psi, void *diag, int diag_fp32,
                                  double *lower, double *upper, double *rhs, const int *list, int n_list,
                                  const int *jac_flag, cudaStream_t s, double *src_out, int first,

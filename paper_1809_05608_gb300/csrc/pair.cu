@@ -237,10 +237,13 @@ __global__ void k_assemble_pair(Prob p, Ws w, const double *__restrict__ psi, TD
 
 // The converged sources of the mixed path, as k_src_mixed forms them: the sums of the ray's last residual
 // plus the kernels times the last, sub-tolerance correction in FP32 (the kernels' leading 24 bits), a
-// thread per (zone, species, group), the block's corrections staged as FP32.
+// thread per (zone, species, group), the block's corrections staged as FP32.  The FP32 sums lose 2^-23 of that
+// correction, which stays below the rounding of the FP64 sums only where the correction is small: for a ray that did
+// not converge, or with `full` (a tolerance above 2^-30), the FP64 sums are formed again at psi, as k_assemble_pair
+// forms them.
 constexpr int kSrcPairThreads = 256;
 __global__ void __launch_bounds__(kSrcPairThreads)
-k_src_pair(Prob p, Ws w, const double *__restrict__ psi, double *__restrict__ src) {
+k_src_pair(Prob p, Ws w, const double *__restrict__ psi, double *__restrict__ src, bool full) {
   extern __shared__ float xs[];                              // the block's zones, [zone][species][group]
   const int n = p.n, n2 = 2 * n;
   const unsigned zrows = (unsigned)(NS * n), zpb = blockDim.x / zrows;
@@ -256,6 +259,23 @@ k_src_pair(Prob p, Ws w, const double *__restrict__ psi, double *__restrict__ sr
   const size_t g = (((size_t)ray * NS + q) * p.n_r + i) * n + k, zr = ((size_t)zi * n + k) * n;
   const float *fi = w.phin32 + zr, *fd = w.phd32 + zr;
   const double *mk = w.pmake + zr, *kl = w.pkill + (((size_t)zi * NS + q) * n + k) * n;
+  const double pk = psi[g], q1 = 1.0 - pk;
+  const double kap = scaled(p, p.kabs, g, q, k);
+  if (full || w.status[ray] != MGFLD_OK) {                   // (uniform over a zone)
+    const double *ps = psi + (g - k), *pb = psi + (((size_t)ray * NS + (q ^ 1)) * p.n_r + i) * n;
+    const double *fin = w.phin + zr, *fout = w.phout + zr;
+    double gain = 0.0, lp = 0.0, mb = 0.0, kb = 0.0;
+    for (int kp = 0; kp < n; ++kp) {
+      const double pv = ps[kp], v = pb[kp];
+      gain += fin[kp] * pv;
+      lp += fout[kp] * pv;
+      mb = fma(mk[kp], v, mb);
+      kb = fma(kl[kp], v, kb);
+    }
+    const double make = w.pmsum[(size_t)zi * n + k] - mb, loss = w.rsum[(size_t)zi * n + k] - lp, j = w.jbuf[g];
+    src[g] = j * q1 - kap * pk + (q1 * gain - pk * loss) + (q1 * make - pk * kb);
+    return;
+  }
   const float *dx = xs + zs * zrows + (size_t)q * n, *dy = xs + zs * zrows + (size_t)(q ^ 1) * n;
   float dg = 0.f, dl = 0.f, dm = 0.f, dk = 0.f;
   for (int kp = 0; kp < n; ++kp) {
@@ -265,11 +285,9 @@ k_src_pair(Prob p, Ws w, const double *__restrict__ psi, double *__restrict__ sr
     dm = fmaf(d2f_exp2(mk[kp], 0), y, dm);
     dk = fmaf(d2f_exp2(kl[kp], 0), y, dk);
   }
-  const double pk = psi[g], q1 = 1.0 - pk;
   const float pf = d2f_exp2(pk, 0);
   // (1 - psi) (dgain - dmake) + psi (dlp - dkill): the FP32 part of the sources
   const float corr = fmaf(1.f - pf, dg - dm, pf * (dl - dk));
-  const double kap = scaled(p, p.kabs, g, q, k);
   const double up = w.g0[g] + (w.pmsum[(size_t)zi * n + k] - w.kinv[g]);
   const double down = (w.rsum[(size_t)zi * n + k] - w.l0[g]) + w.lam[g];
   double S = fma(q1, up, fma(-pk, down, (double)corr));
@@ -277,9 +295,10 @@ k_src_pair(Prob p, Ws w, const double *__restrict__ psi, double *__restrict__ sr
   src[g] = S;
 }
 
-cudaError_t launch_src_pair(const Prob &p, const Ws &w, const double *psi, double *src, cudaStream_t s) {
+cudaError_t launch_src_pair(const Prob &p, const Ws &w, const double *psi, double *src, double tol, cudaStream_t s) {
   const unsigned zrows = (unsigned)(NS * p.n), zpb = kSrcPairThreads / zrows, zones = (unsigned)(p.n_ray * p.n_r);
-  k_src_pair<<<(zones + zpb - 1) / zpb, zpb * zrows, sizeof(float) * zpb * zrows, s>>>(p, w, psi, src);
+  k_src_pair<<<(zones + zpb - 1) / zpb, zpb * zrows, sizeof(float) * zpb * zrows, s>>>(p, w, psi, src,
+                                                                                       tol > 0x1p-30);
   return cudaGetLastError();
 }
 

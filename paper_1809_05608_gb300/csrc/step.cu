@@ -878,7 +878,7 @@ static cudaError_t enqueue_finish(const StepCall &c, Prof *prof, cudaStream_t s)
   cudaError_t e = cudaSuccess;
   if (prof) prof->begin(MGFLD_PROF_FINISH);
   if (c.pair && c.tl.mixed)
-    MGFLD_ENQ(launch_src_pair(c.p, w, c.st.psi, w.src, s));
+    MGFLD_ENQ(launch_src_pair(c.p, w, c.st.psi, w.src, c.tl.tol, s));
   else if (c.pair)
     MGFLD_ENQ(launch_assemble_pair(c.p, w, c.st.psi, w.diag, c.tl.mixed, w.lower, w.upper, w.rhs, nullptr, R, nullptr,
                                    s, w.src, 0));
