@@ -657,9 +657,12 @@ k_factor_w32(int n, int n_r, int n_sys, const TIn *__restrict__ diag, const TC *
 // complements of an M-matrix are nonsingular, so no exchanges are needed.  The Schur term of the next
 // zone is formed from the lane's own rows of the inverse, still in registers (row r of the inverse stays
 // with the lane of row r); the next zone's rows and couplings arrive by asynchronous copies issued one
-// zone ahead.  A zone whose 2 x 2 pivot block is singular or not finite leaves its inverse non-finite;
-// where the launch keeps flags, its system is done again with partial pivoting (without them the outer
-// iteration reports ENAN for the ray).
+// zone ahead.  A zone whose 2 x 2 pivot block is singular or not finite leaves its inverse non-finite, and the
+// outer iteration reports ENAN for the ray.  Where the launch keeps flags (padded and pair blocks), a system is done again
+// with partial pivoting unless its pivot blocks are those of an M-matrix: determinant and diagonal entries positive, no
+// entry above kGrowth times the raw one (elimination only takes from an M-matrix's diagonal).  An iterate with
+// occupations outside [0, 1] makes blocks that are none, and an unnoticed small pivot there factors without a correct
+// digit.  (The check: 3.76 -> 3.78 ms a step at 173 rays of 301 x 13, 25.4 -> 25.5 ms with pairs at 256 of 512 x 20.)
 // Bound by the issue slots of the row updates; measured at 1024 rays of 512 x 20: 2.05 ms.  (Publishing the next
 // pivots before the other row is updated, as k_factor_wide does, spills here: 2.50 ms.)
 template <int NP>
@@ -670,13 +673,15 @@ struct Row2 {
                                                            // 16-byte pieces (conflict-free reads)
 };
 
+constexpr float kGrowth = 4.f;
+
 // CTAs per SM the two-rows-per-lane factor is compiled for (its register budget).
 template <int NP>
 __host__ __device__ constexpr int row2_minb() { return NP <= 20 ? 9 : 6; }
 
 // FULL: n = NP, rows in 16-byte pieces; otherwise rows and columns beyond n are padded with the
-// identity.  spr: systems per ray.  FLAG: bad[listed system] is set to whether a pivot block was
-// singular or not finite.
+// identity.  spr: systems per ray.  FLAG: bad[listed system] is set to whether a pivot block was not an
+// M-matrix's.
 template <int NP, bool FULL, bool FLAG>
 __global__ void __launch_bounds__(64, row2_minb<NP>())
 k_factor_row2(int n_, int n_r, int n_sys, int spr, const float *__restrict__ diag, const float *__restrict__ lower,
@@ -762,6 +767,7 @@ k_factor_row2(int n_, int n_r, int n_sys, int spr, const float *__restrict__ dia
     // -l_r (row r of the previous inverse, this lane's registers) * u_prev (column scaling)
     // (lanes without a system run on whatever their slot holds: they store nothing, and a slot
     // without a system is read by its own lanes only)
+    const float top0 = kGrowth * rows[wid][gs][r0][r0], top1 = kGrowth * rows[wid][gs][r1][r1];   // (FLAG)
     const float l0 = cpl[wid][gs][0][r0], l1 = cpl[wid][gs][0][r1];   // used from the second zone on
     const float u0 = cpl[wid][gs][1][r0], u1 = cpl[wid][gs][1][r1];
 #pragma unroll
@@ -816,7 +822,11 @@ k_factor_row2(int n_, int n_r, int n_sys, int spr, const float *__restrict__ dia
       const float2 q1 = *reinterpret_cast<const float2 *>(&pb[gs][1][p]);
       const float det = fmaf(q0.x, q1.y, -(q0.y * q1.x));
       const float idet = rcp_nr(det);
-      if (FLAG) ok = ok && fabsf(idet) < INFINITY;
+      if (FLAG) {
+        ok = ok && idet > 0.f && idet < INFINITY;
+        const float d = mm == pl ? q0.x : q1.y;               // (NaN fails)
+        if (mm == pl || mm == pl + 1) ok = ok && d > 0.f && d <= (sl == 0 ? top0 : top1);
+      }
       const float i00 = q1.y * idet, i01 = -q0.y * idet, i10 = -q1.x * idet, i11 = q0.x * idet;
       // multipliers of the two rows: owners take the rows of P^{-1} times the pivot rows
       float f00, f01, f10, f11;
@@ -882,6 +892,11 @@ k_factor_row2(int n_, int n_r, int n_sys, int spr, const float *__restrict__ dia
     __syncwarp();
   }
   cp_async_wait_all();
+  if (FLAG) {
+    // every lane of the half-system
+    constexpr unsigned lanes = 0xffffffffu >> (32 - L);
+    ok = ((__ballot_sync(0xffffffffu, ok) >> (gs * L)) & lanes) == lanes;
+  }
   if (half == 1) {
     if (FLAG && g < S && mm == 0) okb[gs] = ok;            // (read after the barrier, the top half's last zone)
     asm volatile("bar.sync 1, 64;" ::: "memory");
@@ -984,9 +999,10 @@ k_factor_wide(int n_, int n_r, int n_sys, int spr, const float *__restrict__ dia
     cp_async_wait_all();
     __syncwarp();
     // the zone's rows minus the Schur term of the previous zone
-    float u[R];
+    float u[R], top[R];                                    // (top: FLAG)
 #pragma unroll
     for (int i = 0; i < R; ++i) {
+      top[i] = kGrowth * rows[half][mm + i * L][mm + i * L];
       const float l = cpl[half][0][mm + i * L];
       u[i] = cpl[half][1][mm + i * L];
 #pragma unroll
@@ -1048,7 +1064,11 @@ k_factor_wide(int n_, int n_r, int n_sys, int spr, const float *__restrict__ dia
       }
       const float det = fmaf(q0.x, q1.y, -(q0.y * q1.x));
       const float idet = rcp_nr(det);
-      if (FLAG) ok = ok && fabsf(idet) < INFINITY;
+      if (FLAG) {
+        ok = ok && idet > 0.f && idet < INFINITY;
+        const float d = mm == pl ? q0.x : q1.y;               // (NaN fails)
+        if (mm == pl || mm == pl + 1) ok = ok && d > 0.f && d <= top[p / L];
+      }
       const float i00 = q1.y * idet, i01 = -q0.y * idet, i10 = -q1.x * idet, i11 = q0.x * idet;
       // one row: minus its two multipliers times the pivot rows; what its columns p and p + 1 become is minus the
       // multipliers (x, y) P^{-1}, in the owners' rows P^{-1}
@@ -1104,6 +1124,7 @@ k_factor_wide(int n_, int n_r, int n_sys, int spr, const float *__restrict__ dia
     __syncwarp();
   }
   cp_async_wait_all();
+  if (FLAG) ok = __all_sync(0xffffffffu, ok) != 0;
   if (half == 1) {
     if (FLAG && lane == 0) okb = ok;                       // (read after the barrier, the top half's last zone)
     asm volatile("bar.sync 1, 64;" ::: "memory");
@@ -1284,8 +1305,8 @@ static cudaError_t run_factor_gj(int n, int n_r, int n_sys, int spr, const float
 // FP32 (bad: n_sys flags of scratch): the blocks of the outer iteration are, up to the sign of the
 // antineutrinos' rows and columns, M-matrices (the pair process couples the partners with
 // non-negative entries, and its weighted column sums cancel against the diagonal as those of the
-// scattering do), so they are eliminated without row exchanges, two rows per lane; a system in which
-// a pivot block is singular or not finite all the same is done again with partial pivoting.
+// scattering do) while the occupations are between 0 and 1, so they are eliminated without row exchanges, two
+// rows per lane; a system whose pivot blocks are not an M-matrix's is done again with partial pivoting.
 cudaError_t launch_factor_rows(int nb, int n_r, int n_sys, int spr, const void *diag, const void *lower,
                                const void *upper, void *dinv, int fp32, int *bad, const int *ray_list, cudaStream_t s,
                                const int *n_dev) {
@@ -1311,7 +1332,7 @@ cudaError_t launch_factor_f32(int n, int n_r, int n_sys, const float *diag, cons
                               const int *n_dev) {
   if (n_sys == 0) return cudaSuccess;
   // padded blocks (28 rows among them, a multiple of 4 that is no padded size): with flags, and a system whose
-  // pivots failed again with partial pivoting
+  // pivot blocks are not an M-matrix's again with partial pivoting
   MGFLD_DISPATCH_NP(n, {
     const cudaError_t e = run_factor_gj<NP>(n, n_r, n_sys, NS, diag, lower32, upper32, dinv, ray_list,
                                             n == NP ? nullptr : bad, s, n_dev);
