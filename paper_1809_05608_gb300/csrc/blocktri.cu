@@ -33,6 +33,10 @@ __device__ inline long system_of(long j, const int *ray_list) {
   return ray_list ? (long)ray_list[j / NS] * NS + (j % NS) : j;
 }
 
+__device__ inline long system_of_spr(long j, const int *ray_list, int spr) {
+  return ray_list ? (long)ray_list[j / spr] * spr + (j % spr) : j;
+}
+
 // Pivot-search key of a row: the value's exponent and leading mantissa bits, then the row; an integer
 // max over the keys finds the largest |x| to 15 mantissa bits, ties going to the lowest
 // row, and the winner's row is 31 - (key & 31).  Rows already used as pivots carry -1.
@@ -166,15 +170,15 @@ k_factor(int n, int n_r, int n_sys, const double *__restrict__ diag, const doubl
   }
 }
 
-// FP64 substitution for many systems, and with factors that a caller of the C ABI holds off the 16-byte
-// boundaries that the ring-fed one (solve.cu) needs; the same operations in the same order (one thread per block row, the
+// FP64 substitution for many systems (spr per ray; the pair systems among them), and with factors that a caller of the C ABI
+// holds off the 16-byte boundaries that the ring-fed one (solve.cu) needs; the same operations in the same order (one thread per block row, the
 // two halves of each system in the same CTA, stepping together): forward g_i = Dinv_i (r_i -
 // l_i g_{i-1}) for i < m and h_i = Dinv_i (r_i - u_i h_{i+1}) for i > m, the middle
 // x_m = Dinv_m (r_m - l_m g_{m-1} - u_m h_{m+1}), then back outward from m.  The forward results
 // are kept in x (which may alias rhs: each zone's rhs is read before its x is written).
 template <int NP>
 __global__ void __launch_bounds__(Pack<NP>::THREADS)
-k_solve(int n, int n_r, int n_sys, const double *__restrict__ dinv, const double *__restrict__ lower,
+k_solve(int n, int n_r, int n_sys, int spr, const double *__restrict__ dinv, const double *__restrict__ lower,
         const double *__restrict__ upper, const double *rhs, double *x, const int *__restrict__ ray_list,
         const int *__restrict__ n_dev) {
   constexpr int SPC = Pack<NP>::SPC;
@@ -182,11 +186,11 @@ k_solve(int n, int n_r, int n_sys, const double *__restrict__ dinv, const double
   __shared__ double mid[SPC / 2][NP];               // h_{m+1}, then x_m
   const int s = threadIdx.x / NP, r = threadIdx.x % NP;
   const int half = s & 1, sl = s >> 1;
-  const int n_sys_e = listed_sys(n_sys, n_dev, NS);
+  const int n_sys_e = listed_sys(n_sys, n_dev, spr);
   if ((long)blockIdx.x * (SPC / 2) >= n_sys_e) return;   // the whole CTA
   const long jsys = (long)blockIdx.x * (SPC / 2) + sl;
   const bool valid = jsys < n_sys_e;
-  const long sys = valid ? system_of(jsys, ray_list) : 0;
+  const long sys = valid ? system_of_spr(jsys, ray_list, spr) : 0;
   const bool realr = valid && r < n;
   const size_t base = (size_t)sys * n_r * n;
   const int m = n_r / 2, B = n_r - 1 - m;
@@ -281,10 +285,6 @@ struct RowCta {
   static constexpr size_t PIVR = sizeof(int) * SPC * NP;         // row chosen at each step
   static constexpr size_t BYTES = TILE + PROW + USHR + PINV + CAND + PIVR;
 };
-
-__device__ inline long system_of_spr(long j, const int *ray_list, int spr) {
-  return ray_list ? (long)ray_list[j / spr] * spr + (j % spr) : j;
-}
 
 template <int KB> __device__ inline int row_key(double x, int r) {
   const unsigned hi = (unsigned)((unsigned long long)__double_as_longlong(x) >> 32) & 0x7fffffffu;
@@ -1216,12 +1216,12 @@ k_solve_w32(int n, int n_r, int n_sys, const float *__restrict__ dinv, const dou
 }
 
 template <int NP>
-static cudaError_t run_solve(int n, int n_r, int n_sys, const void *dinv, const double *lower,
+static cudaError_t run_solve(int n, int n_r, int n_sys, int spr, const void *dinv, const double *lower,
                              const double *upper, const double *rhs, double *x, const int *ray_list,
                              cudaStream_t s, const int *n_dev) {
   constexpr int SPS = Pack<NP>::SPC / 2;             // systems per CTA
   const unsigned grid = (unsigned)((n_sys + SPS - 1) / SPS);
-  k_solve<NP><<<grid, Pack<NP>::THREADS, 0, s>>>(n, n_r, n_sys, (const double *)dinv, lower, upper, rhs, x,
+  k_solve<NP><<<grid, Pack<NP>::THREADS, 0, s>>>(n, n_r, n_sys, spr, (const double *)dinv, lower, upper, rhs, x,
                                                  ray_list, n_dev);
   return cudaGetLastError();
 }
@@ -1362,8 +1362,32 @@ cudaError_t launch_solve(int n, int n_r, int n_sys, const void *dinv, const doub
     return launch_solve_ring64(n, n_r, n_sys, NS, (const double *)dinv, lower, upper, rhs, x, ray_list, err, s, n_dev);
   } else {
     // more systems, or a caller's factors off the 16-byte boundaries that bulk copies start on
-    MGFLD_DISPATCH_NP(n, return (run_solve<NP>(n, n_r, n_sys, dinv, lower, upper, rhs, x, ray_list, s, n_dev)))
+    MGFLD_DISPATCH_NP(n, return (run_solve<NP>(n, n_r, n_sys, NS, dinv, lower, upper, rhs, x, ray_list, s, n_dev)))
   }
+}
+
+// The pair systems' FP64 substitution (nb = 2 n_e rows, two systems per ray; as above the ring-fed one is bound by
+// latency, and its rings leave room for few CTAs an SM: three of 32 rows, two of 40, one of 48): the ring up to the
+// launches that its CTAs hold at once, the thread per row beyond.  Ring / thread per row over 64 zones, us: 4 rows 608
+// systems 52 / 55, 720 61 / 55; 8 rows 608 53 / 61, 800 75 / 65; 12 rows 608 88 / 99, 800 125 / 111; 16 rows 912 133 / 165,
+// 1216 252 / 187; 18 rows 456 184 / 193, 608 231 / 204; 24 rows 456 192 / 229, 608 239 / 234; 26 rows 128 193 / 170,
+// 304 197 / 226, 456 236 / 240; 32 rows 152 211 / 203, 304 239 / 242, 380 296 / 280; 40 rows 304 270 / 363, 340 509 / 408;
+// 48 rows 152 321 / 410, 180 635 / 459, 4096 8453 / 4231.
+static inline bool ring64_pair(int nb, int n_sys) {
+  if (nb <= 16) return n_sys <= (nb == 16 ? 6 : 4) * kSMs;
+  if (nb <= 24) return n_sys <= 3 * kSMs;
+  if (nb <= 32) return n_sys > kSMs && n_sys <= 2 * kSMs;    // (few systems: the row kernel's shorter chain)
+  return n_sys <= (nb <= 40 ? 2 : 1) * kSMs;
+}
+
+cudaError_t launch_solve_pair64(int nb, int n_r, int n_sys, const double *dinv, const double *lower, const double *upper,
+                                const double *rhs, double *x, const int *ray_list, int *err, cudaStream_t s,
+                                const int *n_dev) {
+  if (n_sys == 0) return cudaSuccess;
+  if (nb > 48) return cudaErrorInvalidValue;
+  if (ring64_pair(nb, n_sys))
+    return launch_solve_ring64(nb, n_r, n_sys, 2, dinv, lower, upper, rhs, x, ray_list, err, s, n_dev);
+  MGFLD_DISPATCH_NPW(nb, return (run_solve<NP>(nb, n_r, n_sys, 2, dinv, lower, upper, rhs, x, ray_list, s, n_dev)))
 }
 
 }  // namespace mgfld

@@ -268,6 +268,10 @@ cudaError_t launch_solve_ring(int n, int n_r, int n_sys, int spr, const void *di
 cudaError_t launch_solve_ring64(int n, int n_r, int n_sys, int spr, const double *dinv, const double *lower,
                                 const double *upper, const double *rhs, double *x, const int *ray_list, int *err,
                                 cudaStream_t s, const int *n_dev = nullptr);
+// The FP64 substitution of the pair systems (blocks of nb = 2 n <= 48 rows in the workspace, two systems per ray).
+cudaError_t launch_solve_pair64(int nb, int n_r, int n_sys, const double *dinv, const double *lower, const double *upper,
+                                const double *rhs, double *x, const int *ray_list, int *err, cudaStream_t s,
+                                const int *n_dev = nullptr);
 // Per system (spr per ray): the power of two k that brings max |rhs| into [1/2, 1), and rhs 2^k in FP32.
 cudaError_t launch_sysmax(int n, int n_r, int n_sys, const double *rhs, const int *ray_list, int spr, int *sys_exp,
                           float *rhs32, cudaStream_t s, const int *n_dev = nullptr);

@@ -850,8 +850,8 @@ static cudaError_t enqueue_iteration(const StepCall &c, int it, int n_act, int n
     MGFLD_ENQ(launch_solve(n, NR, n_act * NS, w.dinv, w.lower, w.upper, w.rhs, w.x, c.precision, w.list_act, s, cnt_act,
                            w.counters + 3));
   else
-    MGFLD_ENQ(launch_solve_ring64(2 * n, NR, n_act * 2, 2, (const double *)w.dinv,
-                                  w.lower, w.upper, w.rhs, w.x, w.list_act, w.counters + 3, s, cnt_act));
+    MGFLD_ENQ(launch_solve_pair64(2 * n, NR, n_act * 2, (const double *)w.dinv, w.lower, w.upper, w.rhs, w.x, w.list_act,
+                                  w.counters + 3, s, cnt_act));
   if (prof) prof->end(MGFLD_PROF_SOLVE, 1);
   if (prof) prof->begin(MGFLD_PROF_UPDATE);
   if (!pair && n % 2 == 0 && ((uintptr_t)c.st.psi & 15u) == 0)
