@@ -88,7 +88,9 @@ k_stress(Prob p, Ws w, const double *__restrict__ psi, double *__restrict__ f_ed
 }
 
 // One block per ray, every thread a run of consecutive zones: the enclosed rest mass (block sum), x_j of
-// the edges j + 1/2 below the last zone into scratch, and their suffix sums by runs, warps and the block.  Measured at 256 rays of 512 zones: 60 -> 23 us (a warp per ray, x_j formed twice, before).
+// the edges j + 1/2 below the last zone into scratch, and their suffix sums by runs, warps and the block.  Measured at
+// 256 rays of 512 zones: 60 -> 23 us (a warp per ray, x_j formed twice, before).  Short rays take as many warps as
+// they have zones for: 4000 rays of 64 zones 111 -> 48 us (62 with the warp per ray).
 constexpr int kLapseThreads = 256;
 __global__ void __launch_bounds__(kLapseThreads)
 k_lapse(Prob p, const double *__restrict__ pres, const double *__restrict__ m_inner,
@@ -96,13 +98,13 @@ k_lapse(Prob p, const double *__restrict__ pres, const double *__restrict__ m_in
         double *scratch, double *__restrict__ lapse) {
   __shared__ double wsum[2][kLapseThreads / 32];
   const int ray = blockIdx.x, t = threadIdx.x, lane = t & 31, wid = t >> 5;
-  const int nr = p.n_r, c = (nr + kLapseThreads - 1) / kLapseThreads;
+  const int nr = p.n_r, threads = (int)blockDim.x, warps = threads / 32, c = (nr + threads - 1) / threads;
   const double *rho = p.rho + (size_t)ray * nr, *pr = pres + (size_t)ray * nr, *fe = f_edge + (size_t)ray * nr;
   const double *re = p.r_edge + (size_t)ray * (nr + 1);
   const double *vol = vol_src + (size_t)ray * nr * vol_stride;
   double *xs = scratch + (size_t)ray * nr;
   double m = 0.0;
-  for (int i = t; i < nr; i += kLapseThreads) {
+  for (int i = t; i < nr; i += threads) {
     const double dM = rho[i] * vol[(size_t)i * vol_stride];
     m += dM;
     double x = 0.0;
@@ -118,7 +120,7 @@ k_lapse(Prob p, const double *__restrict__ pres, const double *__restrict__ m_in
   if (lane == 0) wsum[0][wid] = m;
   __syncthreads();
   m = m_inner ? m_inner[ray] : 0.0;
-  for (int j = 0; j < kLapseThreads / 32; ++j) m += wsum[0][j];
+  for (int j = 0; j < warps; ++j) m += wsum[0][j];
   const double a_out = sqrt(1.0 - 2.0 * kG * m / (kC * kC * re[nr]));
   // suffix sums: this run's, of the lanes above in the warp, of the warps above
   const int lo = min(t * c, nr), hi = min(lo + c, nr);
@@ -132,7 +134,7 @@ k_lapse(Prob p, const double *__restrict__ pres, const double *__restrict__ m_in
   if (lane == 0) wsum[1][wid] = v;
   __syncthreads();
   double run = v - acc;
-  for (int j = wid + 1; j < kLapseThreads / 32; ++j) run += wsum[1][j];
+  for (int j = wid + 1; j < warps; ++j) run += wsum[1][j];
   for (int i = hi - 1; i >= lo; --i) {
     run += xs[i];
     lapse[(size_t)ray * nr + i] = a_out * exp(run);
@@ -162,11 +164,16 @@ extern "C" mgfld_status mgfld_stress_lapse(const mgfld_dims *dims, const mgfld_p
   double *fe = io->f_edge ? io->f_edge : w.rhs;
   const int runs = (dims->n_r + kStressZones - 1) / kStressZones;
   const size_t sm = sizeof(double) * ((size_t)(2 * kStressZones + 3) * NS * dims->n_e + kStressZones + 2 + (kStressZones + 1) * (NS + 1));
-  const int row = NS * dims->n_e, threads = kStressThreads / row * row;
+  // (whole rows, no more of them than a run has zones: with few groups a block of 256 would mostly idle; the call at
+  // 4000 rays of 64 zones and one group 535 -> 490 us)
+  const int row = NS * dims->n_e, rows = kStressThreads / row;
+  const int threads = (rows < kStressZones + 2 ? rows : kStressZones + 2) * row;
   k_stress<<<dims->n_ray * runs, threads, sm, s>>>(p, w, state->psi, fe, io->f_zone);
   if (cudaGetLastError() != cudaSuccess) return MGFLD_ECUDA;
   if (io->lapse) {
-    k_lapse<<<dims->n_ray, kLapseThreads, 0, s>>>(p, io->p, io->m_inner, fe, w.zone + ZC_VOL, ZC_N, w.src, io->lapse);
+    const int lanes = (dims->n_r + 31) / 32 * 32;
+    k_lapse<<<dims->n_ray, lanes < kLapseThreads ? lanes : kLapseThreads, 0, s>>>(p, io->p, io->m_inner, fe,
+                                                                                  w.zone + ZC_VOL, ZC_N, w.src, io->lapse);
     if (cudaGetLastError() != cudaSuccess) return MGFLD_ECUDA;
   }
   return MGFLD_OK;
