@@ -3,7 +3,8 @@
 Headline workload: the 2D mixed-precision configuration, 1024 rays (2D, per-ray angular
 perturbations) x 512 radial zones x 20 energy groups x 4 species, dt = 1e-6 s, outer tolerance
 1e-10 (tolmin_psi = 1), with the seeds of that configuration.  A "step" is one implicit transport
-step of every ray (mgfld_step).  Metric: zone*group*species updates per second (n_ray * n_r *
+step of every ray (mgfld_step).  One JSON line with the result goes to standard output, the full record
+(the other paths, rooflines, kernel times) to standard error.  Metric: zone*group*species updates per second (n_ray * n_r *
 n_e * 4 per step / time) for the mixed-precision path (FP32 block factorisation, FP64 residual
 refinement), with the FP64 path at the same tolerance on the same inputs beside it.  A second
 line (`config4`) times the 3D-scale mixed configuration, 4096 rays (64 theta x 64 phi) x 540 x 20
@@ -201,6 +202,31 @@ class ClockSampler:
             return dict(sm_mhz=None, sm_max_mhz=None, reasons=['no samples inside the timed window'])
         return dict(sm_mhz=statistics.median(sm), sm_max_mhz=max(smax), reasons=sorted(reasons),
                     samples=len(sm))
+
+
+# --------------------------------------------------------------------------- result line
+
+RESULT_KEYS = ('metric', 'value', 'unit', 'n_gpus', 'steps', 'warmup', 'ms_per_step', 'higher_is_better', 'scaling',
+               'vs_baseline', 'dtype', 'data', 'config', 'e2e', 'gpu_launches', 'clocks')
+
+
+def result_line(record):
+    """The line on standard output: what identifies the run, its result and the other paths' times, short enough
+    (RESULT_LIMIT characters) to be read whole from the end of a log.  The full record, with every line's rooflines and
+    baselines, goes to standard error."""
+    line = {k: record[k] for k in RESULT_KEYS}
+    roof, cpu = record.get('roofline'), record.get('cpu_baseline')
+    if roof:
+        line['roofline'] = {k: roof[k] for k in ('kernel', 'bound', 'frac')}
+    if cpu:
+        line['cpu_baseline'] = {k: cpu[k] for k in ('value', 'cores', 'kind')}
+    line['ms_per_step_of'] = {k[:-5]: record[k]['ms_per_step'] for k in record if k.endswith('_path')}
+    if 'config4' in record:
+        line['ms_per_step_of']['config4'] = record['config4']['ms_per_step']
+    return line
+
+
+RESULT_LIMIT = 1500
 
 
 # ------------------------------------------------------------------------- traffic record
@@ -1118,7 +1144,8 @@ def main():
                                       iteration='Newton, new factors every iteration'),
         mixed_over_fp64=value / value64,
         **extra)
-    print(json.dumps(line), flush=True)
+    print(json.dumps(line), file=sys.stderr, flush=True)
+    print(json.dumps(result_line(line)), flush=True)
     if dist is not None:
         dist.destroy_process_group()
     return 0
