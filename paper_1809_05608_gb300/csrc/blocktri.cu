@@ -28,23 +28,6 @@ struct Pack {
   static constexpr int THREADS = SPC * NP;
 };
 
-// Map the j-th system of the launch to a global (ray, species) system index.
-__device__ inline long system_of(long j, const int *ray_list) {
-  return ray_list ? (long)ray_list[j / NS] * NS + (j % NS) : j;
-}
-
-__device__ inline long system_of_spr(long j, const int *ray_list, int spr) {
-  return ray_list ? (long)ray_list[j / spr] * spr + (j % spr) : j;
-}
-
-// Pivot-search key of a row: the value's exponent and leading mantissa bits, then the row; an integer
-// max over the keys finds the largest |x| to 15 mantissa bits, ties going to the lowest
-// row, and the winner's row is 31 - (key & 31).  Rows already used as pivots carry -1.
-__device__ inline int pivot_key(double x, int r) {
-  const unsigned hi = (unsigned)((unsigned long long)__double_as_longlong(x) >> 32) & 0x7fffffffu;
-  return (int)((hi & ~31u) | (unsigned)(31 - r));
-}
-
 template <int NP>
 __device__ inline int max_key(const int *__restrict__ c) {
   static_assert(NP % 4 == 0, "padded block sizes are multiples of 4");
@@ -87,7 +70,7 @@ k_factor(int n, int n_r, int n_sys, const double *__restrict__ diag, const doubl
   if ((long)blockIdx.x * (SPC / 2) >= n_sys_e) return;   // the whole CTA
   const long jsys = (long)blockIdx.x * (SPC / 2) + (s >> 1);
   const bool valid = jsys < n_sys_e;
-  const long sys = valid ? system_of(jsys, ray_list) : 0;
+  const long sys = valid ? listed_system(jsys, ray_list, NS) : 0;
   const int m = n_r / 2;
   const int len = half == 0 ? m + 1 : n_r - 1 - m;   // zones of this half; all threads step m + 1 times
 
@@ -190,7 +173,7 @@ k_solve(int n, int n_r, int n_sys, int spr, const double *__restrict__ dinv, con
   if ((long)blockIdx.x * (SPC / 2) >= n_sys_e) return;   // the whole CTA
   const long jsys = (long)blockIdx.x * (SPC / 2) + sl;
   const bool valid = jsys < n_sys_e;
-  const long sys = valid ? system_of_spr(jsys, ray_list, spr) : 0;
+  const long sys = valid ? listed_system(jsys, ray_list, spr) : 0;
   const bool realr = valid && r < n;
   const size_t base = (size_t)sys * n_r * n;
   const int m = n_r / 2, B = n_r - 1 - m;
@@ -332,7 +315,7 @@ k_factor_rows(int n, int n_r, int n_sys, int spr, const TIn *__restrict__ diag, 
   }
   const long jsys = (long)blockIdx.x * (SPC / 2) + (s >> 1);
   const bool valid = jsys < n_sys_e;
-  const long sys = valid ? system_of_spr(jsys, ray_list, spr) : 0;
+  const long sys = valid ? listed_system(jsys, ray_list, spr) : 0;
   const int m = n_r / 2;
   const int len = half == 0 ? m + 1 : n_r - 1 - m;   // zones of this half; all threads step m + 1 times
   const T one = T(1), zero = T(0);
@@ -506,13 +489,12 @@ __device__ inline void gj_invert(float *a, float (*prow)[NP + 4], int r, bool ro
 // static shared memory (two row buffers and the inverse tile per warp) stays under 48 KB.
 template <int NP> __host__ __device__ constexpr int fw_wpc() { return NP > 24 ? 2 : 4; }
 
-// At most 128 registers (NP <= 24), so that four CTAs (eight systems) fit on an SM and the
-// 256-ray workload's 512 CTAs run in a single wave on 152 SMs.
-// The C ABI's factor of arbitrary systems: partial pivoting in every zone.
-template <int NP, typename TIn, typename TC>
+// The C ABI's factor of arbitrary systems: partial pivoting in every zone.  At most 128 registers (NP <= 24), so that four
+// CTAs (eight systems) fit on an SM and the 256-ray workload's 512 CTAs run in a single wave on 152 SMs.
+template <int NP>
 __global__ void __launch_bounds__(fw_wpc<NP>() * 32, MGFLD_FW32_MINB)
-k_factor_w32(int n, int n_r, int n_sys, const TIn *__restrict__ diag, const TC *__restrict__ lower,
-             const TC *__restrict__ upper, float *__restrict__ dinv, const int *__restrict__ ray_list,
+k_factor_w32(int n, int n_r, int n_sys, const double *__restrict__ diag, const double *__restrict__ lower,
+             const double *__restrict__ upper, float *__restrict__ dinv, const int *__restrict__ ray_list,
              const int *__restrict__ n_dev) {
   static_assert(NP % 4 == 0, "rows of NP floats in 16-byte pieces");
   // tile: the natural-order inverse of each warp's last zone (read by the other half at the
@@ -522,57 +504,36 @@ k_factor_w32(int n, int n_r, int n_sys, const TIn *__restrict__ diag, const TC *
   __shared__ __align__(16) float ushr[W][NP];
   __shared__ __align__(16) float prow[W][2][NP + 4];
   __shared__ __align__(16) float rowbuf[W][2][NP][NP];
-  __shared__ __align__(16) TC cplb[W][2][2][32];      // per lane: the next zone's couplings (rows path)
   const int wid = threadIdx.x >> 5, r = threadIdx.x & 31;
   const int half = wid & 1;                          // 0: zones 0..m top-down, 1: zones n_r-1..m+1 bottom-up
   const long jsys = (long)blockIdx.x * (W / 2) + (wid >> 1);
   if (jsys >= listed_sys(n_sys, n_dev, NS)) return;  // both warps of the system leave; no barrier below
-  const long sys = system_of(jsys, ray_list);
+  const long sys = listed_system(jsys, ray_list, NS);
   const bool real = r < n;
   const bool row = r < NP;
-  const bool vec = (n == NP) && sizeof(TIn) == 4;    // 16-byte row loads and stores
   const int m = n_r / 2;
   const int len = half == 0 ? m + 1 : n_r - 1 - m;
   auto zone = [&](int j) { return half == 0 ? j : n_r - 1 - j; };
-  // Next zone's rows, fetched one zone ahead into a double-buffered shared-memory block (each
-  // lane its own row: 16-byte asynchronous copies on the fast path, so no registers hold the
-  // prefetch), and its couplings into registers.  The coupling loads are unconditional (lanes
-  // without a row read row 0) with the conditions applied when the values are consumed, so that
-  // no instruction waits on a load in the zone it was issued.
+  // Next zone's rows, fetched one zone ahead into a double-buffered shared-memory block (each lane its own row, so
+  // that no registers hold the prefetch), and its couplings into registers.  The coupling loads are unconditional
+  // (lanes without a row read row 0) with the conditions applied when the values are consumed, so that no instruction
+  // waits on a load in the zone it was issued.
   const int rr = real ? r : 0;
-  TC nl_raw = TC(0), nu_raw = TC(0);
+  double nl_raw = 0.0, nu_raw = 0.0;
   auto load_row = [&](int j) {
-    const int z = zone(j);
-    const size_t zr = ((size_t)sys * n_r + z) * n + rr;
+    const size_t zr = ((size_t)sys * n_r + zone(j)) * n + rr;
     float *dst = &rowbuf[wid][j & 1][row ? r : 0][0];
-    if (vec) {
-      if (row) {
+    if (row) {
 #pragma unroll
-        for (int c = 0; c < NP; c += 4) cp_async16(dst + c, diag + zr * n + c);
-      }
-      // couplings to the previous zone of this half's sequence (row scaling of its Schur term)
-      // and to the next one (column scaling of this zone's Schur term), in the same copy group
-      cp_async_elem(&cplb[wid][j & 1][0][r], (half == 0 ? lower : upper) + zr);
-      cp_async_elem(&cplb[wid][j & 1][1][r], (half == 0 ? upper : lower) + zr);
-      cp_async_commit();
-    } else {
-      if (row) {
-#pragma unroll
-        for (int c = 0; c < NP; ++c) dst[c] = (real && c < n) ? (float)diag[zr * n + c] : ((c == r) ? 1.f : 0.f);
-      }
-      nl_raw = half == 0 ? lower[zr] : upper[zr];
-      nu_raw = half == 0 ? upper[zr] : lower[zr];
+      for (int c = 0; c < NP; ++c) dst[c] = (real && c < n) ? (float)diag[zr * n + c] : ((c == r) ? 1.f : 0.f);
     }
+    nl_raw = half == 0 ? lower[zr] : upper[zr];
+    nu_raw = half == 0 ? upper[zr] : lower[zr];
   };
   if (len > 0) load_row(0);
   for (int j = 0; j < len; ++j) {
     const int z = zone(j);
     const size_t zrow = ((size_t)sys * n_r + z) * n + r;
-    if (vec) {
-      cp_async_wait_all();
-      nl_raw = cplb[wid][j & 1][0][r];
-      nu_raw = cplb[wid][j & 1][1][r];
-    }
     const float lr = (real && j > 0) ? (float)nl_raw : 0.f;
     const float ur = real ? (float)nu_raw : 0.f;
     if (j + 1 < len) load_row(j + 1);
@@ -629,15 +590,9 @@ k_factor_w32(int n, int n_r, int n_sys, const TIn *__restrict__ diag, const TC *
     if (row) ushr[wid][r] = ur;   // column scaling of this zone's Schur term in the next zone
     if (real) {
       float *out = dinv + zrow * n;
-      if (vec) {
 #pragma unroll
-        for (int c = 0; c < NP; c += 4)
-          *reinterpret_cast<float4 *>(out + c) = *reinterpret_cast<const float4 *>(&tile[wid][r][c]);
-      } else {
-#pragma unroll
-        for (int c = 0; c < NP; ++c)
-          if (c < n) out[c] = tile[wid][r][c];
-      }
+      for (int c = 0; c < NP; ++c)
+        if (c < n) out[c] = tile[wid][r][c];
     }
     __syncwarp();
   }
@@ -708,7 +663,7 @@ k_factor_row2(int n_, int n_r, int n_sys, int spr, const float *__restrict__ dia
   if (j0 >= n_sys_e) return;                               // the whole CTA
   const long jsys = j0 + g;
   const bool valid = g < S && jsys < n_sys_e;
-  const long sys = valid ? system_of_spr(jsys, ray_list, spr) : 0;
+  const long sys = valid ? listed_system(jsys, ray_list, spr) : 0;
   const int gs = g < S ? g : 0;                            // shared-memory slot (idle lanes use 0)
   const int m = n_r / 2;
   const int len = half == 0 ? m + 1 : n_r - 1 - m;
@@ -944,7 +899,7 @@ k_factor_wide(int n_, int n_r, int n_sys, int spr, const float *__restrict__ dia
   const int cg = act ? lane / L : 0, mm = lane % L, c0 = cg * C;
   const long jsys = blockIdx.x;
   if (jsys >= listed_sys(n_sys, n_dev, spr)) return;       // the whole CTA
-  const size_t sys = (size_t)system_of_spr(jsys, ray_list, spr);
+  const size_t sys = (size_t)listed_system(jsys, ray_list, spr);
   const int m = n_r / 2;
   const int len = half == 0 ? m + 1 : n_r - 1 - m;
   auto zone = [&](int j) { return half == 0 ? j : n_r - 1 - j; };
@@ -1147,7 +1102,7 @@ k_solve_w32(int n, int n_r, int n_sys, const float *__restrict__ dinv, const dou
   const int half = wid & 1, slot = wid >> 1;
   const long jsys = (long)blockIdx.x * (kWarpsPerCta / 2) + slot;
   if (jsys >= listed_sys(n_sys, n_dev, NS)) return;
-  const long sys = system_of(jsys, ray_list);
+  const long sys = listed_system(jsys, ray_list, NS);
   const bool real = r < n;
   const size_t base = (size_t)sys * n_r * n;
   const int m = n_r / 2, B = n_r - 1 - m;
@@ -1255,7 +1210,7 @@ cudaError_t launch_factor(int n, int n_r, int n_sys, const double *diag, const d
     })
   MGFLD_DISPATCH_NP(n, constexpr int W = fw_wpc<NP>();
                     const unsigned grid = (unsigned)((n_sys + W / 2 - 1) / (W / 2));
-                    k_factor_w32<NP, double, double><<<grid, W * 32, 0, s>>>(n, n_r, n_sys, diag, lower, upper,
+                    k_factor_w32<NP><<<grid, W * 32, 0, s>>>(n, n_r, n_sys, diag, lower, upper,
                                                                              (float *)dinv, ray_list, n_dev);
                     return cudaGetLastError())
 }
@@ -1280,7 +1235,7 @@ template <int NP>
 static cudaError_t run_factor_gj(int n, int n_r, int n_sys, int spr, const float *diag, const float *lower,
                                    const float *upper, float *dinv, const int *ray_list, int *bad, cudaStream_t s,
                                    const int *n_dev) {
-  if (n != NP && !bad) return cudaErrorInvalidValue;         // the padded kernels store flags
+  if ((n != NP || NP > 32) && !bad) return cudaErrorInvalidValue;   // the padded and the widest kernels store flags
   // A warp per half-system up to about four half-systems on each of the 4 kSMs warp schedulers (two of small
   // blocks, of which k_factor_row2 takes five to sixteen a warp), and for the pair systems' wide blocks at any
   // number.  Both sides, wide / row2, 256 zones: 1216 systems of 12 groups 186 / 173 us, 608 128 / 148 us; of 16
@@ -1296,8 +1251,9 @@ static cudaError_t run_factor_gj(int n, int n_r, int n_sys, int spr, const float
       return cudaGetLastError();
     }
   }
-  const auto kern = n == NP ? (bad ? k_factor_wide<NP, true, true> : k_factor_wide<NP, true, false>)
-                            : k_factor_wide<NP, false, true>;
+  // (without flags: whole blocks of the single species)
+  const auto kern = n != NP ? k_factor_wide<NP, false, true>
+                            : (bad ? k_factor_wide<NP, true, true> : k_factor_wide<NP, true, (NP > 32)>);
   kern<<<n_sys, 64, 0, s>>>(n, n_r, n_sys, spr, diag, lower, upper, dinv, ray_list, bad, n_dev);
   return cudaGetLastError();
 }

@@ -11,8 +11,8 @@
 // holding columns c = w mod 4, which puts an equal share of every pivot step on all four quarters,
 // and the lanes of a warp are the rows: NP / RPL lanes per half, lane c with rows c and c + NP/2 (RPL = 2)
 // or row c (RPL = 1), as many halves per warp as fit.  RPL = 2 fills 30 of 32 lanes at NP = 20 (three
-// halves a CTA, 11 FP64 instructions per warp and pivot step); where the launch has at most one CTA
-// per SM the chain of the pivot search counts instead, and RPL = 1 halves the FMAs behind it.
+// halves a CTA, 11 FP64 instructions per warp and pivot step); in launches of up to four CTAs per SM the chain of
+// the pivot search counts instead, and RPL = 1 halves the FMAs behind it.
 // Both do the same operations on every entry in the same order, those of one thread per row, so the
 // factors are the same bit for bit.  Measured (one factorisation, 512 zones x 20 groups; against
 // thread-per-row CTAs of four systems with two CTA barriers a step): 64 rays, RPL = 1, 7.68 -> 4.49 ms
@@ -22,15 +22,6 @@
 #include "mgfld_internal.cuh"
 
 namespace mgfld {
-
-// 32-bit pivot-search key of row r: the upper word of |x| (sign cleared; non-negative IEEE
-// values order like their bit patterns) with its 5 lowest bits replaced by 31 - r.  One integer
-// max over the keys then finds the largest |x| to 15 mantissa bits, ties going to the lowest
-// row, and the winner's row is 31 - (key & 31).  Rows already used as pivots carry -1.
-__device__ inline int pivot_key(double x, int r) {
-  const unsigned hi = (unsigned)((unsigned long long)__double_as_longlong(x) >> 32) & 0x7fffffffu;
-  return (int)((hi & ~31u) | (unsigned)(31 - r));
-}
 
 template <int NP, int RPL>
 struct Quad {
@@ -187,10 +178,6 @@ __device__ inline void invert64(double (&a)[RPL][NP / 4], typename Quad<NP, RPL>
     for (int q = 0; q < RPL; ++q) a[q][j] = sm.tile[g][c0 + q * L][4 * j + w];
 }
 
-__device__ inline long system64(long j, const int *ray_list) {
-  return ray_list ? (long)ray_list[j / NS] * NS + (j % NS) : j;
-}
-
 // middle = 0: item j is half j & 1 of system j / 2; 1: item j is the middle zone of system j.  Rows and
 // columns beyond the real group count n (<= NP) are padded with the identity.
 template <int NP, int RPL>
@@ -210,7 +197,7 @@ k_factor64(int n, int n_r, int n_sys, const double *__restrict__ diag, const dou
   const bool valid = item < n_items;
   const int m = n_r / 2;
   const int half = middle ? 0 : (int)(item & 1);         // 0: zones 0..m-1 top-down, 1: zones n_r-1..m+1 bottom-up
-  const long sys = valid ? system64(middle ? item : item >> 1, ray_list) : 0;
+  const long sys = valid ? listed_system(middle ? item : item >> 1, ray_list, NS) : 0;
   const int len = middle ? 1 : (half == 0 ? m : n_r - 1 - m);   // zones of this item
   const int steps = middle ? 1 : m;                      // of the CTA
   auto zone = [&](int j) { return middle ? m : (half == 0 ? j : n_r - 1 - j); };
@@ -226,7 +213,7 @@ k_factor64(int n, int n_r, int n_sys, const double *__restrict__ diag, const dou
       const long it = (long)blockIdx.x * S + h;
       const int hf = middle ? 0 : (int)(it & 1);
       if (it >= n_items || j >= (middle ? 1 : (hf == 0 ? m : n_r - 1 - m))) continue;
-      const long sy = system64(middle ? it : it >> 1, ray_list);
+      const long sy = listed_system(middle ? it : it >> 1, ray_list, NS);
       const int z = middle ? m : (hf == 0 ? j : n_r - 1 - j);
       const double *src = diag + ((size_t)sy * n_r + z) * nn;
       if (al16)
@@ -299,7 +286,7 @@ k_factor64(int n, int n_r, int n_sys, const double *__restrict__ diag, const dou
       const long it = (long)blockIdx.x * S + h;
       const int hf = middle ? 0 : (int)(it & 1);
       if (it >= n_items || j >= (middle ? 1 : (hf == 0 ? m : n_r - 1 - m))) continue;
-      const long sy = system64(middle ? it : it >> 1, ray_list);
+      const long sy = listed_system(middle ? it : it >> 1, ray_list, NS);
       const int z = middle ? m : (hf == 0 ? j : n_r - 1 - j);
       double *out = dinv + ((size_t)sy * n_r + z) * nn;
       for (int e = threadIdx.x; e < nn; e += 128) out[e] = sm.tile[h][e / n][e % n];
@@ -324,11 +311,15 @@ cudaError_t launch_factor64(int n, int n_r, int n_sys, const double *diag, const
                             double *dinv, const int *ray_list, cudaStream_t s, const int *n_dev) {
   if (n_sys == 0) return cudaSuccess;
   // RPL = 1 up to four CTAs per SM (1.3 us a pivot step at one CTA, 0.9 of the FP64 units' time at four),
-  // RPL = 2 beyond (half the FP64 instructions per half).
+  // RPL = 2 beyond (half the FP64 instructions per half) from 20 rows on; below, launch_factor takes a thread per
+  // row there, and always up to 4 rows.
   MGFLD_DISPATCH_NP(n, {
-    if (2 * (long)n_sys <= 4L * kSMs * Quad<NP, 1>::S)
-      return (run_factor64<NP, 1>(n, n_r, n_sys, diag, lower, upper, dinv, ray_list, s, n_dev));
-    return (run_factor64<NP, 2>(n, n_r, n_sys, diag, lower, upper, dinv, ray_list, s, n_dev));
+    if constexpr (NP >= 20) {
+      if (2 * (long)n_sys > 4L * kSMs * Quad<NP, 1>::S)
+        return (run_factor64<NP, 2>(n, n_r, n_sys, diag, lower, upper, dinv, ray_list, s, n_dev));
+    }
+    if constexpr (NP == 4) return cudaErrorInvalidValue;
+    else return (run_factor64<NP, 1>(n, n_r, n_sys, diag, lower, upper, dinv, ray_list, s, n_dev));
   })
 }
 

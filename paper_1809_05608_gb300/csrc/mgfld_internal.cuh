@@ -307,6 +307,10 @@ __device__ inline double scaled(const Prob &p, const double *a, size_t g, int q,
 __device__ inline int listed(int n, const int *n_dev) { return n_dev ? *n_dev : n; }
 // The same for a launch over systems, spr systems per listed ray.
 __device__ inline int listed_sys(int n_sys, const int *n_dev, int spr) { return n_dev ? *n_dev * spr : n_sys; }
+// The j-th system of a launch as a global system index (spr systems per ray).
+__device__ inline long listed_system(long j, const int *ray_list, int spr) {
+  return ray_list ? (long)ray_list[j / spr] * spr + (j % spr) : j;
+}
 
 // Exact power-of-two rescaling between FP64 and FP32 by exponent arithmetic on the bit
 // patterns (integer pipe only; mantissa truncated to 24 bits; results below the FP32 normal
@@ -359,6 +363,14 @@ __device__ inline int scale_of_max(unsigned hi_word_max) {
 }
 __device__ inline unsigned abs_hi_word(double v) {
   return (unsigned)((unsigned long long)__double_as_longlong(v) >> 32) & 0x7fffffffu;
+}
+// 32-bit pivot-search key of row r: the upper word of |x| (sign cleared; non-negative IEEE
+// values order like their bit patterns) with its 5 lowest bits replaced by 31 - r.  One integer
+// max over the keys then finds the largest |x| to 15 mantissa bits, ties going to the lowest
+// row, and the winner's row is 31 - (key & 31).  Rows already used as pivots carry -1.
+__device__ inline int pivot_key(double x, int r) {
+  const unsigned hi = (unsigned)((unsigned long long)__double_as_longlong(x) >> 32) & 0x7fffffffu;
+  return (int)((hi & ~31u) | (unsigned)(31 - r));
 }
 // 1/d without FP64-pipe conversions or compares (the pivots of the FP64 Gauss-Jordan steps; the
 // seed of the energy remap's quotients): the mantissa of d, rounded to 24 bits, becomes an FP32

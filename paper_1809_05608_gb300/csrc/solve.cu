@@ -7,11 +7,6 @@
 
 namespace mgfld {
 
-// Map the j-th system of the launch to a global system index (spr systems per ray).
-__device__ inline long listed_system(long j, const int *ray_list, int spr) {
-  return ray_list ? (long)ray_list[j / spr] * spr + (j % spr) : j;
-}
-
 // Per-system power-of-two scaling of the FP32 solve: k such that max |rhs| 2^k lies in [1/2, 1) (from
 // the largest exponent, so the maximum is taken over the upper words of the bit patterns: integer pipe
 // only), then the scaled right-hand side rounded to FP32 once, so that the substitution reads FP32
