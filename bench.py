@@ -438,7 +438,7 @@ def solve_roofline(res, inp):
     # iterations of the active rays: res['iters'] counts (ray, iteration) pairs over the timed steps
     nbytes = per_unit * n_s * n_r * res['iters']
     achieved = nbytes / (prof['ms'] * 1e-3) / 1e9
-    tr = traffic_record('k_solve_tma')
+    tr = traffic_record('k_solve_ring')
     traffic = None
     if tr is not None and solves:
         traffic = tr['bytes'] / tr['units'] * (res['iters'] * n_s / solves)

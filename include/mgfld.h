@@ -113,7 +113,11 @@ typedef struct {
 } mgfld_state;
 
 typedef struct {
-  int precision;       /* mgfld_precision: FP64 Newton, or FP32 factor + FP64 residual refinement */
+  int precision;       /* mgfld_precision: FP64 Newton, or FP32 factor + FP64 residual refinement.  MIXED
+                          without the pair process forms the sources of T, the heating and the
+                          ledgers as the last residual's plus the scattering of the last correction
+                          in FP32: 2^-23 of that correction, far below rounding for a converged ray,
+                          not for one that ends with MGFLD_ENOCONV or at a loose tol */
   double tol;          /* convergence: |d psi| <= tol * max(|psi|, tolmin_psi) for all (i,k,q) (Eq. a62ab) */
   double tolmin_psi;   /* typically 1 (Eq. a62ab) */
   double tol_ye;       /* |d Ye| <= tol_ye * max(Ye, tolmin_ye) */

@@ -1298,9 +1298,9 @@ cudaError_t launch_factor_f32(int n, int n_r, int n_sys, const float *diag, cons
   })
 }
 
-// FP64 substitution, up to how many systems the ring-fed one (a warp per half-system, n of its 32 lanes at work: bound
-// by latency while the FP64 units wait) is the faster one; beyond, the thread per row of k_solve keeps every lane at
-// work.  Ring / k_solve over 256 zones: 20 groups 256 systems 261 / 843 us, 1216 852 / 949, 1280 911 / 1052, 2048 1413 /
+// FP64 substitution, up to how many systems the ring-fed one (a warp per half-system, n of its 32 lanes at work: the
+// shorter chain, but more FP64 instructions for the same rows) is the faster one; beyond, the thread per row of k_solve
+// keeps every lane at work.  Ring / k_solve over 256 zones: 20 groups 256 systems 261 / 843 us, 1216 852 / 949, 1280 911 / 1052, 2048 1413 /
 // 1221 us; 12 groups 1280 637 / 639; 8 groups 1280 446 / 468, 2048 649 / 491; blocks of 16 and of up to 4 rows
 // (bank conflicts; few lanes) 1280 998 / 757 and 282 / 177 us.
 static inline int ring64_systems(int n) { return (n <= 4 || (n > 12 && n <= 16) ? 5 : 8) * kSMs; }
@@ -1322,13 +1322,13 @@ cudaError_t launch_solve(int n, int n_r, int n_sys, const void *dinv, const doub
   }
 }
 
-// The pair systems' FP64 substitution (nb = 2 n_e rows, two systems per ray; as above the ring-fed one is bound by
-// latency, and its rings leave room for few CTAs an SM: three of 32 rows, two of 40, one of 48): the ring up to the
-// launches that its CTAs hold at once, the thread per row beyond.  Ring / thread per row over 64 zones, us: 4 rows 608
-// systems 52 / 55, 720 61 / 55; 8 rows 608 53 / 61, 800 75 / 65; 12 rows 608 88 / 99, 800 125 / 111; 16 rows 912 133 / 165,
-// 1216 252 / 187; 18 rows 456 184 / 193, 608 231 / 204; 24 rows 456 192 / 229, 608 239 / 234; 26 rows 128 193 / 170,
-// 304 197 / 226, 456 236 / 240; 32 rows 152 211 / 203, 304 239 / 242, 380 296 / 280; 40 rows 304 270 / 363, 340 509 / 408;
-// 48 rows 152 321 / 410, 180 635 / 459, 4096 8453 / 4231.
+// The pair systems' FP64 substitution (nb = 2 n_e rows, two systems per ray; as above, and the rings of wide blocks
+// leave room for few CTAs an SM: three of 32 rows, two of 40, one of 48): the ring up to the launches that its CTAs
+// hold at once, the thread per row beyond.  Ring / thread per row over 64 zones, us: 4 rows 608 systems 52 / 55, 720
+// 61 / 55; 8 rows 608 53 / 61, 800 75 / 65; 12 rows 608 88 / 99, 800 125 / 111; 16 rows 912 133 / 165, 1216 252 / 187;
+// 18 rows 456 184 / 193, 608 231 / 204; 24 rows 456 192 / 229, 608 239 / 234; 26 rows 128 193 / 170, 304 197 / 226, 456
+// 236 / 240; 32 rows 152 211 / 203, 304 239 / 242, 380 296 / 280; 40 rows 304 270 / 363, 340 509 / 408; 48 rows 152
+// 321 / 410, 180 635 / 459, 4096 8453 / 4231.
 static inline bool ring64_pair(int nb, int n_sys) {
   if (nb <= 16) return n_sys <= (nb == 16 ? 6 : 4) * kSMs;
   if (nb <= 24) return n_sys <= 3 * kSMs;

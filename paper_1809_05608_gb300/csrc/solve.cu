@@ -474,9 +474,11 @@ cudaError_t launch_solve_ring(int n, int n_r, int n_sys, int spr, const void *di
                                                       sys_exp, err, s, n_dev)))
 }
 
-// FP64 factors (dinv on a 16-byte boundary; rhs and x may be one array; err or null).  Bound by the FP64
-// units with 20 of 32 lanes at work: per substitution at 64 / 256 rays of 512 x 20 1770 -> 495 us /
-// 1834 -> 1634 us, one ray of 64 x 12 115 -> 45 us (a thread per row and CTA barriers before).
+// FP64 factors (dinv on a 16-byte boundary; rhs and x may be one array; err or null).  Bound by the latency of a zone
+// step in small launches and by the FP64 units, with 20 of 32 lanes at work, in large ones: the 22 instructions of a row
+// and step take the units 0.29 of the 0.50 ms at 64 rays of 512 x 20 and 1.17 of the 1.63 ms at 256.  Per substitution at
+// 64 / 256 rays 1770 -> 495 us / 1834 -> 1634 us, one ray of 64 x 12 115 -> 45 us (a thread per row and CTA barriers
+// before, which is the faster one beyond about 1200 systems: launch_solve, launch_solve_pair64).
 cudaError_t launch_solve_ring64(int n, int n_r, int n_sys, int spr, const double *dinv, const double *lower,
                                 const double *upper, const double *rhs, double *x, const int *ray_list, int *err,
                                 cudaStream_t s, const int *n_dev) {
