@@ -617,7 +617,8 @@ k_factor_w32(int n, int n_r, int n_sys, const double *__restrict__ diag, const d
 // with partial pivoting unless its pivot blocks are those of an M-matrix: determinant and diagonal entries positive, no
 // entry above kGrowth times the raw one (elimination only takes from an M-matrix's diagonal).  An iterate with
 // occupations outside [0, 1] makes blocks that are none, and an unnoticed small pivot there factors without a correct
-// digit.  (The check: 3.76 -> 3.78 ms a step at 173 rays of 301 x 13, 25.4 -> 25.5 ms with pairs at 256 of 512 x 20.)
+// digit.  (The check, in integers: a step at 173 rays of 301 x 13 3.75 -> 3.75 ms, 3.78 with FP32 comparisons; with pairs
+// at 256 rays of 512 x 20 25.37 -> 25.48 ms.)
 // Bound by the issue slots of the row updates; measured at 1024 rays of 512 x 20: 2.05 ms.  (Publishing the next
 // pivots before the other row is updated, as k_factor_wide does, spills here: 2.50 ms.)
 template <int NP>
@@ -629,6 +630,9 @@ struct Row2 {
 };
 
 constexpr float kGrowth = 4.f;
+// 0 < d <= top by the bit patterns (top's, 0 if it is not positive; NaN and negative d are above it)
+__device__ inline unsigned growth_limit(float raw) { return raw > 0.f ? __float_as_uint(kGrowth * raw) : 0u; }
+__device__ inline bool in_range(float d, unsigned top) { return __float_as_uint(d) - 1u < top; }
 
 // CTAs per SM the two-rows-per-lane factor is compiled for (its register budget).
 template <int NP>
@@ -722,7 +726,7 @@ k_factor_row2(int n_, int n_r, int n_sys, int spr, const float *__restrict__ dia
     // -l_r (row r of the previous inverse, this lane's registers) * u_prev (column scaling)
     // (lanes without a system run on whatever their slot holds: they store nothing, and a slot
     // without a system is read by its own lanes only)
-    const float top0 = kGrowth * rows[wid][gs][r0][r0], top1 = kGrowth * rows[wid][gs][r1][r1];   // (FLAG)
+    const unsigned top0 = growth_limit(rows[wid][gs][r0][r0]), top1 = growth_limit(rows[wid][gs][r1][r1]);   // (FLAG)
     const float l0 = cpl[wid][gs][0][r0], l1 = cpl[wid][gs][0][r1];   // used from the second zone on
     const float u0 = cpl[wid][gs][1][r0], u1 = cpl[wid][gs][1][r1];
 #pragma unroll
@@ -778,9 +782,8 @@ k_factor_row2(int n_, int n_r, int n_sys, int spr, const float *__restrict__ dia
       const float det = fmaf(q0.x, q1.y, -(q0.y * q1.x));
       const float idet = rcp_nr(det);
       if (FLAG) {
-        ok = ok && idet > 0.f && idet < INFINITY;
-        const float d = mm == pl ? q0.x : q1.y;               // (NaN fails)
-        if (mm == pl || mm == pl + 1) ok = ok && d > 0.f && d <= (sl == 0 ? top0 : top1);
+        ok = ok && idet > 0.f && (p + 2 < NP || idet < INFINITY);   // (an infinite one makes the next NaN)
+        if (mm == pl || mm == pl + 1) ok = ok && in_range(mm == pl ? q0.x : q1.y, sl == 0 ? top0 : top1);
       }
       const float i00 = q1.y * idet, i01 = -q0.y * idet, i10 = -q1.x * idet, i11 = q0.x * idet;
       // multipliers of the two rows: owners take the rows of P^{-1} times the pivot rows
@@ -954,10 +957,11 @@ k_factor_wide(int n_, int n_r, int n_sys, int spr, const float *__restrict__ dia
     cp_async_wait_all();
     __syncwarp();
     // the zone's rows minus the Schur term of the previous zone
-    float u[R], top[R];                                    // (top: FLAG)
+    float u[R];
+    unsigned top[R];                                       // (FLAG)
 #pragma unroll
     for (int i = 0; i < R; ++i) {
-      top[i] = kGrowth * rows[half][mm + i * L][mm + i * L];
+      top[i] = growth_limit(rows[half][mm + i * L][mm + i * L]);
       const float l = cpl[half][0][mm + i * L];
       u[i] = cpl[half][1][mm + i * L];
 #pragma unroll
@@ -1020,9 +1024,8 @@ k_factor_wide(int n_, int n_r, int n_sys, int spr, const float *__restrict__ dia
       const float det = fmaf(q0.x, q1.y, -(q0.y * q1.x));
       const float idet = rcp_nr(det);
       if (FLAG) {
-        ok = ok && idet > 0.f && idet < INFINITY;
-        const float d = mm == pl ? q0.x : q1.y;               // (NaN fails)
-        if (mm == pl || mm == pl + 1) ok = ok && d > 0.f && d <= top[p / L];
+        ok = ok && idet > 0.f && (p + 2 < NP || idet < INFINITY);   // (an infinite one makes the next NaN)
+        if (mm == pl || mm == pl + 1) ok = ok && in_range(mm == pl ? q0.x : q1.y, top[p / L]);
       }
       const float i00 = q1.y * idet, i01 = -q0.y * idet, i10 = -q1.x * idet, i11 = q0.x * idet;
       // one row: minus its two multipliers times the pivot rows; what its columns p and p + 1 become is minus the
